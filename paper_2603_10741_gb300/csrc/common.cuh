@@ -195,8 +195,8 @@ struct lat_ctx {
   DBuf<double> KRP, Coarse, CoarseInv;
   DBuf<float> CoarseInv32;             // FP32 copy of the coarse inverse (mixed modes)
   int64_t coarse32_ld = 0;             // its row stride (a multiple of 4)
-  DBuf<double> tP, gP, xP;            // per-cell primal buffer [n_P][n_cells], primal vectors
-  DBuf<float> tP32, Phi32;            // FP32 per-cell primal buffer and Phi copy (mixed modes)
+  DBuf<double> gP, xP;                // primal vectors
+  DBuf<float> Phi32;                  // FP32 copy of Phi (mixed modes)
   DBuf<float> x32, y32;               // mixed-precision local vectors
   DBuf<double> kv_tmp[6];             // saddle-point sized temporaries
   DBuf<double> pcg_ws;                // interface PCG vectors (5 x n_lambda)

@@ -795,44 +795,74 @@ __global__ void __launch_bounds__(256)
   }
 }
 
-// corner values of every cell from the primal vector: tP[j][s] = xP[pidx[s][j]] (0 for a
-// Dirichlet primal DOF), in the precision of the product that follows
-template <typename T>
-__global__ void k_gather_tp(int n_cells, int n_P, const int* __restrict__ pidx, const double* __restrict__ xP,
-                            T* __restrict__ tP) {
-  const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (t >= (int64_t)n_cells * n_P) return;
-  const int s = (int)(t / n_P), j = (int)(t - (int64_t)s * n_P);
-  const int p = pidx[t];
-  tP[(size_t)j * n_cells + s] = p >= 0 ? (T)xP[p] : T(0);
-}
+// Y_R^s += Phi^{slot(s)} x_P^s on the rows of the view, x_P^s the cell's corner values (0 for a
+// Dirichlet primal DOF); rows n_K.. of the grid clear the corner rows (their values went to g_P).
+// A CTA owns 32 consecutive cells and kPhiRows rows: it gathers the cells' corner values (kPhiCols
+// at a time: 8 or 24 without enrichment, hundreds with a deep one) into shared memory ([j][cell],
+// conflict free), then every warp takes its four rows together with a lane per cell, so that a row's read-modify-write is one coalesced 256-byte segment, four of them
+// in flight, and the Phi row is a broadcast VEC-wide load (cells of a layer share their key).
+// Bound by the 17 bytes per entry of Y and its mask.  The form before (a thread per cell walking
+// 32 rows one after the other, corner values gathered by a launch of its own) was a chain of
+// dependent loads: 72 us per launch on the 10^3 strut lattice and 44 us on 16 ring cells, where it
+// was 30 % of a load step.  T = FP32 in the mixed modes (an FP32 copy of Phi, part of their FP32
+// preconditioner).
+constexpr int kPhiRows = 32, kPhiCols = 96;
 
-// Y_R^s += Phi^{slot(s)} tP[:, s] on rows [RB y, RB (y + 1)) of the view (a thread per cell: the
-// cell's corner values are coalesced reads that stay in L1 across the RB rows, Phi rows are
-// broadcast within a warp of cells of one key); rows n_K.. of the grid clear the corner rows
-// (their values went to g_P).  T = FP32 in the mixed modes (an FP32 copy of Phi, part of their
-// FP32 preconditioner).
-template <typename T>
-__global__ void __launch_bounds__(128)
-    k_phi_rows(int n_cells, int n_K, int n_P, int RB, int64_t kstride, const T* __restrict__ Phi,
-               const int* __restrict__ slot, const int* __restrict__ rdofs, const T* __restrict__ tP,
-               const uint8_t* __restrict__ fixed, const int* __restrict__ pdofs, double* __restrict__ Y) {
-  const int s = blockIdx.x * 128 + threadIdx.x;
-  if (s >= n_cells) return;
-  const T* tp = tP + s;
-  const int i0 = blockIdx.y * RB, i1 = min(i0 + RB, n_K + n_P);
+template <typename T, int VEC>
+__global__ void __launch_bounds__(256)
+    k_phi_rows(int n_cells, int n_K, int n_P, int64_t kstride, const T* __restrict__ Phi,
+               const int* __restrict__ slot, const int* __restrict__ rdofs, const int* __restrict__ pidx,
+               const double* __restrict__ xP, const uint8_t* __restrict__ fixed, const int* __restrict__ pdofs,
+               double* __restrict__ Y) {
+  struct alignas(sizeof(T) * VEC) Vec { T v[VEC]; };
+  constexpr int RW = kPhiRows / 8;                      // rows of a warp
+  __shared__ T tps[kPhiCols * 32];
+  const int s0 = blockIdx.x * 32, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int nc = min(32, n_cells - s0);
+  const int s = s0 + min(lane, nc - 1);
+  const bool live = lane < nc;
   const T* phs = Phi + (size_t)slot[s] * kstride;
-  for (int i = i0; i < i1; ++i) {
-    if (i >= n_K) {
-      Y[(size_t)pdofs[i - n_K] * n_cells + s] = 0.0;
-      continue;
-    }
-    const T* ph = phs + (size_t)i * n_P;
-    T v = 0;
-    for (int j = 0; j < n_P; ++j) v = fma(ph[j], tp[(size_t)j * n_cells], v);
-    const size_t e = (size_t)rdofs[i] * n_cells + s;
-    Y[e] = fixed[e] ? 0.0 : Y[e] + (double)v;
+  const int i0 = blockIdx.y * kPhiRows + warp * RW;
+  double* dst[RW];
+  double y[RW];
+  bool on[RW];
+#pragma unroll
+  for (int u = 0; u < RW; ++u) {                        // the rows' reads, ahead of the corner values
+    const int i = i0 + u;
+    const bool row = i < n_K, clear = !row && i < n_K + n_P;
+    const size_t e = (size_t)(row ? rdofs[i] : clear ? pdofs[i - n_K] : 0) * n_cells + s;
+    on[u] = row && !fixed[e];
+    y[u] = on[u] ? Y[e] : 0.0;
+    dst[u] = live && (row || clear) ? Y + e : nullptr;
   }
+  T v[RW];
+#pragma unroll
+  for (int u = 0; u < RW; ++u) v[u] = T(0);
+  for (int j0 = 0; j0 < n_P; j0 += kPhiCols) {
+    const int nj = min(kPhiCols, n_P - j0);             // a multiple of VEC
+    if (j0 > 0) __syncthreads();
+    for (int t = threadIdx.x; t < nc * nj; t += 256) {
+      const int c = t / nj, j = t - c * nj;
+      const int p = pidx[(size_t)(s0 + c) * n_P + j0 + j];
+      tps[j * 32 + c] = p >= 0 ? (T)xP[p] : T(0);
+    }
+    __syncthreads();
+    for (int j = 0; j < nj; j += VEC) {
+      T t[VEC];
+#pragma unroll
+      for (int q = 0; q < VEC; ++q) t[q] = tps[(j + q) * 32 + lane];
+#pragma unroll
+      for (int u = 0; u < RW; ++u) {
+        if (i0 + u >= n_K) continue;                    // warp-uniform
+        const Vec ph = *reinterpret_cast<const Vec*>(phs + (size_t)(i0 + u) * n_P + j0 + j);
+#pragma unroll
+        for (int q = 0; q < VEC; ++q) v[u] = fma(ph.v[q], t[q], v[u]);
+      }
+    }
+  }
+#pragma unroll
+  for (int u = 0; u < RW; ++u)
+    if (dst[u]) *dst[u] = on[u] ? y[u] + (double)v[u] : 0.0;
 }
 
 
@@ -1342,25 +1372,20 @@ void kinv(lat_ctx* h, const double* v, double* w, KinvMode mode = KINV_FULL, con
     run_coarse_solve(h, h->gP.p, pr_of(h, w));
   }
   if (h->n_primal) {
-    // w_R += Phi x_P on the view's rows (corner values gathered per cell first); the extra nP
-    // rows clear the corner rows
-    constexpr int RB = 32;
-    const dim3 grid(div_up(ns, 128), div_up(nKr + nP, RB));
-    const int64_t gt = (int64_t)ns * nP;
-    if (lo && h->Phi32.p) {
-      h->tP32.ensure((size_t)gt);
-      LAT_LAUNCH(h, k_gather_tp<float><<<div_up(gt, 256), 256, 0, h->stream>>>(ns, nP, h->pidx.p, pr_of(h, w),
-                                                                               h->tP32.p));
-      LAT_LAUNCH(h, k_phi_rows<float><<<grid, 128, 0, h->stream>>>(
-          ns, nKr, nP, RB, (int64_t)nR * nP, h->Phi32.p + (size_t)lo_r * nP, h->key_slot.p, rr, h->tP32.p,
-          h->loc_fixed.p, h->pdofs.p, wl));
+    // w_R += Phi x_P on the view's rows; the extra nP rows clear the corner rows
+    const dim3 grid(div_up(ns, 32), div_up(nKr + nP, kPhiRows));
+    const int64_t kst = (int64_t)nR * nP;
+    auto go = [&](auto kern, const auto* Phi) {
+      LAT_LAUNCH(h, kern<<<grid, 256, 0, h->stream>>>(ns, nKr, nP, kst, Phi + (size_t)lo_r * nP, h->key_slot.p, rr,
+                                                        h->pidx.p, pr_of(h, w), h->loc_fixed.p, h->pdofs.p, wl));
+    };
+    // 16-byte Phi loads where a row is a whole number of them (3D corners: 24 values), else scalar
+    if (lo) {
+      if (nP % 4 == 0) go(k_phi_rows<float, 4>, h->Phi32.p);
+      else go(k_phi_rows<float, 1>, h->Phi32.p);
     } else {
-      h->tP.ensure((size_t)gt);
-      LAT_LAUNCH(h, k_gather_tp<double><<<div_up(gt, 256), 256, 0, h->stream>>>(ns, nP, h->pidx.p, pr_of(h, w),
-                                                                                h->tP.p));
-      LAT_LAUNCH(h, k_phi_rows<double><<<grid, 128, 0, h->stream>>>(
-          ns, nKr, nP, RB, (int64_t)nR * nP, h->Phi.p + (size_t)lo_r * nP, h->key_slot.p, rr, h->tP.p,
-          h->loc_fixed.p, h->pdofs.p, wl));
+      if (nP % 2 == 0) go(k_phi_rows<double, 2>, h->Phi.p);
+      else go(k_phi_rows<double, 1>, h->Phi.p);
     }
     LAT_CHECK_LAUNCH();
   } else {
