@@ -285,76 +285,88 @@ __global__ void __launch_bounds__(128)
   }
 }
 
-// cell vectors of every tile, BF16 pairs in the tiled layout: XT[tile][kx][core_off(c, k)] with
+// BF16 pairs of eight consecutive K entries of one cell: the high parts and the BF16 roundings of
+// the remainders, as the two 16-byte core-matrix rows they are stored as
+__device__ __forceinline__ void split8(const float (&v)[8], uint4& hi, uint4& lo) {
+  uint32_t h[4], l[4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const __nv_bfloat162 a = __floats2bfloat162_rn(v[2 * q], v[2 * q + 1]);
+    const float2 f = __bfloat1622float2(a);
+    const __nv_bfloat162 b = __floats2bfloat162_rn(v[2 * q] - f.x, v[2 * q + 1] - f.y);
+    h[q] = *reinterpret_cast<const uint32_t*>(&a);
+    l[q] = *reinterpret_cast<const uint32_t*>(&b);
+  }
+  hi = make_uint4(h[0], h[1], h[2], h[3]);
+  lo = make_uint4(l[0], l[1], l[2], l[3]);
+}
+
+// Cell vectors of every tile, BF16 pairs in the tiled layout: XT[tile][kx][core_off(c, k)] with
 // kx = kp (high part) or KP + kp (low part), cell c = position c0 + c of the tile's key segment
-// (zero past the segment's end), column kp * 64 + k of the view (zero beyond n_K).  One CTA per
-// (tile, kp); gathered 8-byte reads, 16-byte writes.
+// (zero past the segment's end), column kp * 64 + k of the view (zero beyond n_K).  A thread owns
+// one cell and eight consecutive columns, i.e. one 16-byte row of a core matrix: its eight reads
+// are in flight together (a warp's are 32 consecutive cells of a row), eight neighbouring threads
+// store one whole 128-byte core matrix, and nothing goes through shared memory.  Bound by the
+// reads' latency and L2: with a CTA per (tile, panel) and the panel staged in shared memory there
+// were 243 CTAs of dependent reads on the 10^3 strut lattice, 41 us per launch against 15 us.
 template <int TN>
-__global__ void k_pack_xt(int n_cells, int n_K, int KP, const double* __restrict__ X, const int* __restrict__ tile_seg,
-                          const int* __restrict__ tile_c0, const int* __restrict__ seg_ptr, const int* __restrict__ perm,
-                          const int* __restrict__ rc, __nv_bfloat16* __restrict__ XT) {
+__global__ void __launch_bounds__(TN)
+    k_pack_xt(int n_cells, int n_K, int KP, const double* __restrict__ X, const int* __restrict__ tile_seg,
+              const int* __restrict__ tile_c0, const int* __restrict__ seg_ptr, const int* __restrict__ perm,
+              const int* __restrict__ rc, __nv_bfloat16* __restrict__ XT) {
   constexpr int BE = TN * TK;
-  __shared__ __align__(16) __nv_bfloat16 hi[BE], lo[BE];
-  const int tile = blockIdx.x, kp = blockIdx.y;
-  const int c0 = tile_c0[tile];
-  const int c_end = seg_ptr[tile_seg[tile] + 1];
-  for (int t = threadIdx.x; t < TN * TK; t += blockDim.x) {
-    const int k = t / TN, c = t % TN;                          // consecutive threads: consecutive cells
-    const int pos = c0 + c, gk = kp * TK + k;
-    float v = 0.f;
-    if (pos < c_end && gk < n_K) v = (float)X[(size_t)rc[gk] * n_cells + perm[pos]];
-    const __nv_bfloat16 h = __float2bfloat16(v);
-    hi[core_off(c, k)] = h;
-    lo[core_off(c, k)] = __float2bfloat16(v - __bfloat162float(h));
-  }
-  __syncthreads();
-  uint4* dh = reinterpret_cast<uint4*>(XT + ((size_t)tile * 2 * KP + kp) * BE);
-  uint4* dl = reinterpret_cast<uint4*>(XT + ((size_t)tile * 2 * KP + KP + kp) * BE);
-  for (int t = threadIdx.x; t < BE / 8; t += blockDim.x) {
-    dh[t] = reinterpret_cast<const uint4*>(hi)[t];
-    dl[t] = reinterpret_cast<const uint4*>(lo)[t];
-  }
+  const int tile = blockIdx.x, kp = blockIdx.y >> 3, c = threadIdx.x;
+  const int g0 = blockIdx.y * 8;                               // first column of the eight
+  const int pos = tile_c0[tile] + c;
+  const bool in = pos < seg_ptr[tile_seg[tile] + 1];
+  const int s = in ? perm[pos] : 0;
+  float v[8];
+#pragma unroll
+  for (int q = 0; q < 8; ++q) v[q] = in && g0 + q < n_K ? (float)X[(size_t)rc[g0 + q] * n_cells + s] : 0.f;
+  uint4 hi, lo;
+  split8(v, hi, lo);
+  __nv_bfloat16* dst = XT + ((size_t)tile * 2 * KP + kp) * BE + core_off(c, (blockIdx.y & 7) * 8);
+  *reinterpret_cast<uint4*>(dst) = hi;
+  *reinterpret_cast<uint4*>(dst + (size_t)KP * BE) = lo;
 }
 
 // the same tiles for an operand supported on the dual DOFs and given as B^T lambda (scaled by
 // 1/multiplicity when lsc is given): each copy's value is formed from its multipliers through
-// the per-(dual DOF, cell) table instead of being scattered into a zeroed local vector first
+// the per-(dual DOF, cell) table instead of being scattered into a zeroed local vector first.
+// Formed in FP32 (the value is rounded to FP32 and split into a BF16 pair anyway): only the two
+// multiplier reads convert from FP64, the FP64 pipe being the narrow one here.
 template <int TN>
-__global__ void k_pack_lam(int n_cells, int n_D, int KP, const double* __restrict__ lam, const int2* __restrict__ lk,
-                           const float* __restrict__ lsc, const int* __restrict__ tile_seg,
-                           const int* __restrict__ tile_c0, const int* __restrict__ seg_ptr,
-                           const int* __restrict__ perm, __nv_bfloat16* __restrict__ XT) {
+__global__ void __launch_bounds__(TN)
+    k_pack_lam(int n_cells, int n_D, int KP, const double* __restrict__ lam, const int2* __restrict__ lk,
+               const float* __restrict__ lsc, const int* __restrict__ tile_seg, const int* __restrict__ tile_c0,
+               const int* __restrict__ seg_ptr, const int* __restrict__ perm, __nv_bfloat16* __restrict__ XT) {
   constexpr int BE = TN * TK;
-  __shared__ __align__(16) __nv_bfloat16 hi[BE], lo[BE];
-  const int tile = blockIdx.x, kp = blockIdx.y;
-  const int c0 = tile_c0[tile];
-  const int c_end = seg_ptr[tile_seg[tile] + 1];
-  for (int t = threadIdx.x; t < TN * TK; t += blockDim.x) {
-    const int k = t / TN, c = t % TN;                          // consecutive threads: consecutive cells
-    const int pos = c0 + c, gk = kp * TK + k;
-    float v = 0.f;
-    if (pos < c_end && gk < n_D) {
-      const size_t q = (size_t)gk * n_cells + perm[pos];
-      // formed in FP32 (the value is rounded to FP32 and split into a BF16 pair anyway): only
-      // the two multiplier reads convert from FP64, the FP64 pipe being the narrow one here
-      const int2 l = lk[q];
-      float a = 0.f;
-      if (l.x) a = l.x > 0 ? __double2float_rn(lam[l.x - 1]) : -__double2float_rn(lam[-l.x - 1]);
-      if (l.y) a += l.y > 0 ? __double2float_rn(lam[l.y - 1]) : -__double2float_rn(lam[-l.y - 1]);
-      if (lsc) a *= lsc[q];
-      v = a;
-    }
-    const __nv_bfloat16 h = __float2bfloat16(v);
-    hi[core_off(c, k)] = h;
-    lo[core_off(c, k)] = __float2bfloat16(v - __bfloat162float(h));
+  const int tile = blockIdx.x, kp = blockIdx.y >> 3, c = threadIdx.x;
+  const int g0 = blockIdx.y * 8;
+  const int pos = tile_c0[tile] + c;
+  const bool in = pos < seg_ptr[tile_seg[tile] + 1];
+  const int s = in ? perm[pos] : 0;
+  int2 l[8];
+  float sc[8], v[8];
+#pragma unroll
+  for (int q = 0; q < 8; ++q) {
+    const bool ok = in && g0 + q < n_D;
+    const size_t e = (size_t)(g0 + q) * n_cells + s;
+    l[q] = ok ? lk[e] : make_int2(0, 0);
+    sc[q] = ok && lsc ? lsc[e] : 1.f;
   }
-  __syncthreads();
-  uint4* dh = reinterpret_cast<uint4*>(XT + ((size_t)tile * 2 * KP + kp) * BE);
-  uint4* dl = reinterpret_cast<uint4*>(XT + ((size_t)tile * 2 * KP + KP + kp) * BE);
-  for (int t = threadIdx.x; t < BE / 8; t += blockDim.x) {
-    dh[t] = reinterpret_cast<const uint4*>(hi)[t];
-    dl[t] = reinterpret_cast<const uint4*>(lo)[t];
+#pragma unroll
+  for (int q = 0; q < 8; ++q) {
+    float a = 0.f;
+    if (l[q].x) a = l[q].x > 0 ? __double2float_rn(lam[l[q].x - 1]) : -__double2float_rn(lam[-l[q].x - 1]);
+    if (l[q].y) a += l[q].y > 0 ? __double2float_rn(lam[l[q].y - 1]) : -__double2float_rn(lam[-l[q].y - 1]);
+    v[q] = a * sc[q];
   }
+  uint4 hi, lo;
+  split8(v, hi, lo);
+  __nv_bfloat16* dst = XT + ((size_t)tile * 2 * KP + kp) * BE + core_off(c, (blockIdx.y & 7) * 8);
+  *reinterpret_cast<uint4*>(dst) = hi;
+  *reinterpret_cast<uint4*>(dst + (size_t)KP * BE) = lo;
 }
 
 // a view of G (rows_v rows of n_K columns from (G, row stride ldsrc, key stride kstride)) as BF16
@@ -431,11 +443,11 @@ void launch_tc(lat_ctx* h, const double* X, double* Y, KinvMode mode, const int*
   const int KPmax = std::max(1, div_up(h->n_R, TK));
   h->Xb16.ensure((size_t)n_tiles * 2 * KPmax * C::B_ELEMS);
   if (lam)   // the dual view's operand is B^T lambda (mode KINV_DUAL: columns = the dual DOFs)
-    LAT_LAUNCH(h, k_pack_lam<TN><<<dim3(n_tiles, KP), 256, 0, h->stream>>>(h->n_cells, nKc, KP, lam, h->dual_lk.p,
+    LAT_LAUNCH(h, k_pack_lam<TN><<<dim3(n_tiles, KP * 8), TN, 0, h->stream>>>(h->n_cells, nKc, KP, lam, h->dual_lk.p,
                                                                             nullptr, tseg, tc0, h->seg_ptr.p,
                                                                             h->perm.p, h->Xb16.p));
   else
-    LAT_LAUNCH(h, k_pack_xt<TN><<<dim3(n_tiles, KP), 256, 0, h->stream>>>(h->n_cells, nKc, KP, X, tseg, tc0,
+    LAT_LAUNCH(h, k_pack_xt<TN><<<dim3(n_tiles, KP * 8), TN, 0, h->stream>>>(h->n_cells, nKc, KP, X, tseg, tc0,
                                                                            h->seg_ptr.p, h->perm.p, rc, h->Xb16.p));
   LAT_CUDA(cudaFuncSetAttribute(k_local_tc<TN, MW>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 (int)C::SMEM_BYTES));
@@ -460,11 +472,11 @@ void launch_sdd_tc(lat_ctx* h, const double* X, double* Y, const double* lam) {
   const int KPmax = std::max(1, div_up(h->n_R, TK));
   h->Xb16.ensure((size_t)h->max_tiles_tc * 2 * KPmax * C::B_ELEMS);
   if (lam)   // the operand is B_D^T lambda: B^T lambda scaled by 1/multiplicity
-    LAT_LAUNCH(h, k_pack_lam<TN><<<dim3(h->max_tiles_tc, KP), 256, 0, h->stream>>>(
+    LAT_LAUNCH(h, k_pack_lam<TN><<<dim3(h->max_tiles_tc, KP * 8), TN, 0, h->stream>>>(
                       h->n_cells, nD, KP, lam, h->dual_lk.p, h->dual_lsc.p, h->tile_seg_tc.p, h->tile_c0_tc.p,
                       h->seg_ptr.p, h->perm.p, h->Xb16.p));
   else
-    LAT_LAUNCH(h, k_pack_xt<TN><<<dim3(h->max_tiles_tc, KP), 256, 0, h->stream>>>(h->n_cells, nD, KP, X, h->tile_seg_tc.p,
+    LAT_LAUNCH(h, k_pack_xt<TN><<<dim3(h->max_tiles_tc, KP * 8), TN, 0, h->stream>>>(h->n_cells, nD, KP, X, h->tile_seg_tc.p,
                                                                                 h->tile_c0_tc.p, h->seg_ptr.p, h->perm.p,
                                                                                 rd, h->Xb16.p));
   LAT_CUDA(cudaFuncSetAttribute(k_local_tc<TN, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
