@@ -190,8 +190,7 @@ struct lat_ctx {
   DBuf<int> class_rep_d;
   DBuf<__nv_bfloat16> G16[4], Xb16;    // BF16 local matrices (one view per KinvMode, then the dual
                                        // Schur complements S_DD), packed cell vectors
-  int g16_ld[4] = {0, 0, 0, 0};        // their row strides
-  int64_t g16_lo[4] = {0, 0, 0, 0};    // offset of the low BF16 part after the high part
+  int g16_ld[4] = {0, 0, 0, 0};        // their K panels
   DBuf<double> KRP, Coarse, CoarseInv;
   DBuf<float> CoarseInv32;             // FP32 copy of the coarse inverse (mixed modes)
   int64_t coarse32_ld = 0;             // its row stride (a multiple of 4)
@@ -427,11 +426,9 @@ int coarse_coop_grid(lat_ctx* h);
 constexpr int64_t kDenseCoarseLimit = 8192;   // largest padded coarse size N m kept as a dense inverse
 constexpr int kWideSweepRows = 512;           // block-LU steps of larger blocks run over the whole GPU
 constexpr int kTcCells = 128;                 // cells per tensor-core tile (the MMA's N)
-constexpr int kTcRowTiles = 1;                // 128-row tiles per tensor-core CTA (sharing each B panel)
 void run_coarse_block_solve(lat_ctx* h, const double* g, double* x);
 void run_g_to_bf16(lat_ctx* h, size_t n);
 // which part of the local inverse a product uses (see kinv in feti.cu)
 enum KinvMode { KINV_FULL = 0, KINV_DUAL = 1, KINV_DUAL_IN = 2 };
-void run_local_tc(lat_ctx* h, const double* X, double* Y, KinvMode mode);
-void run_sdd_tc(lat_ctx* h, const double* X, double* Y, const double* lam = nullptr);
-void run_local_tc_lam(lat_ctx* h, const double* lam, double* Y);
+void run_local_tc(lat_ctx* h, const double* X, double* Y, KinvMode mode, const double* lam = nullptr);
+void run_sdd_tc(lat_ctx* h, const double* lam, double* Y);

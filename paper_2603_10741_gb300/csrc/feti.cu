@@ -1380,8 +1380,7 @@ void kinv(lat_ctx* h, const double* v, double* w, KinvMode mode = KINV_FULL, con
     }
   } else if (h->prec == LAT_MIXED_BF16) {
     // tcgen05, BF16 operands, FP32 accumulation
-    if (lam) run_local_tc_lam(h, lam, wl);
-    else run_local_tc(h, v, wl, mode);
+    run_local_tc(h, v, wl, mode, lam);
   } else {
     KernelTimer kt(h, tg_segmm[mode]);
     dim3 grid(h->max_tiles, div_up(nKr + nP, 64));
@@ -1458,7 +1457,7 @@ void dual_precond(lat_ctx* h, const double* r, double* z, double* t1, double* t2
     const size_t shm = (size_t)nD * sizeof(double);
     const bool seg = (int64_t)h->n_keys * 8 <= h->n_cells;
     if (fused) {
-      run_sdd_tc(h, nullptr, t2, r);   // tcgen05, BF16 operand pairs, FP32 accumulation; operand B_D^T r
+      run_sdd_tc(h, r, t2);   // tcgen05, BF16 operand pairs, FP32 accumulation; operand B_D^T r
     } else if (seg) {
       KernelTimer kt(h, "dual_schur");
       const int* rd = h->rdofs.p + h->n_I;

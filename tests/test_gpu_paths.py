@@ -52,3 +52,30 @@ def test_local_inverse_by_enrichment_and_cell_count(L, cell, dims, level):
     err = (back[:nd] - v[:nd]).abs().max().item() / v[:nd].abs().max().item()
     assert err < 1e-9, err
     lat.close()
+
+
+@pytest.mark.parametrize("cell,dims", [
+    (latgen.strut_cell(12, 0.15), (3, 3, 4)),    # 3 tiles of 9-18 cells x 21 row tiles: K split over 4 CTAs
+    (latgen.strut_cell(12, 0.15), (6, 6, 12)),   # 105 tiles, segments of 36 and 360 cells: split over 2
+    (latgen.strut_cell(12, 0.15), (9, 9, 9)),    # 168 tiles: not split; a segment of 567 cells
+    (latgen.ring_cell(4), (8, 9)),               # 24 remaining DOFs: fewer K panels than a cluster of 4
+])
+def test_tensor_core_product_by_tile_count(L, cell, dims):
+    """K^-rom in BF16 mode against the FP64 mode: ~16-bit operand pairs, FP32 sums (tolerance as in
+    test_gpu_solver.py's tensor-core tests)."""
+    case = _case(cell, dims)
+    outs = []
+    for prec in (0, 2):
+        lat = L.Lattice.from_case(case, prec)
+        u = lat.lattice_predictor(0.1 * case.top_displacement(1))
+        lat.select_principal_cells(u, 1e-3, 1)
+        lat.lattice_set_timing(True)
+        lat.lattice_prepare_solver(u, lat.lattice_default_opts(max_enrich=0, precond_tangent=1))
+        rng = np.random.default_rng(7)
+        s = lat.sizes
+        v = lat.feti_from_global(torch.tensor(rng.uniform(-1, 1, s.n_dof), device="cuda"))
+        outs.append(lat.feti_apply(1, v)[: s.n_loc * s.n_cells + s.n_primal].cpu().numpy())
+        assert prec == 0 or lat.lattice_kernel_time("local_tc")[1] > 0
+        lat.close()
+    err = np.linalg.norm(outs[1] - outs[0]) / np.linalg.norm(outs[0])
+    assert err < 1e-4, err
