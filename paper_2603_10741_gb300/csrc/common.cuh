@@ -91,7 +91,10 @@ struct lat_ctx {
   // reference cell
   DBuf<double> gradX[2], W[2];  // [n_el][nq][nen][dim], [n_el][nq]
   DBuf<int> elems;              // [n_el][nen]
-  DBuf<int> elem_blk;           // [n_el][nen][nen] block index of (a, b)
+  DBuf<int> elem_blk;           // [n_el][nen][nen] block index of (a, b); bit 30: the first element, in
+                                // colour order, to touch the block
+  DBuf<double> Jinv;            // [n_el][2^dim][dim*dim] 2^-dim J0^{-1} at the full rule's points
+  DBuf<int> node_el_ptr, node_el;  // node -> element * nen + local node, ascending
   std::vector<int> color_start; // host offsets into color_elems
   DBuf<int> color_elems;
   DBuf<int> blk_ptr, blk_col;   // node-block CSR of the local pattern
@@ -316,6 +319,29 @@ __device__ __forceinline__ double det_inv<3>(const double (&F)[3][3], double (&F
   Fi[1][2] = (F[0][2] * F[1][0] - F[0][0] * F[1][2]) * r;
   Fi[2][2] = (F[0][0] * F[1][1] - F[0][1] * F[1][0]) * r;
   return J;
+}
+
+// det F and the cofactors C = det F F^{-T}
+template <int D>
+__device__ __forceinline__ double det_cof(const double (&F)[D][D], double (&C)[D][D]) {
+  if constexpr (D == 2) {
+    C[0][0] = F[1][1];
+    C[0][1] = -F[1][0];
+    C[1][0] = -F[0][1];
+    C[1][1] = F[0][0];
+    return F[0][0] * F[1][1] - F[0][1] * F[1][0];
+  } else {
+    C[0][0] = F[1][1] * F[2][2] - F[1][2] * F[2][1];
+    C[0][1] = F[1][2] * F[2][0] - F[1][0] * F[2][2];
+    C[0][2] = F[1][0] * F[2][1] - F[1][1] * F[2][0];
+    C[1][0] = F[0][2] * F[2][1] - F[0][1] * F[2][2];
+    C[1][1] = F[0][0] * F[2][2] - F[0][2] * F[2][0];
+    C[1][2] = F[0][1] * F[2][0] - F[0][0] * F[2][1];
+    C[2][0] = F[0][1] * F[1][2] - F[0][2] * F[1][1];
+    C[2][1] = F[0][2] * F[1][0] - F[0][0] * F[1][2];
+    C[2][2] = F[0][0] * F[1][1] - F[0][1] * F[1][0];
+    return F[0][0] * C[0][0] + F[0][1] * C[0][1] + F[0][2] * C[0][2];
+  }
 }
 
 // deterministic block reductions (fixed shape, fixed order)

@@ -49,6 +49,7 @@ void build_geometry(lat_ctx* h, const double* X, const int* E) {
     const int nq = (int)pts.size();
     h->nq[red] = nq;
     std::vector<double> gX((size_t)h->n_el * nq * nen * d), Wv((size_t)h->n_el * nq);
+    std::vector<double> Ji(red ? 0 : (size_t)h->n_el * nq * d * d);
     for (int e = 0; e < h->n_el; ++e) {
       for (int q = 0; q < nq; ++q) {
         // reference shape-function gradients d phi_a / d xi
@@ -100,8 +101,12 @@ void build_geometry(lat_ctx* h, const double* X, const int* E) {
             gX[(((size_t)e * nq + q) * nen + a) * d + k] = v;
           }
         Wv[(size_t)e * nq + q] = wq[q] * det;
+        if (!red)
+          for (int l = 0; l < d; ++l)
+            for (int k = 0; k < d; ++k) Ji[(((size_t)e * nq + q) * d + l) * d + k] = inv[l][k] / (double)(1 << d);
       }
     }
+    if (!red) h->Jinv.upload(Ji, h->stream);
     h->gradX[red].upload(gX, h->stream);
     h->W[red].upload(Wv, h->stream);
   }
@@ -136,7 +141,6 @@ void build_pattern_and_colors(lat_ctx* h, const int* E) {
         eb[((size_t)e * nen + a) * nen + b] = (int)(std::lower_bound(beg, end, nb) - h->h_blk_col.begin());
       }
     }
-  h->elem_blk.upload(eb, h->stream);
   h->blk_ptr.upload(h->h_blk_ptr, h->stream);
   h->blk_col.upload(h->h_blk_col, h->stream);
   if (h->dim == 3) build_node_groups(h);
@@ -164,6 +168,28 @@ void build_pattern_and_colors(lat_ctx* h, const int* E) {
     h->color_start[c + 1] = (int)ce.size();
   }
   h->color_elems.upload(ce, h->stream);
+  // the first element of every block in colour order
+  std::vector<char> seen(h->n_blk, 0);
+  for (int e : ce) {
+    int* b = eb.data() + (size_t)e * nen * nen;
+    for (int q = 0; q < nen * nen; ++q)
+      if (!seen[b[q]]) {
+        seen[b[q]] = 1;
+        b[q] |= 1 << 30;
+      }
+  }
+  h->elem_blk.upload(eb, h->stream);
+  // elements of every node
+  std::vector<int> nptr(nn + 1, 0), nsrc;
+  std::vector<std::vector<int>> at(nn);
+  for (int e = 0; e < h->n_el; ++e)
+    for (int a = 0; a < nen; ++a) at[E[e * nen + a]].push_back(e * nen + a);
+  for (int a = 0; a < nn; ++a) {
+    nptr[a + 1] = nptr[a] + (int)at[a].size();
+    nsrc.insert(nsrc.end(), at[a].begin(), at[a].end());
+  }
+  h->node_el_ptr.upload(nptr, h->stream);
+  h->node_el.upload(nsrc, h->stream);
 }
 
 void build_maps(lat_ctx* h, const lat_mesh_desc* ds) {
@@ -616,7 +642,7 @@ extern "C" lat_status lattice_destroy(lat_handle h) {
   if (h->cap_stream) cudaStreamDestroy(h->cap_stream);
   // DBuf members free themselves through release(); walk them explicitly
   auto rel = [](auto& b) { b.release(); };
-  rel(h->gradX[0]); rel(h->gradX[1]); rel(h->W[0]); rel(h->W[1]); rel(h->elems); rel(h->elem_blk);
+  rel(h->gradX[0]); rel(h->gradX[1]); rel(h->W[0]); rel(h->W[1]); rel(h->elems); rel(h->elem_blk); rel(h->Jinv); rel(h->node_el_ptr); rel(h->node_el);
   rel(h->color_elems); rel(h->blk_ptr); rel(h->blk_col); rel(h->cell_nodes); rel(h->mu_cell);
   rel(h->copy_ptr); rel(h->copy_idx); rel(h->dof_fixed); rel(h->dir_unit); rel(h->aff_unit);
   rel(h->corner_of_node); rel(h->rdofs); rel(h->pdofs); rel(h->rpos); rel(h->pidx);

@@ -7,6 +7,7 @@ import pytest
 import torch
 
 import latgen
+from oracle import cell as OC
 from oracle import newton as ON
 from oracle.assembly import Problem
 
@@ -79,3 +80,39 @@ def test_tensor_core_product_by_tile_count(L, cell, dims):
         lat.close()
     err = np.linalg.norm(outs[1] - outs[0]) / np.linalg.norm(outs[0])
     assert err < 1e-4, err
+
+
+def _rel(a, b):
+    return np.abs(np.asarray(a) - np.asarray(b)).max() / np.abs(np.asarray(b)).max()
+
+
+@pytest.mark.parametrize("cell,dims", [
+    (latgen.solid_cell(1, 2), (3, 1)),           # one element per cell: 4 of a warp's lanes
+    (latgen.solid_cell(3, 3), (1, 2, 1)),        # 27 elements: a last warp with 24 lanes
+    (latgen.solid_cell(9, 3), (2, 1, 1)),        # 729 elements: forces staged in two parts
+    (latgen.ring_cell(4), (13, 3)),              # 39 cells: one CTA per cell; 38 and fewer: eight
+])
+def test_residual_and_tangent_by_element_and_cell_count(L, cell, dims):
+    """Forces and tangents, both rules, of all cells and of a list, against the oracle (FP64 sums in
+    another order: 1e-11 of the largest entry, as in test_gpu_kernels.py)."""
+    case = _case(cell, dims)
+    prob = Problem(case)
+    u = latgen.smooth_state(case.lattice, 0.01, 11).ravel()
+    lat = L.Lattice.from_case(case)
+    ud = torch.tensor(u, device="cuda")
+    ul = prob.local(u)
+    n = prob.lat.n_cells
+    out = lat.assemble_residual_tangent(ud, local_forces=True, tangent=True)
+    f_ref = OC.internal_force(prob.cell, ul, prob.mu_cells, prob.lam).reshape(n, -1).T
+    assert _rel(out["f"].cpu(), f_ref) < 1e-11
+    assert _rel(out["r"].cpu(), prob.residual(u)) < 1e-11
+    assert abs(out["min_detF"] - OC.min_jacobian(prob.cell, ul).min()) < 1e-12
+    K_ref = OC.tangent(prob.cell, ul, prob.mu_cells, prob.lam)
+    assert _rel(out["K"].cpu(), K_ref) < 1e-11
+    cells = np.arange(n - 1, -1, -1)[:38].astype(np.int32)
+    ct = torch.tensor(cells, device="cuda")
+    for quad in (0, 1):
+        K = lat.assemble_residual_tangent(ud, quad=quad, cells=ct, residual=False, tangent=True)["K"].cpu()
+        ref = OC.tangent(prob.cell, ul[cells], prob.mu_cells[cells], prob.lam, reduced=quad == 1)
+        assert _rel(K, ref) < 1e-11
+    lat.close()
