@@ -189,7 +189,7 @@ struct lat_ctx {
   DBuf<float> G32;
   DBuf<double> SDD;                   // [n_keys][n_D][n_D] dual Schur complements
   DBuf<float> SDD32;
-  DBuf<double> gj_P, gj_C, gj_R;      // Gauss-Jordan workspace (pivot inverse, column and row panels)
+  DBuf<double> gj_P, gj_C, gj_R;      // inversion workspace (pivot inverse, panel A_.p and A_.p A_pp^-1)
   DBuf<int> class_rep_d;
   DBuf<__nv_bfloat16> G16[4], Xb16;    // BF16 local matrices (one view per KinvMode, then the dual
                                        // Schur complements S_DD), packed cell vectors

@@ -345,116 +345,186 @@ __global__ void k_densify(int n_keys, const int* __restrict__ key_list, int n_cl
   }
 }
 
-// --- blocked in-place Gauss-Jordan inversion of SPD matrices (batched) -----------------------
-// step with pivot block p = [k0, k0+kw):  Pi = A_pp^{-1};  A_ij -= A_ip Pi A_pj (i,j not in p);
-// A_pj = Pi A_pj;  A_ip = -A_ip Pi;  A_pp = Pi.
+// --- blocked in-place inversion of symmetric matrices (batched): the sweep operator --------------
+// Step with pivot block p = [k0, k0+kw), C = A_.p (all rows), Pi = A_pp^{-1}, R = C Pi:
+//   A_ij -= C_i R_j^T  (i, j not in p);   A_ip = R_i;   A_pp = -Pi.
+// With this sign convention every intermediate matrix is symmetric (Gauss-Jordan's are symmetric up
+// to the signs of swept columns), so only the lower triangle is worked on, half the multiply-adds
+// of the FP64 pipe that bounds the update (three 2616 matrices: 93 ms per inversion with both
+// triangles, 47 ms now), and the final matrix is -A^{-1}, mirrored and negated at the end.  Pivots are
+// those of Gauss-Jordan.
 constexpr int GJB = 32;
+constexpr int kSwRows = 16;   // rows of R per CTA
 
-__global__ void k_gj_pivot(int n, int64_t bs, int k0, int kw, double* __restrict__ A, double* __restrict__ Pinv,
-                           double* __restrict__ Cbuf, int* __restrict__ flag, int neg_bit) {
-  __shared__ double M[GJB][GJB + 1];
-  const int b = blockIdx.x;
-  double* a = A + (size_t)b * bs;
-  const int t = threadIdx.x;  // 1024 threads: (i, j)
-  const int i = t / GJB, j = t % GJB;
-  if (i < kw && j < kw) M[i][j] = a[(size_t)(k0 + i) * n + k0 + j];
-  // column panel copy (old values) for the trailing update
-  for (int r = t; r < n * kw; r += blockDim.x) {
-    const int row = r / kw, c = r % kw;
-    Cbuf[((size_t)b * n + row) * GJB + c] = a[(size_t)row * n + k0 + c];
+// 1 / x from the hardware's approximation (about 20 bits) and one cubically convergent correction
+// r (1 + e + e^2), e = 1 - x r: three dependent FP64 operations; the division outside its range
+__device__ __forceinline__ double pivot_rcp(double x) {
+  if (!(fabs(x) > 1e-290 && fabs(x) < 1e290)) return x != 0.0 ? 1.0 / x : 0.0;
+  double r;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+  const double e = fma(-x, r, 1.0);
+  return fma(r, fma(e, e, e), r);
+}
+
+// Sweeps of the symmetric kw x kw pivot block M in shared memory by 1 x 1 pivots (256 threads), M
+// <- -M^{-1}.  A chain of kw dependent steps, and a dependent FP64 operation takes about 100 clocks:
+// warp 0 runs the chain alone (it keeps the diagonal, so the next reciprocal is formed while the
+// other warps apply the step), the 528 entries of the triangle stay in the others' registers, and
+// a step's column and products go through shared memory.  30 us for 32 columns when every step
+// waited for the division and the division for the step, 24 us now (cold caches).
+__device__ void sweep_pivot(int kw, double (&M)[GJB][GJB + 1], double (&col)[2][GJB], double (&rp)[GJB],
+                            int* __restrict__ flag, int neg_bit) {
+  const int t = threadIdx.x, n_e = kw * (kw + 1) / 2;
+  constexpr int NU = 3;                        // 224 threads x 3 >= 528
+  double m[NU], diag = 0.0, d = 0.0;
+  int ei[NU], ej[NU];
+#pragma unroll
+  for (int u = 0; u < NU; ++u) {
+    const int e = t - 32 + 224 * u;
+    ei[u] = ej[u] = -1;
+    m[u] = 0.0;
+    if (t < 32 || e >= n_e) continue;
+    int i = (int)((sqrtf(8.f * (float)e + 1.f) - 1.f) * 0.5f);   // row of entry e of the packed triangle
+    if ((i + 1) * (i + 2) / 2 <= e) ++i;
+    if (i * (i + 1) / 2 > e) --i;
+    ei[u] = i;
+    ej[u] = e - i * (i + 1) / 2;
+    m[u] = M[i][ej[u]];
   }
-  __syncthreads();
-  // one reciprocal per pivot (thread 0) and the scaled pivot row, then one multiply-add per entry:
-  // FP64 runs at two multiply-adds per clock per SM, so the 32 x 32 sweep is kept to the minimum
-  __shared__ double rowp[GJB];
-  __shared__ double dsh;
+  auto check = [&](double piv) {
+    if (t != 0 || !flag) return;
+    if (!(fabs(piv) > 0.0) || !isfinite(piv)) atomicOr(flag, 1);
+    else if (piv < 0.0) atomicOr(flag, neg_bit);
+  };
+  if (t < 32) {
+    col[0][t] = t < kw ? M[t][0] : 0.0;
+    diag = t < kw ? M[t][t] : 0.0;
+    const double piv = __shfl_sync(0xffffffffu, diag, 0);
+    check(piv);
+    d = pivot_rcp(piv);
+  }
   for (int p = 0; p < kw; ++p) {
-    if (t == 0) {
-      const double piv = M[p][p];
-      if (!(fabs(piv) > 0.0) || !isfinite(piv)) atomicOr(flag, 1);
-      else if (piv < 0.0) atomicOr(flag, neg_bit);
-      dsh = piv != 0.0 ? 1.0 / piv : 0.0;
+    const double (&c)[GJB] = col[p & 1];
+    double (&next)[GJB] = col[(p + 1) & 1];
+    double ct = 0.0, rt = 0.0;
+    if (t < 32) {
+      ct = c[t];
+      rt = t == p ? -d : ct * d;
+      rp[t] = rt;
     }
     __syncthreads();
-    const double d = dsh;
-    if (t < kw) rowp[t] = t == p ? d : M[p][t] * d;   // new pivot row
-    double mip = 0.0, mij = 0.0;
-    if (i < kw && j < kw) {
-      mip = M[i][p];
-      mij = M[i][j];
-    }
-    __syncthreads();
-    if (i < kw && j < kw) {
-      if (i == p) M[i][j] = rowp[j];
-      else if (j == p) M[i][j] = -mip * d;
-      else M[i][j] = fma(-mip, rowp[j], mij);
+    if (t < 32) {
+      diag = fma(-ct, rt, diag);
+      const double piv = __shfl_sync(0xffffffffu, diag, min(p + 1, 31));
+      if (p + 1 < kw) {
+        check(piv);
+        d = pivot_rcp(piv);
+      }
+    } else {
+#pragma unroll
+      for (int u = 0; u < NU; ++u) {
+        const int i = ei[u], j = ej[u];
+        if (i < 0) continue;
+        m[u] = i == p ? rp[j] : j == p ? rp[i] : fma(-c[i], rp[j], m[u]);
+        if (i == p + 1) next[j] = m[u];        // row and column p + 1, the diagonal entry from i == j
+        else if (j == p + 1) next[i] = m[u];
+      }
     }
     __syncthreads();
   }
-  if (i < kw && j < kw) Pinv[(size_t)b * GJB * GJB + i * GJB + j] = M[i][j];
-}
-
-// Rbuf[b][m][j] = sum_l Pinv[m][l] A[k0+l][j]  (new pivot rows); a CTA covers 8 columns and
-// every thread one (m, j) entry, so that even a single matrix spreads over many SMs
-__global__ void __launch_bounds__(256) k_gj_rows(int n, int64_t bs, int k0, int kw, const double* __restrict__ A,
-                                                 const double* __restrict__ Pinv, double* __restrict__ Rbuf) {
-  const int b = blockIdx.y;
-  const double* a = A + (size_t)b * bs;
-  const double* P = Pinv + (size_t)b * GJB * GJB;
-  __shared__ double Ps[GJB][GJB + 1];
-  __shared__ double Cs[GJB][8];
-  const int j0 = blockIdx.x * 8;
-  for (int t = threadIdx.x; t < GJB * GJB; t += blockDim.x) {
-    const int r = t / GJB, c = t % GJB;
-    Ps[r][c] = (r < kw && c < kw) ? P[t] : 0.0;
-  }
-  {
-    const int l = threadIdx.x / 8, c = threadIdx.x % 8;
-    const int gj = j0 + c;
-    Cs[l][c] = (l < kw && gj < n) ? a[(size_t)(k0 + l) * n + gj] : 0.0;
-  }
+#pragma unroll
+  for (int u = 0; u < NU; ++u)
+    if (ei[u] >= 0) M[ei[u]][ej[u]] = M[ej[u]][ei[u]] = m[u];
   __syncthreads();
-  const int m = threadIdx.x / 8, c = threadIdx.x % 8;
-  const int j = j0 + c;
-  if (m >= kw || j >= n) return;
-  double v;
-  if (j >= k0 && j < k0 + kw) {
-    v = Ps[m][j - k0];
-  } else {
-    v = 0.0;
-#pragma unroll 8
-    for (int l = 0; l < GJB; ++l) v = fma(Ps[m][l], Cs[l][c], v);
-  }
-  Rbuf[((size_t)b * GJB + m) * n + j] = v;
 }
 
-// trailing update over T x T tiles (T = 16, 32 or 64: small batches take small tiles so that
-// every SM gets work); every tile reads only Cbuf / Rbuf / Pinv, so tiles are independent
+__device__ __forceinline__ void load_pivot(int n, int k0, int kw, const double* __restrict__ a,
+                                           double (&M)[GJB][GJB + 1]) {
+  for (int t = threadIdx.x; t < GJB * GJB; t += 256) {
+    const int i = t / GJB, j = t % GJB;
+    M[i][j] = i < kw && j < kw ? a[(size_t)(k0 + max(i, j)) * n + k0 + min(i, j)] : 0.0;
+  }
+}
+
+// Pinv[b] = Pi (one CTA per matrix)
+__global__ void __launch_bounds__(256) k_sw_pivot(int n, int64_t bs, int k0, int kw, const double* __restrict__ A,
+                                                  double* __restrict__ Pinv, int* __restrict__ flag, int neg_bit) {
+  __shared__ double M[GJB][GJB + 1], col[2][GJB], rp[GJB];
+  const int b = blockIdx.x;
+  load_pivot(n, k0, kw, A + (size_t)b * bs, M);
+  __syncthreads();
+  sweep_pivot(kw, M, col, rp, flag, neg_bit);
+  for (int t = threadIdx.x; t < GJB * GJB; t += 256) Pinv[(size_t)b * GJB * GJB + t] = -M[t / GJB][t % GJB];
+}
+
+// C and R for kSwRows rows per CTA.  OWN: every CTA inverts the pivot block itself, which saves a
+// launch on the chain of steps; taken while the CTAs are no more than the SMs (redundant inversions
+// on one SM share its FP64 pipe).
+template <bool OWN>
+__global__ void __launch_bounds__(256) k_sw_rows(int n, int64_t bs, int k0, int kw, const double* __restrict__ A,
+                                                 double* __restrict__ Pinv, double* __restrict__ Cbuf,
+                                                 double* __restrict__ Rbuf, int* __restrict__ flag, int neg_bit) {
+  __shared__ double M[GJB][GJB + 1], col[2][GJB], rp[GJB];
+  __shared__ double Cs[kSwRows][GJB + 1];
+  const int b = blockIdx.y, i0 = blockIdx.x * kSwRows;
+  const double* a = A + (size_t)b * bs;
+  const double sgn = OWN ? -1.0 : 1.0;
+  // columns of the panel above the pivot block are read as rows of the lower triangle
+  const bool above = i0 + kSwRows <= k0;
+  for (int t = threadIdx.x; t < kSwRows * GJB; t += 256) {
+    const int r = above ? t % kSwRows : t / GJB, c = above ? t / kSwRows : t % GJB;
+    const int i = i0 + r, k = k0 + c;
+    Cs[r][c] = i < n && c < kw ? a[(size_t)max(i, k) * n + min(i, k)] : 0.0;
+  }
+  if (OWN) {
+    load_pivot(n, k0, kw, a, M);
+    __syncthreads();
+    sweep_pivot(kw, M, col, rp, blockIdx.x == 0 ? flag : nullptr, neg_bit);
+    if (blockIdx.x == 0)
+      for (int t = threadIdx.x; t < GJB * GJB; t += 256) Pinv[(size_t)b * GJB * GJB + t] = -M[t / GJB][t % GJB];
+  } else {
+    for (int t = threadIdx.x; t < GJB * GJB; t += 256) M[t / GJB][t % GJB] = Pinv[(size_t)b * GJB * GJB + t];
+    __syncthreads();
+  }
+  for (int t = threadIdx.x; t < kSwRows * GJB; t += 256) {
+    const int r = t / GJB, c = t % GJB;
+    if (i0 + r >= n) continue;
+    double v0 = 0.0, v1 = 0.0;
+#pragma unroll 8
+    for (int l = 0; l < GJB; l += 2) {
+      v0 = fma(Cs[r][l], M[l][c], v0);
+      v1 = fma(Cs[r][l + 1], M[l + 1][c], v1);
+    }
+    const size_t o = ((size_t)b * n + i0 + r) * GJB + c;
+    Cbuf[o] = Cs[r][c];
+    Rbuf[o] = sgn * (v0 + v1);
+  }
+}
+
+// trailing update over the lower T x T tiles (T = 16, 32 or 64: small batches take small tiles so
+// that every SM gets work); every tile reads only Cbuf / Rbuf / Pinv, so tiles are independent
 template <int T>
-__global__ void __launch_bounds__(256) k_gj_update(int n, int64_t bs, int k0, int kw, double* __restrict__ A,
+__global__ void __launch_bounds__(256) k_sw_update(int n, int64_t bs, int k0, int kw, double* __restrict__ A,
                                                    const double* __restrict__ Pinv, const double* __restrict__ Cbuf,
                                                    const double* __restrict__ Rbuf) {
   constexpr int U = T / 16;
-  const int b = blockIdx.z;
+  const int b = blockIdx.y;
+  int ti = (int)((sqrtf(8.f * (float)blockIdx.x + 1.f) - 1.f) * 0.5f);
+  while ((ti + 1) * (ti + 2) / 2 <= (int)blockIdx.x) ++ti;
+  while (ti * (ti + 1) / 2 > (int)blockIdx.x) --ti;
+  const int tj = (int)blockIdx.x - ti * (ti + 1) / 2;
   double* a = A + (size_t)b * bs;
   const double* C = Cbuf + (size_t)b * n * GJB;
-  const double* R = Rbuf + (size_t)b * GJB * n;
+  const double* R = Rbuf + (size_t)b * n * GJB;
   const double* P = Pinv + (size_t)b * GJB * GJB;
   __shared__ double Cs[T][GJB + 1];
-  __shared__ double Rs[GJB][T + 1];
-  const int i0 = blockIdx.y * T, j0 = blockIdx.x * T;
+  __shared__ double Rs[T][GJB + 1];
+  const int i0 = ti * T, j0 = tj * T;
   const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
-  for (int t = threadIdx.x; t < T * GJB; t += blockDim.x) {
+  for (int t = threadIdx.x; t < T * GJB; t += 256) {
     const int r = t / GJB, c = t % GJB;
-    const int gi = i0 + r;
-    Cs[r][c] = (gi < n && c < kw) ? C[(size_t)gi * GJB + c] : 0.0;
-  }
-  for (int t = threadIdx.x; t < GJB * T; t += blockDim.x) {
-    const int r = t / T, c = t % T;
-    const int gj = j0 + c;
-    double v = 0.0;
-    if (gj < n && r < kw) v = (gj >= k0 && gj < k0 + kw) ? P[r * GJB + (gj - k0)] : R[(size_t)r * n + gj];
-    Rs[r][c] = v;
+    Cs[r][c] = i0 + r < n ? C[(size_t)(i0 + r) * GJB + c] : 0.0;
+    Rs[r][c] = j0 + r < n ? R[(size_t)(j0 + r) * GJB + c] : 0.0;
   }
   __syncthreads();
   double acc[U][U];
@@ -467,7 +537,7 @@ __global__ void __launch_bounds__(256) k_gj_update(int n, int64_t bs, int k0, in
 #pragma unroll
     for (int u = 0; u < U; ++u) cv[u] = Cs[ty + 16 * u][l];
 #pragma unroll
-    for (int v = 0; v < U; ++v) rv[v] = Rs[l][tx + 16 * v];
+    for (int v = 0; v < U; ++v) rv[v] = Rs[tx + 16 * v][l];
 #pragma unroll
     for (int u = 0; u < U; ++u)
 #pragma unroll
@@ -484,10 +554,26 @@ __global__ void __launch_bounds__(256) k_gj_update(int n, int64_t bs, int k0, in
       if (gj >= n) continue;
       const bool jp = gj >= k0 && gj < k0 + kw;
       double* dst = a + (size_t)gi * n + gj;
-      if (ip) *dst = jp ? P[(gi - k0) * GJB + (gj - k0)] : R[(size_t)(gi - k0) * n + gj];
-      else if (jp) *dst = -acc[u][v];        // -A_ip Pi   (Rs holds Pi on pivot columns)
-      else *dst -= acc[u][v];                // A_ij - A_ip (Pi A_pj)
+      if (ip) *dst = jp ? -P[(gi - k0) * GJB + (gj - k0)] : Rs[tx + 16 * v][gi - k0];
+      else if (jp) *dst = R[(size_t)gi * GJB + (gj - k0)];
+      else *dst -= acc[u][v];
     }
+  }
+}
+
+// swept matrix -> inverse: A_ij = A_ji = -(lower triangle), 32 x 32 tiles
+__global__ void __launch_bounds__(256) k_sw_finish(int n, int64_t bs, double* __restrict__ A) {
+  __shared__ double S[32][33];
+  if (blockIdx.x > blockIdx.y) return;
+  double* a = A + (size_t)blockIdx.z * bs;
+  const int i0 = blockIdx.y * 32, j0 = blockIdx.x * 32, tx = threadIdx.x % 32, ty = threadIdx.x / 32;
+  for (int r = ty; r < 32; r += 8)
+    S[r][tx] = i0 + r < n && j0 + tx < n ? -a[(size_t)(i0 + r) * n + j0 + tx] : 0.0;
+  __syncthreads();
+  const bool diag = blockIdx.x == blockIdx.y;
+  for (int r = ty; r < 32; r += 8) {
+    if (i0 + r < n && j0 + tx < n) a[(size_t)(i0 + r) * n + j0 + tx] = diag && tx > r ? S[tx][r] : S[r][tx];
+    if (!diag && j0 + r < n && i0 + tx < n) a[(size_t)(j0 + r) * n + i0 + tx] = S[tx][r];
   }
 }
 
@@ -498,7 +584,7 @@ __global__ void k_gj_snapshot(int n, int64_t bs, int split, const double* __rest
   const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (t >= (int64_t)m * m) return;
   const int i = (int)(t / m), j = (int)(t % m);
-  snap[(size_t)b * m * m + t] = A[(size_t)b * bs + (size_t)(split + i) * n + split + j];
+  snap[(size_t)b * m * m + t] = A[(size_t)b * bs + (size_t)(split + max(i, j)) * n + split + min(i, j)];
 }
 
 // Phi = -G K_RP [k][n_R][n_P]; Phi^T is also stored as rows n_R.. of the augmented local
@@ -1041,10 +1127,10 @@ struct SolverTmp {
 // ---------------------------------------------------------------------------------------------
 }  // namespace
 
-// invert `batch` n x n matrices stored with a stride of bs elements (in place).  With split in
-// (0, n) the pivot blocks stop at `split` once: the trailing block [split, n)^2 then holds the
-// Schur complement A_22 - A_21 A_11^{-1} A_12, copied to snap ([batch][n-split]^2) before the
-// sweep continues.
+// invert `batch` symmetric n x n matrices stored with a stride of bs elements (in place; the lower
+// triangle is read).  With split in (0, n) the pivot blocks stop at `split` once: the trailing block
+// [split, n)^2 then holds the Schur complement A_22 - A_21 A_11^{-1} A_12, copied to snap
+// ([batch][n-split]^2) before the sweep continues.
 void gj_invert(lat_ctx* h, double* A, int n, int batch, int64_t bs, int neg_bit, int split,
                double* snap) {
   // workspace kept in the handle: no allocation and no host synchronisation per inversion
@@ -1053,31 +1139,37 @@ void gj_invert(lat_ctx* h, double* A, int n, int batch, int64_t bs, int neg_bit,
   DBuf<double>& Rbuf = h->gj_R;
   Pinv.ensure((size_t)batch * GJB * GJB);
   Cbuf.ensure((size_t)batch * n * GJB);
-  Rbuf.ensure((size_t)batch * GJB * n);
+  Rbuf.ensure((size_t)batch * n * GJB);
   if (snap && split == 0) {
     LAT_LAUNCH(h, k_gj_snapshot<<<dim3(div_up((int64_t)n * n, 256), batch), 256, 0, h->stream>>>(n, bs, 0, A, snap));
     LAT_CHECK_LAUNCH();
   }
+  const int T = fp64_tile(n, batch, h->n_sm);
+  const dim3 rows(div_up(n, kSwRows), batch);
+  const int64_t per = div_up(n, T);
+  const dim3 tiles((unsigned)(per * (per + 1) / 2), batch);
   for (int k0 = 0; k0 < n;) {
     int kw = std::min(GJB, n - k0);
     if (split > 0 && k0 < split) kw = std::min(kw, split - k0);
     {
       KernelTimer kt(h, "gj_pivot");
-      LAT_LAUNCH(h, k_gj_pivot<<<batch, 1024, 0, h->stream>>>(n, bs, k0, kw, A, Pinv.p, Cbuf.p, h->flag.p, neg_bit));
-      LAT_LAUNCH(h, k_gj_rows<<<dim3(div_up(n, 8), batch), 256, 0, h->stream>>>(n, bs, k0, kw, A, Pinv.p, Rbuf.p));
+      if ((int64_t)rows.x * batch <= h->n_sm) {
+        LAT_LAUNCH(h, k_sw_rows<true><<<rows, 256, 0, h->stream>>>(n, bs, k0, kw, A, Pinv.p, Cbuf.p, Rbuf.p, h->flag.p,
+                                                                   neg_bit));
+      } else {
+        LAT_LAUNCH(h, k_sw_pivot<<<batch, 256, 0, h->stream>>>(n, bs, k0, kw, A, Pinv.p, h->flag.p, neg_bit));
+        LAT_LAUNCH(h, k_sw_rows<false><<<rows, 256, 0, h->stream>>>(n, bs, k0, kw, A, Pinv.p, Cbuf.p, Rbuf.p,
+                                                                    h->flag.p, neg_bit));
+      }
     }
     {
       KernelTimer kt(h, "gj_update");
-      const int T = fp64_tile(n, batch, h->n_sm);
-      if (T == 64)
-        LAT_LAUNCH(h, k_gj_update<64><<<dim3(div_up(n, 64), div_up(n, 64), batch), 256, 0, h->stream>>>(
-                          n, bs, k0, kw, A, Pinv.p, Cbuf.p, Rbuf.p));
-      else if (T == 32)
-        LAT_LAUNCH(h, k_gj_update<32><<<dim3(div_up(n, 32), div_up(n, 32), batch), 256, 0, h->stream>>>(
-                          n, bs, k0, kw, A, Pinv.p, Cbuf.p, Rbuf.p));
-      else
-        LAT_LAUNCH(h, k_gj_update<16><<<dim3(div_up(n, 16), div_up(n, 16), batch), 256, 0, h->stream>>>(
-                          n, bs, k0, kw, A, Pinv.p, Cbuf.p, Rbuf.p));
+      auto go = [&](auto kern) {
+        LAT_LAUNCH(h, kern<<<tiles, 256, 0, h->stream>>>(n, bs, k0, kw, A, Pinv.p, Cbuf.p, Rbuf.p));
+      };
+      if (T == 64) go(k_sw_update<64>);
+      else if (T == 32) go(k_sw_update<32>);
+      else go(k_sw_update<16>);
     }
     LAT_CHECK_LAUNCH();
     k0 += kw;
@@ -1087,11 +1179,9 @@ void gj_invert(lat_ctx* h, double* A, int n, int batch, int64_t bs, int neg_bit,
       LAT_CHECK_LAUNCH();
     }
   }
+  LAT_LAUNCH(h, k_sw_finish<<<dim3(div_up(n, 32), div_up(n, 32), batch), 256, 0, h->stream>>>(n, bs, A));
+  LAT_CHECK_LAUNCH();
 }
-
-
-namespace {
-}  // namespace
 
 // principal tangents the local blocks are built from: the full K^r, or its material part
 // evaluated at u_glob for the same principal cells (precond_tangent, Section 3.1.4)

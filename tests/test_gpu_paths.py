@@ -116,3 +116,29 @@ def test_residual_and_tangent_by_element_and_cell_count(L, cell, dims):
         ref = OC.tangent(prob.cell, ul[cells], prob.mu_cells[cells], prob.lam, reduced=quad == 1)
         assert _rel(K, ref) < 1e-11
     lat.close()
+
+
+@pytest.mark.parametrize("cell,dims,lu", [
+    (latgen.ring_cell(2), (2, 9), 0),        # blocks of 8 and 12 rows: less than one pivot block
+    (latgen.solid_cell(6, 2), (9, 9), 0),    # 90 remaining DOFs: 32 + 32 + 26, split inside a pivot block
+    (latgen.solid_cell(4, 3), (3, 3, 3), 1), # 351 remaining DOFs, 81 of them interior; coarse blocks as block LU
+])
+def test_symmetric_inverse_by_size(L, cell, dims, lu):
+    """Local and coarse inverses by sweeps: K^-rom K~ = I on the force-all path, whose every local
+    block and coarse block goes through the batched inversion."""
+    case = _case(cell, dims)
+    prob = Problem(case)
+    lat = L.Lattice.from_case(case)
+    ud = torch.tensor(ON.predictor(prob, 1, None, None), device="cuda")
+    lat.select_principal_cells(ud, 0.0, 1, force_all=True)
+    lat.lattice_prepare_solver(ud, lat.lattice_default_opts(precond_tangent=0, max_enrich=0, coarse_block_lu=lu))
+    s = lat.sizes
+    nd = s.n_loc * s.n_cells + s.n_primal
+    v = lat.feti_from_global(torch.tensor(np.random.default_rng(5).uniform(-1, 1, s.n_dof), device="cuda"))
+    v[nd:] = 0
+    Kv = lat.feti_apply(0, v)
+    Kv[nd:] = 0
+    back = lat.feti_apply(1, Kv)
+    err = (back[:nd] - v[:nd]).abs().max().item() / v[:nd].abs().max().item()
+    assert err < 1e-9, err
+    lat.close()
