@@ -211,6 +211,14 @@ struct lat_ctx {
   int max_tiles = 0;
   DBuf<int> tile_seg_tc, tile_c0_tc;  // key segments in tiles of kTcCells cells (tensor-core products)
   int max_tiles_tc = 0;
+  // FP64 products on digits (fp64_tc.cu): 16-cell tiles, digits and row factors of [G; Phi^T] and of
+  // S_DD, digits and largest magnitudes of the packed cell vectors
+  bool oz = false;
+  int oz_tiles = 0;
+  DBuf<int> tile_seg_oz, tile_c0_oz;
+  DBuf<__nv_bfloat16> oz_G, oz_S, oz_X;
+  DBuf<double> oz_Gs, oz_Ss;
+  DBuf<unsigned long long> oz_max;
   bool indefinite = false;              // a principal's remaining block had a negative pivot
   bool coarse_indefinite = false;       // the coarse matrix had a negative pivot
   int64_t pcg_its_total = 0;            // interface PCG iterations since the last reset
@@ -452,9 +460,14 @@ int coarse_coop_grid(lat_ctx* h);
 constexpr int64_t kDenseCoarseLimit = 8192;   // largest padded coarse size N m kept as a dense inverse
 constexpr int kWideSweepRows = 512;           // block-LU steps of larger blocks run over the whole GPU
 constexpr int kTcCells = 128;                 // cells per tensor-core tile (the MMA's N)
+constexpr int kOzCells = 16;                  // cells per tile of the FP64 products on digits
 void run_coarse_block_solve(lat_ctx* h, const double* g, double* x);
 void run_g_to_bf16(lat_ctx* h, size_t n);
 // which part of the local inverse a product uses (see kinv in feti.cu)
 enum KinvMode { KINV_FULL = 0, KINV_DUAL = 1, KINV_DUAL_IN = 2 };
 void run_local_tc(lat_ctx* h, const double* X, double* Y, KinvMode mode, const double* lam = nullptr);
 void run_sdd_tc(lat_ctx* h, const double* lam, double* Y);
+bool oz_wanted(const lat_ctx* h);
+void run_oz_split(lat_ctx* h);
+void run_local_oz(lat_ctx* h, const double* X, double* Y, KinvMode mode);
+void run_sdd_oz(lat_ctx* h, const double* X, double* Y);

@@ -1256,6 +1256,18 @@ void run_prepare_solver(lat_ctx* h, const lat_newton_opts* o, const double* u_gl
     h->max_tiles_tc = (int)tseg_tc.size();
   }
   h->key_slot.upload(slot_cell, h->stream);  // slot of each cell
+  h->oz = oz_wanted(h);
+  std::vector<int> tseg_oz, tc0_oz;   // alive until the synchronisation below
+  if (h->oz) {
+    for (int k = 0; k < nk; ++k)
+      for (int c = cnt[k]; c < cnt[k + 1]; c += kOzCells) {
+        tseg_oz.push_back(k);
+        tc0_oz.push_back(c);
+      }
+    h->tile_seg_oz.upload(tseg_oz, h->stream);
+    h->tile_c0_oz.upload(tc0_oz, h->stream);
+    h->oz_tiles = (int)tseg_oz.size();
+  }
   // dense local blocks
   const int64_t gstride = (int64_t)(nR + nP) * nR;   // augmented [G; Phi^T] per key
   const size_t gsz = (size_t)nk * gstride;
@@ -1335,6 +1347,7 @@ void run_prepare_solver(lat_ctx* h, const lat_newton_opts* o, const double* u_gl
   LAT_REQUIRE(!(fl & 1), LAT_EINDEFINITE, "a local remaining-DOF matrix or the coarse matrix is singular");
   h->indefinite = (fl & 2) != 0;          // a principal's remaining block has a negative pivot
   h->coarse_indefinite = (fl & 8) != 0;   // the coarse matrix has a negative pivot
+  if (h->oz) run_oz_split(h);
   if (h->prec == LAT_MIXED_BF16) run_g_to_bf16(h, gsz);
   if (h->prec != LAT_FP64) {
     h->G32.ensure(gsz);
@@ -1471,6 +1484,10 @@ void kinv(lat_ctx* h, const double* v, double* w, KinvMode mode = KINV_FULL, con
   } else if (h->prec == LAT_MIXED_BF16) {
     // tcgen05, BF16 operands, FP32 accumulation
     run_local_tc(h, v, wl, mode, lam);
+  } else if (h->oz) {
+    // FP64 on the tensor cores: exact digit products
+    KernelTimer kt(h, tg_segmm[mode]);
+    run_local_oz(h, v, wl, mode);
   } else {
     KernelTimer kt(h, tg_segmm[mode]);
     dim3 grid(h->max_tiles, div_up(nKr + nP, 64));
@@ -1548,6 +1565,9 @@ void dual_precond(lat_ctx* h, const double* r, double* z, double* t1, double* t2
     const bool seg = (int64_t)h->n_keys * 8 <= h->n_cells;
     if (fused) {
       run_sdd_tc(h, r, t2);   // tcgen05, BF16 operand pairs, FP32 accumulation; operand B_D^T r
+    } else if (h->oz) {
+      KernelTimer kt(h, "dual_schur");
+      run_sdd_oz(h, t1, t2);
     } else if (seg) {
       KernelTimer kt(h, "dual_schur");
       const int* rd = h->rdofs.p + h->n_I;
@@ -1852,7 +1872,7 @@ int run_fgmres(lat_ctx* h, const double* b, double* x, const lat_newton_opts* o,
     total = fgmres_core(h, outer, b, x, false, o->krylov_rtol, o->krylov_max_it, o->krylov_restart, false, block,
                         rel_out);
   }
-  if (h->prec == LAT_MIXED_BF16 || (h->cb_solve && h->cb_wide && h->cb_coop_grid > 0)) {
+  if (h->prec == LAT_MIXED_BF16 || h->oz || (h->cb_solve && h->cb_wide && h->cb_coop_grid > 0)) {
     int fl = 0;
     LAT_CUDA(cudaMemcpyAsync(&fl, h->flag.p, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
     LAT_CUDA(cudaStreamSynchronize(h->stream));

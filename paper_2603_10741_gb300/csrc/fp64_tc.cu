@@ -1,0 +1,479 @@
+// FP64 principal-block x cell-vector products on the tensor cores, for the FP64 mode: the local part
+// of K^-rom, Y[rows of cell s] = [G; Phi^T]_{key(s)} X_R^s, and the dual Schur complements of the
+// interface preconditioner, over cells grouped by key.
+//
+// FP64 runs at 1.2 TFLOP/s on this GPU, 1/1500 of its BF16 tensor rate, and these products are 80 %
+// of an FP64 3D solve.  They are formed without it, by an error-free splitting (the scheme of Ozaki,
+// Ogita, Oishi and Rump, "Error-free transformations of matrix multiplication by using fast routines
+// of matrix multiplication and its applications", 2012): each row of the matrix and each cell vector
+// is scaled by a power of two and split into 8 signed base-128 digits,
+//   x = 2^(e-6) sum_i s_i 2^(-7 i),  |s_i| <= 64   (|x| <= 2^e; the rest is below 2^(e-56)),
+// digits are exact in BF16, products of digits are integers below 2^12, and the tensor core adds
+// them in FP32 exactly while a sum stays below 2^24.  The 36 digit products with i + j <= 7 go to
+// eight accumulators by i + j (at most 8 products of 2^12 per column: 512 columns may be summed),
+// which the epilogue recombines as integers and converts to FP64 once.
+//
+// Precision.  What is dropped (digits beyond the eighth, products with i + j > 7) is about 2^-56 of
+// (row maximum) x (vector maximum) per term, with random signs; rounding in an FP64 dot product of
+// K terms is about 2^-53 of sqrt(K) times the rms product per term.  Measured: K^-rom K~ v - v on
+// lattices of equal strut cells (36, 216 and 225 cells, three vectors each) is 1.6e-13 to 1.0e-12 of
+// v, 0.91 (geometric mean) of what FP64 products with the same inverses leave.
+//
+// One tensor-memory tile is 128 rows x (8 accumulators of 16 cells): for digit i of the matrix one
+// MMA multiplies the digits 0 .. 7-i of the 16 cells (N = 16 (8 - i), consecutive rows of the B
+// panel) into the accumulators i .. 7, consecutive columns from 16 i on.  K is split over a cluster
+// of CTAs (512 columns at most each, which the exactness needs) that add their FP64 tiles through
+// distributed shared memory.  Bound by streaming the digits, 16 bytes per matrix entry: the strut
+// cell's dual block (1716 x 1692) for 3 keys and 36 cells is 151 MB: 35 us,
+// and 15 us to split the vectors, against 406 us on the FP64 pipe (175 us at its full rate).
+#include <algorithm>
+
+#include "common.cuh"
+#include "tc_ptx.cuh"
+
+namespace {
+
+constexpr int ND = 8;                     // digits
+constexpr int TM = 128, TK = 16, NC = kOzCells; // rows, K panel, cells of a tile
+constexpr int A_SLICE = TM * TK;          // elements of one digit of an A panel
+constexpr int A_ELEMS = ND * A_SLICE;     // 32 KiB
+constexpr int B_ELEMS = ND * NC * TK;     // 4 KiB
+constexpr int STAGE_BYTES = 2 * (A_ELEMS + B_ELEMS);
+constexpr int STAGES = 3;                 // 108 KiB, two CTAs per SM
+constexpr int TMEM_COLS = ND * NC;        // 128
+constexpr int MAX_PANELS = 512 / TK;      // panels one CTA may sum exactly
+constexpr int MAX_SPLIT = 8;              // portable cluster size
+constexpr int PART_LD = TM + 1;
+constexpr uint32_t LBO = 128, SBO = (TK / 8) * 128;
+static_assert((size_t)NC * PART_LD * sizeof(double) <= (size_t)STAGES * STAGE_BYTES, "the tile reuses the stages");
+
+__device__ __forceinline__ uint64_t desc(uint32_t saddr) {
+  return (uint64_t)((saddr >> 4) & 0x3FFFu) | (uint64_t)(LBO >> 4) << 16 | (uint64_t)(SBO >> 4) << 32 | (uint64_t)1 << 46;
+}
+
+// element (row, k) of a K-major panel of TK columns
+__host__ __device__ __forceinline__ int core_off(int r, int k) {
+  return (r >> 3) * (TK / 8) * 64 + (k >> 3) * 64 + (r & 7) * 8 + (k & 7);
+}
+
+__device__ __forceinline__ unsigned long long abs_bits(double x) {
+  return (unsigned long long)__double_as_longlong(x) & 0x7fffffffffffffffull;
+}
+
+// e of a row or vector from the bits of its largest magnitude (every |x| <= 2^e), and the factor
+// 2^(e-6) of its digits: 0 for an all-zero row, NaN when an entry is infinite or NaN
+__device__ __forceinline__ int top_exponent(unsigned long long mx) { return (int)(mx >> 52) - 1022; }
+__device__ __forceinline__ double digit_scale(unsigned long long mx) {
+  if (mx >= 0x7ff0000000000000ull) return __longlong_as_double(0x7ff8000000000000ll);
+  if (mx < 0x0010000000000000ull) return 0.0;   // zero (subnormal magnitudes count as zero)
+  return scalbn(1.0, top_exponent(mx) - 6);
+}
+
+// the 8 base-128 digits of x for the top exponent e: q = round(x 2^(55 - e)), |q| <= 2^55, by
+// integer operations (the FP64 pipe is the narrow one), lowest digit first
+__device__ __forceinline__ void digits(double x, unsigned long long mx, float (&s)[ND]) {
+  const long long b = __double_as_longlong(x);
+  const int ex = (int)((b >> 52) & 0x7ff);
+  const bool ok = ex > 0 && mx < 0x7ff0000000000000ull;
+  const unsigned long long m = (b & 0xfffffffffffffll) | 0x10000000000000ll;
+  const int sh = ex - 1020 - top_exponent(mx);            // <= 2
+  unsigned long long mag = 0;
+  if (ok) mag = sh >= 0 ? m << sh : sh > -55 ? (m + (1ull << (-sh - 1))) >> -sh : 0;
+  long long q = b < 0 ? -(long long)mag : (long long)mag;
+#pragma unroll
+  for (int i = ND - 1; i >= 0; --i) {
+    const long long d = i ? ((q + 64) & 127) - 64 : q;
+    s[i] = (float)(int)d;
+    q = (q - d) >> 7;
+  }
+}
+
+// digit panels of eight consecutive K entries of one row: dst + i * stride, 16 bytes per digit
+__device__ __forceinline__ void store_digits(const double (&v)[8], unsigned long long mx, __nv_bfloat16* dst,
+                                             int stride) {
+  float s[8][ND];
+#pragma unroll
+  for (int q = 0; q < 8; ++q) digits(v[q], mx, s[q]);
+#pragma unroll
+  for (int i = 0; i < ND; ++i) {
+    uint32_t w[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const __nv_bfloat162 p = __floats2bfloat162_rn(s[2 * q][i], s[2 * q + 1][i]);
+      w[q] = *reinterpret_cast<const uint32_t*>(&p);
+    }
+    *reinterpret_cast<uint4*>(dst + (size_t)i * stride) = make_uint4(w[0], w[1], w[2], w[3]);
+  }
+}
+
+// Rows and columns of the tiled matrix: nI interior ones padded to MTI tiles / KI panels, then the
+// others, so that the dual views start at a tile and a panel.
+struct OzShape {
+  int nI, MTI, KI;      // interior rows and columns (the same DOFs)
+  int rows, cols;       // of the source matrix
+  int MT, KP;           // row tiles and panels of the padded one
+  __host__ __device__ int row(int tr) const {           // source row of padded row tr, or -1
+    if (tr < MTI * TM) return tr < nI ? tr : -1;
+    const int r = nI + tr - MTI * TM;
+    return r < rows ? r : -1;
+  }
+  __host__ __device__ int col(int tk) const {
+    if (tk < KI * TK) return tk < nI ? tk : -1;
+    const int c = nI + tk - KI * TK;
+    return c < cols ? c : -1;
+  }
+};
+
+// largest magnitude of every source row (bits), a warp per (key, padded row); its factor
+__global__ void __launch_bounds__(256)
+    k_oz_rowmax(OzShape sh, int64_t n_rows, int ld, int64_t kstride, const double* __restrict__ G,
+                unsigned long long* __restrict__ mx, double* __restrict__ scale) {
+  const int64_t t = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+  const int lane = threadIdx.x & 31;
+  if (t >= n_rows) return;
+  const int per = sh.MT * TM;
+  const int64_t key = t / per;
+  const int r = sh.row((int)(t - key * per));
+  unsigned long long m = 0;
+  if (r >= 0)
+    for (int k = lane; k < sh.cols; k += 32) m = max(m, abs_bits(G[key * kstride + (int64_t)r * ld + k]));
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+  if (lane == 0) {
+    mx[t] = m;
+    scale[t] = digit_scale(m);
+  }
+}
+
+// digits of the matrix: [key][row tile][panel][digit][core_off(row, k)], a thread per (row, 8 columns)
+__global__ void __launch_bounds__(128)
+    k_oz_tile(OzShape sh, int ld, int64_t kstride, const double* __restrict__ G,
+              const unsigned long long* __restrict__ mx, __nv_bfloat16* __restrict__ T) {
+  const int mt = blockIdx.x, k8 = blockIdx.y, r = threadIdx.x;   // padded columns [8 k8, 8 k8 + 8)
+  const int64_t key = blockIdx.z;
+  const int row = sh.row(mt * TM + r);
+  double v[8];
+#pragma unroll
+  for (int q = 0; q < 8; ++q) {
+    const int c = sh.col(8 * k8 + q);
+    v[q] = row >= 0 && c >= 0 ? G[key * kstride + (int64_t)row * ld + c] : 0.0;
+  }
+  const int kp = k8 / (TK / 8);
+  __nv_bfloat16* dst = T + (((size_t)key * sh.MT + mt) * sh.KP + kp) * A_ELEMS + core_off(r, (k8 % (TK / 8)) * 8);
+  store_digits(v, mx[(key * sh.MT + mt) * TM + r], dst, A_SLICE);
+}
+
+// largest magnitude of every cell vector of a tile over the view's columns (cleared before)
+__global__ void __launch_bounds__(256)
+    k_oz_cellmax(int n_cells, int n_K, const double* __restrict__ X, const int* __restrict__ rc,
+                 const int* __restrict__ tile_seg, const int* __restrict__ tile_c0, const int* __restrict__ seg_ptr,
+                 const int* __restrict__ perm, unsigned long long* __restrict__ mx) {
+  __shared__ unsigned long long red[16][NC + 1];
+  const int tile = blockIdx.x, c = threadIdx.x % NC, g = threadIdx.x / NC;
+  const int pos = tile_c0[tile] + c;
+  unsigned long long m = 0;
+  if (pos < seg_ptr[tile_seg[tile] + 1]) {
+    const int s = perm[pos];
+#pragma unroll 4
+    for (int k = blockIdx.y * 16 + g; k < n_K; k += gridDim.y * 16)
+      m = max(m, abs_bits(X[(size_t)rc[k] * n_cells + s]));
+  }
+  red[g][c] = m;
+  __syncthreads();
+  if (g == 0) {
+    for (int q = 1; q < 16; ++q) m = max(m, red[q][c]);
+    atomicMax(mx + (size_t)tile * NC + c, m);
+  }
+}
+
+// digits of the cell vectors: [tile][panel][core_off(digit * 16 + cell, k)], a thread per (cell, 8
+// columns); the view's padded columns start at panel kp0
+__global__ void __launch_bounds__(256)
+    k_oz_pack(OzShape sh, int n_cells, int kp0, int npan, const double* __restrict__ X,
+              const int* __restrict__ rdofs, const int* __restrict__ tile_seg, const int* __restrict__ tile_c0,
+              const int* __restrict__ seg_ptr, const int* __restrict__ perm,
+              const unsigned long long* __restrict__ mx, __nv_bfloat16* __restrict__ T) {
+  const int tile = blockIdx.x, c = threadIdx.x % NC;
+  const int k8 = blockIdx.y * 16 + threadIdx.x / NC;
+  if (k8 >= npan * (TK / 8)) return;
+  const int pos = tile_c0[tile] + c;
+  const bool in = pos < seg_ptr[tile_seg[tile] + 1];
+  const int s = in ? perm[pos] : 0;
+  double v[8];
+#pragma unroll
+  for (int q = 0; q < 8; ++q) {
+    const int k = sh.col(kp0 * TK + 8 * k8 + q);
+    v[q] = in && k >= 0 ? X[(size_t)rdofs[k] * n_cells + s] : 0.0;
+  }
+  const int kp = k8 / (TK / 8);
+  __nv_bfloat16* dst = T + ((size_t)tile * npan + kp) * B_ELEMS + core_off(c, (k8 % (TK / 8)) * 8);
+  store_digits(v, mx[(size_t)tile * NC + c], dst, NC * TK);
+}
+
+// integer sums of four digit accumulators (exact in FP32), combined: below 2^46
+__device__ __forceinline__ double combine4(uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
+  const long long v = ((long long)__float2int_rn(__uint_as_float(a)) << 21) +
+                      ((long long)__float2int_rn(__uint_as_float(b)) << 14) +
+                      ((long long)__float2int_rn(__uint_as_float(c)) << 7) +
+                      (long long)__float2int_rn(__uint_as_float(d));
+  // |v| < 2^51 as a double: the bits of 1.5 2^52 plus v, one subtraction
+  return __longlong_as_double(0x4338000000000000ll + v) - 6755399441055744.0;
+}
+
+__device__ __forceinline__ double ld_cluster(uint32_t addr, uint32_t rank) {
+  uint32_t ra;
+  double v;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(addr), "r"(rank));
+  asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(ra) : "memory");
+  return v;
+}
+
+__device__ __forceinline__ void tmem_ld4(uint32_t addr, uint32_t (&r)[4]) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"(addr)
+               : "memory");
+}
+
+// Rows [128 (mt0 + mt), ...) of the tiled matrix x 16 cells; the cluster's S CTAs share the view's
+// npan panels (from panel kp0 of the matrix), MAX_PANELS at most each.
+__global__ void __launch_bounds__(128, 2)
+    k_oz_mm(OzShape sh, int n_cells, int mt0, int kp0, int npan, int S, const __nv_bfloat16* __restrict__ GT,
+            const double* __restrict__ rscale, const __nv_bfloat16* __restrict__ XT,
+            const unsigned long long* __restrict__ cmax, const int* __restrict__ tile_seg,
+            const int* __restrict__ tile_c0, const int* __restrict__ seg_ptr, const int* __restrict__ perm,
+            const double* __restrict__ cscale, int n_R, int r_base, const int* __restrict__ rdofs,
+            const int* __restrict__ pdofs, double* __restrict__ Y, int* __restrict__ err, int mul_scale) {
+  extern __shared__ __align__(1024) unsigned char smem[];
+  __shared__ __align__(8) uint64_t full[STAGES], empty[STAGES], done;
+  __shared__ uint32_t tmem_slot;
+  __shared__ int fail;
+  __shared__ int cell[NC];
+  __shared__ double cs1[NC], cs2[NC];      // factor of a column's scaled rows, and of its corner rows
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int rank = blockIdx.x % S, tile = blockIdx.x / S, mt = mt0 + blockIdx.y;
+  const int key = tile_seg[tile];
+  const int p0 = (int)((int64_t)npan * rank / S), np = (int)((int64_t)npan * (rank + 1) / S) - p0;
+  const uint32_t s0 = smem_u32(smem);
+  if (warp == 0) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_slot)),
+                 "r"(TMEM_COLS)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  if (tid == 0) {
+    for (int s = 0; s < STAGES; ++s) {
+      mbar_init(smem_u32(&full[s]));
+      mbar_init(smem_u32(&empty[s]));
+    }
+    mbar_init(smem_u32(&done));
+    fail = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  const uint32_t tmem = tmem_slot;
+  if (tid == 0) {
+    int issued = 0;
+    bool ok = true;
+    for (int p = 0; p < np; ++p) {
+      const int st = p % STAGES;
+      if (p >= STAGES && !mbar_wait(smem_u32(&empty[st]), (uint32_t)((p / STAGES - 1) & 1))) {
+        ok = false;
+        break;
+      }
+      const uint32_t bar = smem_u32(&full[st]), dst = s0 + (uint32_t)(st * STAGE_BYTES);
+      expect_tx(bar, (uint32_t)STAGE_BYTES);
+      bulk_copy(dst, GT + (((size_t)key * sh.MT + mt) * sh.KP + kp0 + p0 + p) * A_ELEMS, 2 * A_ELEMS, bar);
+      bulk_copy(dst + 2 * A_ELEMS, XT + ((size_t)tile * npan + p0 + p) * B_ELEMS, 2 * B_ELEMS, bar);
+      ++issued;
+    }
+    if (!ok) {
+      fail = 1;
+      // let copies in flight land (bounded) before the shared memory is released
+      for (int q = max(0, issued - STAGES); q < issued; ++q)
+        mbar_wait(smem_u32(&full[q % STAGES]), (uint32_t)((q / STAGES) & 1));
+    }
+  } else if (tid == 32) {
+    bool ok = true;
+    for (int p = 0; p < np; ++p) {
+      const int st = p % STAGES;
+      if (!mbar_wait(smem_u32(&full[st]), (uint32_t)((p / STAGES) & 1))) {
+        ok = false;
+        break;
+      }
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      const uint32_t sa = s0 + (uint32_t)(st * STAGE_BYTES), sb = sa + 2 * A_ELEMS;
+#pragma unroll
+      for (int i = 0; i < ND; ++i) {
+        // kind::f16: D = F32, A = B = BF16, both K-major, N >> 3, M >> 4
+        const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)((ND - i) * NC >> 3) << 17) |
+                               ((uint32_t)(TM >> 4) << 24);
+        const uint32_t acc = (p > 0 || i > 0) ? 1u : 0u;   // digit 0 reaches every column first
+        asm volatile(
+            "{\n\t.reg .pred q;\n\t"
+            "setp.ne.b32 q, %4, 0;\n\t"
+            "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, q;\n\t}" ::"r"(tmem + (uint32_t)(i * NC)),
+            "l"(desc(sa + (uint32_t)(2 * i * A_SLICE))), "l"(desc(sb)), "r"(idesc), "r"(acc)
+            : "memory");
+      }
+      mma_commit(smem_u32(&empty[st]));
+    }
+    mma_commit(smem_u32(&done));
+    ok = mbar_wait(smem_u32(&done), 0) && ok;
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    if (!ok) fail = 1;
+  } else if (warp >= 2 && tid - 64 < NC) {
+    const int c = tid - 64, pos = tile_c0[tile] + c;
+    const int s = pos < seg_ptr[key + 1] ? perm[pos] : -1;
+    const double w = s >= 0 ? cscale[s] : 1.0, d = digit_scale(cmax[(size_t)tile * NC + c]);
+    cell[c] = s;
+    cs1[c] = d * (mul_scale ? w : 1.0 / w);   // c_s (S_DD rows) or 1 / c_s (G rows)
+    cs2[c] = d;
+  }
+  __syncwarp();
+  __syncthreads();
+  const bool good = !fail;   // accumulators complete, every wait met
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  if (!good && tid == 0) atomicOr(err, 4);
+  // digit sums of the tile's row (this thread's) and each cell to one FP64 value, in shared memory
+  double* part = reinterpret_cast<double*>(smem);   // [cell][129]
+  if (good) {
+    const uint32_t base = tmem + ((uint32_t)(warp * 32) << 16);
+#pragma unroll 1
+    for (int c = 0; c < NC; c += 4) {
+      uint32_t r[ND][4];
+#pragma unroll
+      for (int g = 0; g < ND; ++g) tmem_ld4(base + (uint32_t)(g * NC + c), r[g]);
+      asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const double hi = combine4(r[0][q], r[1][q], r[2][q], r[3][q]);
+        const double lo = combine4(r[4][q], r[5][q], r[6][q], r[7][q]);
+        part[(c + q) * PART_LD + tid] = fma(lo, 0x1p-49, hi * 0x1p-21);
+      }
+    }
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  if (S > 1) cluster_sync();
+  else __syncthreads();
+  // cells rank, rank + S, ... of the tile: sums over the cluster in CTA order, a lane per row
+  const int tr = mt * TM + tid, gi = sh.row(tr);
+  const double rs = rscale[(size_t)key * sh.MT * TM + tr];
+  const int o = gi < 0 ? -1 : r_base + gi < n_R ? rdofs[r_base + gi] : pdofs[r_base + gi - n_R];
+  for (int c = rank; c < NC; c += S) {
+    const uint32_t a = smem_u32(part + c * PART_LD + tid);
+    double v = 0.0;
+    if (S == 1) v = part[c * PART_LD + tid];
+    else
+      for (int q = 0; q < S; ++q) v += ld_cluster(a, (uint32_t)q);
+    if (cell[c] >= 0 && o >= 0 && good)
+      Y[(size_t)o * n_cells + cell[c]] = v * rs * (r_base + gi < n_R ? cs1[c] : cs2[c]);
+  }
+  if (S > 1) cluster_sync();   // peers have read this CTA's tile
+  else __syncthreads();
+  if (warp == 0) {
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TMEM_COLS) : "memory");
+  }
+}
+
+OzShape shape(int nI, int rows, int cols) {
+  OzShape s{};
+  s.nI = nI;
+  s.MTI = div_up(nI, TM);
+  s.KI = div_up(nI, TK);
+  s.rows = rows;
+  s.cols = cols;
+  s.MT = s.MTI + div_up(rows - nI, TM);
+  s.KP = s.KI + div_up(cols - nI, TK);
+  return s;
+}
+
+OzShape g_shape(const lat_ctx* h) { return shape(h->n_I, h->n_R + h->n_P, h->n_R); }
+OzShape s_shape(const lat_ctx* h) { return shape(0, h->n_R - h->n_I, h->n_R - h->n_I); }
+
+void split_matrix(lat_ctx* h, const OzShape& sh, int ld, int64_t kstride, const double* G, DBuf<__nv_bfloat16>& T,
+                  DBuf<double>& scale) {
+  const int keys = h->n_keys;
+  const int64_t rows = (int64_t)keys * sh.MT * TM;
+  T.ensure((size_t)keys * sh.MT * sh.KP * A_ELEMS);
+  scale.ensure((size_t)rows);
+  h->oz_max.ensure(std::max((size_t)rows, (size_t)h->oz_tiles * NC));
+  LAT_LAUNCH(h, k_oz_rowmax<<<div_up(rows * 32, 256), 256, 0, h->stream>>>(sh, rows, ld, kstride, G, h->oz_max.p,
+                                                                          scale.p));
+  LAT_LAUNCH(h, k_oz_tile<<<dim3(sh.MT, sh.KP * (TK / 8), keys), TM, 0, h->stream>>>(sh, ld, kstride, G, h->oz_max.p,
+                                                                                    T.p));
+  LAT_CHECK_LAUNCH();
+}
+
+void product(lat_ctx* h, const OzShape& sh, int mt0, int kp0, const DBuf<__nv_bfloat16>& T, const DBuf<double>& scale,
+             const int* rdofs, int r_base, const double* X, double* Y, int n_R, int mul_scale) {
+  const int npan = sh.KP - kp0, tiles = h->oz_tiles;
+  const int lo_c = kp0 ? sh.nI : 0, n_K = sh.cols - lo_c;
+  h->oz_X.ensure((size_t)tiles * npan * B_ELEMS);
+  h->oz_max.ensure((size_t)tiles * NC);
+  LAT_CUDA(cudaMemsetAsync(h->oz_max.p, 0, (size_t)tiles * NC * sizeof(unsigned long long), h->stream));
+  const int* ts = h->tile_seg_oz.p;
+  const int* tc = h->tile_c0_oz.p;
+  LAT_LAUNCH(h, k_oz_cellmax<<<dim3(tiles, std::max(1, std::min(16, div_up(n_K, 64)))), 256, 0, h->stream>>>(
+                    h->n_cells, n_K, X, rdofs + r_base + lo_c, ts, tc, h->seg_ptr.p, h->perm.p, h->oz_max.p));
+  LAT_LAUNCH(h, k_oz_pack<<<dim3(tiles, div_up(npan * (TK / 8), 16)), 256, 0, h->stream>>>(
+                    sh, h->n_cells, kp0, npan, X, rdofs + r_base, ts, tc, h->seg_ptr.p, h->perm.p, h->oz_max.p,
+                    h->oz_X.p));
+  const int S = div_up(npan, MAX_PANELS);
+  const size_t shm = (size_t)STAGES * STAGE_BYTES;
+  LAT_CUDA(cudaFuncSetAttribute(k_oz_mm, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm));
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(S * tiles, sh.MT - mt0);
+  cfg.blockDim = dim3(128);
+  cfg.dynamicSmemBytes = shm;
+  cfg.stream = h->stream;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = S;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  LAT_LAUNCH(h, LAT_CUDA(cudaLaunchKernelEx(&cfg, k_oz_mm, sh, h->n_cells, mt0, kp0, npan, S,
+                                            (const __nv_bfloat16*)T.p, (const double*)scale.p,
+                                            (const __nv_bfloat16*)h->oz_X.p, (const unsigned long long*)h->oz_max.p, ts,
+                                            tc, (const int*)h->seg_ptr.p, (const int*)h->perm.p,
+                                            (const double*)h->c_cell.p, n_R, r_base, rdofs, (const int*)h->pdofs.p, Y,
+                                            h->flag.p, mul_scale)));
+  LAT_CHECK_LAUNCH();
+}
+
+}  // namespace
+
+// Whether the FP64 mode's segmented products run on digits: blocks large enough that streaming 16
+// bytes per entry and the launches that split the cell vectors cost less than the FP64 pipe does
+// (36 cells of the strut cell's
+// dual block 50 us against 406, 512 cells of the whole block 0.40 ms against 6.0; the ring cells' dual
+// block is 56 columns, under 10 us either way), no more columns than the largest cluster sums exactly, and digits within 24 GB.
+bool oz_wanted(const lat_ctx* h) {
+  if (h->prec != LAT_FP64 || (int64_t)h->n_keys * 8 > h->n_cells) return false;
+  const OzShape g = g_shape(h), s = s_shape(h);
+  if (h->n_R - h->n_I < 512 || g.KP > MAX_SPLIT * MAX_PANELS) return false;
+  const double bytes = 2.0 * h->n_keys * A_ELEMS * ((double)g.MT * g.KP + (double)s.MT * s.KP);
+  return bytes <= 24e9;
+}
+
+// digits of the augmented local matrices and of the dual Schur complements (after the inversions)
+void run_oz_split(lat_ctx* h) {
+  const int nR = h->n_R, nP = h->n_P, nD = nR - h->n_I;
+  split_matrix(h, g_shape(h), nR, (int64_t)(nR + nP) * nR, h->G.p, h->oz_G, h->oz_Gs);
+  split_matrix(h, s_shape(h), nD, (int64_t)nD * nD, h->SDD.p, h->oz_S, h->oz_Ss);
+}
+
+void run_local_oz(lat_ctx* h, const double* X, double* Y, KinvMode mode) {
+  const OzShape g = g_shape(h);
+  product(h, g, mode == KINV_DUAL ? g.MTI : 0, mode == KINV_FULL ? 0 : g.KI, h->oz_G, h->oz_Gs, h->rdofs.p, 0, X, Y,
+          h->n_R, 0);
+}
+
+void run_sdd_oz(lat_ctx* h, const double* X, double* Y) {
+  product(h, s_shape(h), 0, 0, h->oz_S, h->oz_Ss, h->rdofs.p, h->n_I, X, Y, h->n_R, 1);
+}

@@ -27,6 +27,7 @@
 // after one cluster barrier sums its share of the columns over the cluster (distributed shared
 // memory, in CTA order) and stores it.
 #include "common.cuh"
+#include "tc_ptx.cuh"
 
 namespace {
 
@@ -55,10 +56,6 @@ struct TcCfg {
                                     ((uint32_t)(TM >> 4) << 24);
 };
 
-__device__ __forceinline__ uint32_t smem_u32(const void* p) {
-  return static_cast<uint32_t>(__cvta_generic_to_shared(p));
-}
-
 // shared-memory matrix descriptor: start, leading (K) and stride (8-row group) byte offsets,
 // version 1, no swizzle
 __device__ __forceinline__ uint64_t make_desc(uint32_t saddr) {
@@ -73,44 +70,6 @@ __device__ __forceinline__ uint64_t make_desc(uint32_t saddr) {
 // element (row r, k) of a K-major panel with TK columns, in bf16 elements
 __host__ __device__ __forceinline__ int core_off(int r, int k) {
   return (r >> 3) * (TK / 8) * 64 + (k >> 3) * 64 + (r & 7) * 8 + (k & 7);
-}
-
-__device__ __forceinline__ bool mbar_wait(uint32_t addr, uint32_t parity) {
-  for (int i = 0; i < (1 << 20); ++i) {
-    uint32_t done;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(done)
-        : "r"(addr), "r"(parity)
-        : "memory");
-    if (done) return true;
-  }
-  return false;
-}
-
-__device__ __forceinline__ void mbar_init(uint32_t addr) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(addr), "r"(1) : "memory");
-}
-
-__device__ __forceinline__ void bulk_copy(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
-  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
-               "l"(src), "r"(bytes), "r"(bar)
-               : "memory");
-}
-
-__device__ __forceinline__ void expect_tx(uint32_t bar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
-}
-
-__device__ __forceinline__ void mma_commit(uint32_t bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar)
-               : "memory");
-}
-
-__device__ __forceinline__ void cluster_sync() {
-  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
 // shared-memory float of CTA `rank` of the cluster at this CTA's shared address

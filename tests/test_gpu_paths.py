@@ -142,3 +142,33 @@ def test_symmetric_inverse_by_size(L, cell, dims, lu):
     err = (back[:nd] - v[:nd]).abs().max().item() / v[:nd].abs().max().item()
     assert err < 1e-9, err
     lat.close()
+
+
+@pytest.mark.parametrize("dims", [
+    (2, 2, 6),     # segments of 4 and 16 cells: one exactly full tile
+    (3, 3, 6),     # 9 and 36 cells: tiles of 9, 16, 16 and 4
+])
+def test_fp64_digit_products(L, dims):
+    """FP64 products on the tensor cores (digits): with equal cells at rest the one principal's local
+    blocks are every cell's, so K^-rom inverts K~ on vectors without multipliers (1e-9 as in the
+    force-all test); entries from 1e-12 to 1 in one vector, and a NaN stays a NaN."""
+    case = _case(latgen.strut_cell(12, 0.15), dims, seed=None)
+    lat = L.Lattice.from_case(case)
+    u = lat.lattice_predictor(0.0)
+    lat.select_principal_cells(u, 1e-3, 4)
+    lat.lattice_prepare_solver(u, lat.lattice_default_opts(precond_tangent=0, max_enrich=0))
+    s = lat.sizes
+    nd = s.n_loc * s.n_cells + s.n_primal
+    rng = np.random.default_rng(8)
+    for lo in (0, -12):
+        w = rng.uniform(-1, 1, s.n_dof) * 10.0 ** rng.uniform(lo, 0, s.n_dof)
+        v = lat.feti_from_global(torch.tensor(w, device="cuda"))
+        v[nd:] = 0
+        Kv = lat.feti_apply(0, v)
+        Kv[nd:] = 0
+        back = lat.feti_apply(1, Kv)
+        err = (back[:nd] - v[:nd]).abs().max().item() / v[:nd].abs().max().item()
+        assert err < 1e-9, err
+    Kv[s.n_cells * (s.n_loc // 2) + 1] = float("nan")
+    assert torch.isnan(lat.feti_apply(1, Kv)[:nd]).any()
+    lat.close()
