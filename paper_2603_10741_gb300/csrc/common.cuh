@@ -219,6 +219,11 @@ struct lat_ctx {
   DBuf<__nv_bfloat16> oz_G, oz_S, oz_X;
   DBuf<double> oz_Gs, oz_Ss;
   DBuf<unsigned long long> oz_max;
+  // large inversions (fp64_tc.cu): digits of the panel C (A operand), of R and Pi (B operand), their
+  // row maxima, the pivot block and R = C Pi
+  DBuf<__nv_bfloat16> sp_C, sp_B;
+  DBuf<unsigned long long> sp_max;
+  DBuf<double> sp_P, sp_R;
   bool indefinite = false;              // a principal's remaining block had a negative pivot
   bool coarse_indefinite = false;       // the coarse matrix had a negative pivot
   int64_t pcg_its_total = 0;            // interface PCG iterations since the last reset
@@ -454,6 +459,10 @@ void build_feti(lat_ctx* h, int level);
 void prepare_enriched(lat_ctx* h, const lat_newton_opts* o, const double* u_glob);
 void gj_invert(lat_ctx* h, double* A, int n, int batch, int64_t bs, int neg_bit, int split = -1,
                double* snap = nullptr);
+void sweep_small(lat_ctx* h, double* A, int n, int batch, int64_t bs, int neg_bit);
+void run_sweep_panel(lat_ctx* h, double* A, int n, int batch, int64_t bs, int k0, int kw, int neg_bit);
+constexpr int kSweepPanel = 128;              // panel width of the large inversions
+constexpr int kSweepLarge = 384;              // matrices from this size on are swept in such panels
 void run_coarse_blocked(lat_ctx* h, const double* S, int64_t np, bool dense);
 bool coarse_block_plan(lat_ctx* h, bool fallback = false);
 int coarse_coop_grid(lat_ctx* h);

@@ -1127,12 +1127,10 @@ struct SolverTmp {
 // ---------------------------------------------------------------------------------------------
 }  // namespace
 
-// invert `batch` symmetric n x n matrices stored with a stride of bs elements (in place; the lower
-// triangle is read).  With split in (0, n) the pivot blocks stop at `split` once: the trailing block
-// [split, n)^2 then holds the Schur complement A_22 - A_21 A_11^{-1} A_12, copied to snap
-// ([batch][n-split]^2) before the sweep continues.
-void gj_invert(lat_ctx* h, double* A, int n, int batch, int64_t bs, int neg_bit, int split,
-               double* snap) {
+namespace {
+
+// one step of the sweep on the FP64 pipe: pivot block [k0, k0 + kw), kw <= 32
+void sweep_step(lat_ctx* h, double* A, int n, int batch, int64_t bs, int k0, int kw, int neg_bit) {
   // workspace kept in the handle: no allocation and no host synchronisation per inversion
   DBuf<double>& Pinv = h->gj_P;
   DBuf<double>& Cbuf = h->gj_C;
@@ -1140,47 +1138,69 @@ void gj_invert(lat_ctx* h, double* A, int n, int batch, int64_t bs, int neg_bit,
   Pinv.ensure((size_t)batch * GJB * GJB);
   Cbuf.ensure((size_t)batch * n * GJB);
   Rbuf.ensure((size_t)batch * n * GJB);
-  if (snap && split == 0) {
-    LAT_LAUNCH(h, k_gj_snapshot<<<dim3(div_up((int64_t)n * n, 256), batch), 256, 0, h->stream>>>(n, bs, 0, A, snap));
-    LAT_CHECK_LAUNCH();
-  }
   const int T = fp64_tile(n, batch, h->n_sm);
   const dim3 rows(div_up(n, kSwRows), batch);
   const int64_t per = div_up(n, T);
   const dim3 tiles((unsigned)(per * (per + 1) / 2), batch);
-  for (int k0 = 0; k0 < n;) {
-    int kw = std::min(GJB, n - k0);
-    if (split > 0 && k0 < split) kw = std::min(kw, split - k0);
-    {
-      KernelTimer kt(h, "gj_pivot");
-      if ((int64_t)rows.x * batch <= h->n_sm) {
-        LAT_LAUNCH(h, k_sw_rows<true><<<rows, 256, 0, h->stream>>>(n, bs, k0, kw, A, Pinv.p, Cbuf.p, Rbuf.p, h->flag.p,
-                                                                   neg_bit));
-      } else {
-        LAT_LAUNCH(h, k_sw_pivot<<<batch, 256, 0, h->stream>>>(n, bs, k0, kw, A, Pinv.p, h->flag.p, neg_bit));
-        LAT_LAUNCH(h, k_sw_rows<false><<<rows, 256, 0, h->stream>>>(n, bs, k0, kw, A, Pinv.p, Cbuf.p, Rbuf.p,
-                                                                    h->flag.p, neg_bit));
-      }
-    }
-    {
-      KernelTimer kt(h, "gj_update");
-      auto go = [&](auto kern) {
-        LAT_LAUNCH(h, kern<<<tiles, 256, 0, h->stream>>>(n, bs, k0, kw, A, Pinv.p, Cbuf.p, Rbuf.p));
-      };
-      if (T == 64) go(k_sw_update<64>);
-      else if (T == 32) go(k_sw_update<32>);
-      else go(k_sw_update<16>);
-    }
-    LAT_CHECK_LAUNCH();
-    k0 += kw;
-    if (snap && k0 == split && split < n) {
-      const int m = n - split;
-      LAT_LAUNCH(h, k_gj_snapshot<<<dim3(div_up((int64_t)m * m, 256), batch), 256, 0, h->stream>>>(n, bs, split, A, snap));
-      LAT_CHECK_LAUNCH();
+  {
+    KernelTimer kt(h, "gj_pivot");
+    if ((int64_t)rows.x * batch <= h->n_sm) {
+      LAT_LAUNCH(h, k_sw_rows<true><<<rows, 256, 0, h->stream>>>(n, bs, k0, kw, A, Pinv.p, Cbuf.p, Rbuf.p, h->flag.p,
+                                                                 neg_bit));
+    } else {
+      LAT_LAUNCH(h, k_sw_pivot<<<batch, 256, 0, h->stream>>>(n, bs, k0, kw, A, Pinv.p, h->flag.p, neg_bit));
+      LAT_LAUNCH(h, k_sw_rows<false><<<rows, 256, 0, h->stream>>>(n, bs, k0, kw, A, Pinv.p, Cbuf.p, Rbuf.p, h->flag.p,
+                                                                  neg_bit));
     }
   }
+  KernelTimer kt(h, "gj_update");
+  auto go = [&](auto kern) {
+    LAT_LAUNCH(h, kern<<<tiles, 256, 0, h->stream>>>(n, bs, k0, kw, A, Pinv.p, Cbuf.p, Rbuf.p));
+  };
+  if (T == 64) go(k_sw_update<64>);
+  else if (T == 32) go(k_sw_update<32>);
+  else go(k_sw_update<16>);
+  LAT_CHECK_LAUNCH();
+}
+
+void sweep_finish(lat_ctx* h, double* A, int n, int batch, int64_t bs) {
   LAT_LAUNCH(h, k_sw_finish<<<dim3(div_up(n, 32), div_up(n, 32), batch), 256, 0, h->stream>>>(n, bs, A));
   LAT_CHECK_LAUNCH();
+}
+
+}  // namespace
+
+// inverses of small matrices (the pivot blocks of the large ones)
+void sweep_small(lat_ctx* h, double* A, int n, int batch, int64_t bs, int neg_bit) {
+  for (int k0 = 0; k0 < n; k0 += GJB) sweep_step(h, A, n, batch, bs, k0, std::min(GJB, n - k0), neg_bit);
+  sweep_finish(h, A, n, batch, bs);
+}
+
+// invert `batch` symmetric n x n matrices stored with a stride of bs elements (in place; the lower
+// triangle is read).  With split in (0, n) the pivot blocks stop at `split` once: the trailing block
+// [split, n)^2 then holds the Schur complement A_22 - A_21 A_11^{-1} A_12, copied to snap
+// ([batch][n-split]^2) before the sweep continues.  From kSweepLarge rows on the sweep takes panels of
+// 128 columns with the updates on the tensor cores (fp64_tc.cu); below, the chain of
+// pivot blocks bounds both forms and the panels only add launches (25 ring blocks of 568 rows: 235
+// us of update per 32 columns before, 102 us per 128 now).
+void gj_invert(lat_ctx* h, double* A, int n, int batch, int64_t bs, int neg_bit, int split,
+               double* snap) {
+  auto snapshot = [&](int at) {
+    const int64_t m = n - at;
+    LAT_LAUNCH(h, k_gj_snapshot<<<dim3(div_up(m * m, 256), batch), 256, 0, h->stream>>>(n, bs, at, A, snap));
+    LAT_CHECK_LAUNCH();
+  };
+  if (snap && split == 0) snapshot(0);
+  const bool large = n >= kSweepLarge;
+  for (int k0 = 0; k0 < n;) {
+    int kw = std::min(large ? kSweepPanel : GJB, n - k0);
+    if (split > 0 && k0 < split) kw = std::min(kw, split - k0);
+    if (large) run_sweep_panel(h, A, n, batch, bs, k0, kw, neg_bit);
+    else sweep_step(h, A, n, batch, bs, k0, kw, neg_bit);
+    k0 += kw;
+    if (snap && k0 == split && split < n) snapshot(split);
+  }
+  sweep_finish(h, A, n, batch, bs);
 }
 
 // principal tangents the local blocks are built from: the full K^r, or its material part
@@ -1344,6 +1364,7 @@ void run_prepare_solver(lat_ctx* h, const lat_newton_opts* o, const double* u_gl
   int fl = 0;
   LAT_CUDA(cudaMemcpyAsync(&fl, h->flag.p, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
   LAT_CUDA(cudaStreamSynchronize(h->stream));
+  LAT_REQUIRE(!(fl & 4), LAT_ETIMEOUT, "a tensor-core wait in a local inversion gave up");
   LAT_REQUIRE(!(fl & 1), LAT_EINDEFINITE, "a local remaining-DOF matrix or the coarse matrix is singular");
   h->indefinite = (fl & 2) != 0;          // a principal's remaining block has a negative pivot
   h->coarse_indefinite = (fl & 8) != 0;   // the coarse matrix has a negative pivot

@@ -69,22 +69,24 @@ __device__ __forceinline__ double digit_scale(unsigned long long mx) {
   return scalbn(1.0, top_exponent(mx) - 6);
 }
 
-// the 8 base-128 digits of x for the top exponent e: q = round(x 2^(55 - e)), |q| <= 2^55, by
-// integer operations (the FP64 pipe is the narrow one), lowest digit first
+// the 8 base-2^DB digits of x for the top exponent e: q = round(x 2^(7 DB + 6 - e)), |q| <=
+// 2^(7 DB + 6), by integer operations (the FP64 pipe is the narrow one), lowest digit first
+template <int DB>
 __device__ __forceinline__ void digits(double x, unsigned long long mx, float (&s)[ND]) {
+  constexpr long long half = 1ll << (DB - 1), mask = (1ll << DB) - 1;
   const long long b = __double_as_longlong(x);
   const int ex = (int)((b >> 52) & 0x7ff);
   const bool ok = ex > 0 && mx < 0x7ff0000000000000ull;
   const unsigned long long m = (b & 0xfffffffffffffll) | 0x10000000000000ll;
-  const int sh = ex - 1020 - top_exponent(mx);            // <= 2
+  const int sh = ex - 1022 - top_exponent(mx) + 7 * DB - 47;   // x = m 2^(ex - 1075); at most 7 DB - 47
   unsigned long long mag = 0;
   if (ok) mag = sh >= 0 ? m << sh : sh > -55 ? (m + (1ull << (-sh - 1))) >> -sh : 0;
   long long q = b < 0 ? -(long long)mag : (long long)mag;
 #pragma unroll
   for (int i = ND - 1; i >= 0; --i) {
-    const long long d = i ? ((q + 64) & 127) - 64 : q;
+    const long long d = i ? ((q + half) & mask) - half : q;
     s[i] = (float)(int)d;
-    q = (q - d) >> 7;
+    q = (q - d) >> DB;
   }
 }
 
@@ -93,7 +95,7 @@ __device__ __forceinline__ void store_digits(const double (&v)[8], unsigned long
                                              int stride) {
   float s[8][ND];
 #pragma unroll
-  for (int q = 0; q < 8; ++q) digits(v[q], mx, s[q]);
+  for (int q = 0; q < 8; ++q) digits<7>(v[q], mx, s[q]);
 #pragma unroll
   for (int i = 0; i < ND; ++i) {
     uint32_t w[4];
@@ -210,11 +212,12 @@ __global__ void __launch_bounds__(256)
   store_digits(v, mx[(size_t)tile * NC + c], dst, NC * TK);
 }
 
-// integer sums of four digit accumulators (exact in FP32), combined: below 2^46
+// integer sums of four digit accumulators (exact in FP32, up to 2^24), combined: below 2^50
+template <int DB>
 __device__ __forceinline__ double combine4(uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
-  const long long v = ((long long)__float2int_rn(__uint_as_float(a)) << 21) +
-                      ((long long)__float2int_rn(__uint_as_float(b)) << 14) +
-                      ((long long)__float2int_rn(__uint_as_float(c)) << 7) +
+  const long long v = ((long long)__float2int_rn(__uint_as_float(a)) << (3 * DB)) +
+                      ((long long)__float2int_rn(__uint_as_float(b)) << (2 * DB)) +
+                      ((long long)__float2int_rn(__uint_as_float(c)) << DB) +
                       (long long)__float2int_rn(__uint_as_float(d));
   // |v| < 2^51 as a double: the bits of 1.5 2^52 plus v, one subtraction
   return __longlong_as_double(0x4338000000000000ll + v) - 6755399441055744.0;
@@ -349,8 +352,8 @@ __global__ void __launch_bounds__(128, 2)
       asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
-        const double hi = combine4(r[0][q], r[1][q], r[2][q], r[3][q]);
-        const double lo = combine4(r[4][q], r[5][q], r[6][q], r[7][q]);
+        const double hi = combine4<7>(r[0][q], r[1][q], r[2][q], r[3][q]);
+        const double lo = combine4<7>(r[4][q], r[5][q], r[6][q], r[7][q]);
         part[(c + q) * PART_LD + tid] = fma(lo, 0x1p-49, hi * 0x1p-21);
       }
     }
@@ -476,4 +479,266 @@ void run_local_oz(lat_ctx* h, const double* X, double* Y, KinvMode mode) {
 
 void run_sdd_oz(lat_ctx* h, const double* X, double* Y) {
   product(h, s_shape(h), 0, 0, h->oz_S, h->oz_Ss, h->rdofs.p, h->n_I, X, Y, h->n_R, 1);
+}
+
+// ------------------------------------------------------------------------------------------------
+// Large symmetric inversions (gj_invert) by sweeps of 128-column panels, the rank-128 updates on digits
+// ------------------------------------------------------------------------------------------------
+// The sweep of a panel p (see feti.cu): C = A_.p, Pi = A_pp^{-1} by sweeps of 32 columns, R = C Pi and
+// A_ij -= C_i R_j^T on the lower triangle.  Both products run on digits: C as the A operand (a row's
+// digits scaled by its own maximum), the rows of Pi (symmetric) and of R as the B operand, 128
+// columns at most, so base-256 digits (|s| <= 128, products up to 2^14, 8 of them over 128 columns)
+// still sum exactly and what is dropped is about 2^-62 of the row maxima; base-128 digits left
+// inverses of the strut cell's blocks 2.4 times further off than FP64 sweeps do.  An entry of A then takes four FP64 operations per panel
+// instead of 128.  Per panel: the chain of the pivot block (four 32-column steps, 26 us each), two
+// products and the splitting of C, Pi and R.  Three 2616 matrices: 9 ms against 53 ms.
+namespace {
+
+constexpr int SW = kSweepPanel;
+constexpr int SP = SW / TK;                // K panels
+constexpr int SN = 32;                     // columns of a product's tile
+constexpr int SB_ELEMS = ND * SN * TK;     // 8 KiB
+constexpr int SSTAGE_BYTES = 2 * (A_ELEMS + SB_ELEMS);
+constexpr int SSTAGES = 2;                 // 80 KiB, two CTAs per SM
+constexpr int SCOLS = ND * SN;             // 256 tensor-memory columns
+
+// digits of one row of a panel (128 values in shared memory, zero beyond the panel's width) by one
+// warp: lane l takes the columns 4l .. 4l + 3; the row's largest magnitude goes to *mx.  base: the
+// row's core-matrix position in the first panel; pstride / dstride: elements between panels / digits
+__device__ __forceinline__ void row_digits(const double* v, int lane, __nv_bfloat16* base, int pstride, int dstride,
+                                           unsigned long long* mx) {
+  double x[4];
+  unsigned long long m = 0;
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    x[q] = v[4 * lane + q];
+    m = max(m, abs_bits(x[q]));
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+  if (lane == 0) *mx = m;
+  float s[4][ND];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) digits<8>(x[q], m, s[q]);
+  const int k = 4 * lane;
+  __nv_bfloat16* d = base + (size_t)(k / TK) * pstride + core_off(0, k % TK);
+#pragma unroll
+  for (int i = 0; i < ND; ++i) {
+    const __nv_bfloat162 a = __floats2bfloat162_rn(s[0][i], s[1][i]), b = __floats2bfloat162_rn(s[2][i], s[3][i]);
+    *reinterpret_cast<uint2*>(d + (size_t)i * dstride) =
+        make_uint2(*reinterpret_cast<const uint32_t*>(&a), *reinterpret_cast<const uint32_t*>(&b));
+  }
+}
+
+// C's digits [b][row tile][panel][digit][128 x 16] and row maxima, 32 rows per CTA (rows above the
+// panel are read as columns of the lower triangle); the CTAs that hold panel rows also copy A_pp
+__global__ void __launch_bounds__(256)
+    k_sp_panel(int n, int64_t bs, int k0, int kw, int MT, const double* __restrict__ A, __nv_bfloat16* __restrict__ Cd,
+               unsigned long long* __restrict__ cmax, double* __restrict__ P) {
+  __shared__ double S[32][SW + 1];
+  const int b = blockIdx.y, i0 = blockIdx.x * 32, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const double* a = A + (size_t)b * bs;
+  const bool above = i0 + 32 <= k0;
+  for (int t = threadIdx.x; t < 32 * SW; t += 256) {
+    const int r = above ? t % 32 : t / SW, c = above ? t / 32 : t % SW;
+    const int i = i0 + r, k = k0 + c;
+    const double v = i < n && c < kw ? a[(size_t)max(i, k) * n + min(i, k)] : 0.0;
+    S[r][c] = v;
+    if (i >= k0 && i < k0 + kw && c < kw) P[(size_t)b * SW * SW + (size_t)(i - k0) * kw + c] = v;
+  }
+  __syncthreads();
+  for (int r = warp; r < 32; r += 8) {
+    const int row = i0 + r;   // rows up to the padded tile's end have zero digits
+    if (row >= MT * TM) continue;
+    __nv_bfloat16* base = Cd + ((size_t)b * MT + row / TM) * SP * A_ELEMS + core_off(row % TM, 0);
+    row_digits(S[r], lane, base, A_ELEMS, A_SLICE, cmax + (size_t)b * MT * TM + row);
+  }
+}
+
+// digits of the rows of an [rows][ld] FP64 matrix (kw columns) as a B operand:
+// [b][32-row tile][panel][core_off(digit * 32 + row, k)]
+__global__ void __launch_bounds__(256)
+    k_sp_rows(int rows, int ld, int64_t bs, int kw, int NT, const double* __restrict__ X, __nv_bfloat16* __restrict__ Xd,
+              unsigned long long* __restrict__ xmax) {
+  __shared__ double S[8][SW];
+  const int b = blockIdx.y, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int row = blockIdx.x * 8 + warp;
+  for (int c = lane; c < SW; c += 32) S[warp][c] = row < rows && c < kw ? X[(size_t)b * bs + (size_t)row * ld + c] : 0.0;
+  __syncwarp();
+  if (row >= NT * SN) return;
+  __nv_bfloat16* base = Xd + ((size_t)b * NT + row / SN) * SP * SB_ELEMS + core_off(row % SN, 0);
+  row_digits(S[warp], lane, base, SB_ELEMS, SN * TK, xmax + (size_t)b * NT * SN + row);
+}
+
+// One 128 x 32 tile of C B^T.  UPDATE: A_ij -= (C R^T)_ij on the lower triangle, A_ip = R_i, A_pp =
+// -Pi; else: R = C Pi (B the rows of Pi).
+template <bool UPDATE>
+__global__ void __launch_bounds__(128, 2)
+    k_sp_mm(int n, int64_t bs, int k0, int kw, int MT, int NT, const __nv_bfloat16* __restrict__ Cd,
+            const unsigned long long* __restrict__ cmax, const __nv_bfloat16* __restrict__ Bd,
+            const unsigned long long* __restrict__ bmax, const double* __restrict__ P, double* __restrict__ R,
+            double* __restrict__ A, int* __restrict__ err) {
+  extern __shared__ __align__(1024) unsigned char smem[];
+  __shared__ __align__(8) uint64_t full[SSTAGES], empty[SSTAGES], done;
+  __shared__ uint32_t tmem_slot;
+  __shared__ int fail;
+  __shared__ double cs[SN];
+  const int tid = threadIdx.x, warp = tid >> 5, b = blockIdx.y;
+  int mt, nt;
+  if (UPDATE) {   // lower tiles: 4 (mt + 1) column tiles per row tile
+    mt = (int)((sqrtf(2.f * (float)blockIdx.x + 1.f) - 1.f) * 0.5f);
+    while (2 * (mt + 1) * (mt + 2) <= (int)blockIdx.x) ++mt;
+    while (2 * mt * (mt + 1) > (int)blockIdx.x) --mt;
+    nt = (int)blockIdx.x - 2 * mt * (mt + 1);
+  } else {
+    mt = blockIdx.x / NT;
+    nt = blockIdx.x % NT;
+  }
+  if (nt >= NT) return;
+  const int np = (kw + TK - 1) / TK;
+  const uint32_t s0 = smem_u32(smem);
+  if (warp == 0) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_slot)),
+                 "r"(SCOLS)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  if (tid == 0) {
+    for (int s = 0; s < SSTAGES; ++s) {
+      mbar_init(smem_u32(&full[s]));
+      mbar_init(smem_u32(&empty[s]));
+    }
+    mbar_init(smem_u32(&done));
+    fail = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  const uint32_t tmem = tmem_slot;
+  if (tid == 0) {
+    int issued = 0;
+    bool ok = true;
+    for (int p = 0; p < np; ++p) {
+      const int st = p % SSTAGES;
+      if (p >= SSTAGES && !mbar_wait(smem_u32(&empty[st]), (uint32_t)((p / SSTAGES - 1) & 1))) {
+        ok = false;
+        break;
+      }
+      const uint32_t bar = smem_u32(&full[st]), dst = s0 + (uint32_t)(st * SSTAGE_BYTES);
+      expect_tx(bar, (uint32_t)SSTAGE_BYTES);
+      bulk_copy(dst, Cd + (((size_t)b * MT + mt) * SP + p) * A_ELEMS, 2 * A_ELEMS, bar);
+      bulk_copy(dst + 2 * A_ELEMS, Bd + (((size_t)b * NT + nt) * SP + p) * SB_ELEMS, 2 * SB_ELEMS, bar);
+      ++issued;
+    }
+    if (!ok) {
+      fail = 1;
+      for (int q = max(0, issued - SSTAGES); q < issued; ++q)
+        mbar_wait(smem_u32(&full[q % SSTAGES]), (uint32_t)((q / SSTAGES) & 1));
+    }
+  } else if (tid == 32) {
+    bool ok = true;
+    for (int p = 0; p < np; ++p) {
+      const int st = p % SSTAGES;
+      if (!mbar_wait(smem_u32(&full[st]), (uint32_t)((p / SSTAGES) & 1))) {
+        ok = false;
+        break;
+      }
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      const uint32_t sa = s0 + (uint32_t)(st * SSTAGE_BYTES), sb = sa + 2 * A_ELEMS;
+#pragma unroll
+      for (int i = 0; i < ND; ++i) {
+        const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)((ND - i) * SN >> 3) << 17) |
+                               ((uint32_t)(TM >> 4) << 24);
+        const uint32_t acc = (p > 0 || i > 0) ? 1u : 0u;
+        asm volatile(
+            "{\n\t.reg .pred q;\n\t"
+            "setp.ne.b32 q, %4, 0;\n\t"
+            "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, q;\n\t}" ::"r"(tmem + (uint32_t)(i * SN)),
+            "l"(desc(sa + (uint32_t)(2 * i * A_SLICE))), "l"(desc(sb)), "r"(idesc), "r"(acc)
+            : "memory");
+      }
+      mma_commit(smem_u32(&empty[st]));
+    }
+    mma_commit(smem_u32(&done));
+    ok = mbar_wait(smem_u32(&done), 0) && ok;
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    if (!ok) fail = 1;
+  } else if (tid >= 64 && tid < 64 + SN) {
+    cs[tid - 64] = digit_scale(bmax[((size_t)b * NT + nt) * SN + tid - 64]) * 0x1p-24;
+  }
+  __syncwarp();
+  __syncthreads();
+  const bool good = !fail;
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  if (!good && tid == 0) atomicOr(err, 4);
+  if (good) {
+    const uint32_t base = tmem + ((uint32_t)(warp * 32) << 16);
+    const int gi = mt * TM + tid, j0 = nt * SN;
+    const double rs = digit_scale(cmax[((size_t)b * MT + mt) * TM + tid]);
+    double* a = A + (size_t)b * bs;
+    const double* Rb = R + (size_t)b * n * SW;
+    const bool ip = gi >= k0 && gi < k0 + kw;
+#pragma unroll 1
+    for (int c = 0; c < SN; c += 4) {
+      uint32_t r[ND][4];
+#pragma unroll
+      for (int g = 0; g < ND; ++g) tmem_ld4(base + (uint32_t)(g * SN + c), r[g]);
+      asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const double hi = combine4<8>(r[0][q], r[1][q], r[2][q], r[3][q]);
+        const double lo = combine4<8>(r[4][q], r[5][q], r[6][q], r[7][q]);
+        const double v = fma(lo, 0x1p-32, hi), f = rs * cs[c + q];
+        const int gj = j0 + c + q;
+        if (!UPDATE) {
+          if (gi < n && gj < SW) R[((size_t)b * n + gi) * SW + gj] = v * f;
+        } else if (gi < n && gj <= gi) {
+          const bool jp = gj >= k0 && gj < k0 + kw;
+          double* dst = a + (size_t)gi * n + gj;
+          if (ip) *dst = jp ? -P[(size_t)b * SW * SW + (size_t)(gi - k0) * kw + (gj - k0)] : Rb[(size_t)gj * SW + (gi - k0)];
+          else if (jp) *dst = Rb[(size_t)gi * SW + (gj - k0)];
+          else *dst = fma(-f, v, *dst);
+        }
+      }
+    }
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  if (warp == 0) {
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(SCOLS) : "memory");
+  }
+}
+
+}  // namespace
+
+// one panel [k0, k0 + kw) of the sweep of `batch` n x n matrices (lower triangles)
+void run_sweep_panel(lat_ctx* h, double* A, int n, int batch, int64_t bs, int k0, int kw, int neg_bit) {
+  const int MT = div_up(n, TM), NT = div_up(n, SN), PT = SW / SN;
+  h->sp_C.ensure((size_t)batch * MT * SP * A_ELEMS);
+  h->sp_B.ensure((size_t)batch * (NT + PT) * SP * SB_ELEMS);
+  h->sp_max.ensure((size_t)batch * (MT * TM + (NT + PT) * SN));
+  h->sp_P.ensure((size_t)batch * SW * SW);
+  h->sp_R.ensure((size_t)batch * n * SW);
+  unsigned long long* cmax = h->sp_max.p;
+  unsigned long long* rmax = cmax + (size_t)batch * MT * TM;
+  unsigned long long* pmax = rmax + (size_t)batch * NT * SN;
+  __nv_bfloat16* Rd = h->sp_B.p;
+  __nv_bfloat16* Pd = Rd + (size_t)batch * NT * SP * SB_ELEMS;
+  const size_t shm = (size_t)SSTAGES * SSTAGE_BYTES;
+  LAT_CUDA(cudaFuncSetAttribute(k_sp_mm<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm));
+  LAT_CUDA(cudaFuncSetAttribute(k_sp_mm<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm));
+  LAT_LAUNCH(h, k_sp_panel<<<dim3(MT * TM / 32, batch), 256, 0, h->stream>>>(n, bs, k0, kw, MT, A, h->sp_C.p, cmax,
+                                                                            h->sp_P.p));
+  sweep_small(h, h->sp_P.p, kw, batch, (int64_t)SW * SW, neg_bit);
+  LAT_LAUNCH(h, k_sp_rows<<<dim3(SW / 8, batch), 256, 0, h->stream>>>(kw, kw, (int64_t)SW * SW, kw, PT, h->sp_P.p, Pd,
+                                                                      pmax));
+  LAT_LAUNCH(h, k_sp_mm<false><<<dim3(MT * PT, batch), 128, shm, h->stream>>>(n, bs, k0, kw, MT, PT, h->sp_C.p, cmax, Pd,
+                                                                              pmax, h->sp_P.p, h->sp_R.p, A, h->flag.p));
+  LAT_LAUNCH(h, k_sp_rows<<<dim3(NT * SN / 8, batch), 256, 0, h->stream>>>(n, SW, (int64_t)n * SW, kw, NT, h->sp_R.p, Rd,
+                                                                          rmax));
+  LAT_LAUNCH(h, k_sp_mm<true><<<dim3(2 * MT * (MT + 1), batch), 128, shm, h->stream>>>(
+                    n, bs, k0, kw, MT, NT, h->sp_C.p, cmax, Rd, rmax, h->sp_P.p, h->sp_R.p, A, h->flag.p));
+  LAT_CHECK_LAUNCH();
 }

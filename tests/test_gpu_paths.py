@@ -122,6 +122,8 @@ def test_residual_and_tangent_by_element_and_cell_count(L, cell, dims):
     (latgen.ring_cell(2), (2, 9), 0),        # blocks of 8 and 12 rows: less than one pivot block
     (latgen.solid_cell(6, 2), (9, 9), 0),    # 90 remaining DOFs: 32 + 32 + 26, split inside a pivot block
     (latgen.solid_cell(4, 3), (3, 3, 3), 1), # 351 remaining DOFs, 81 of them interior; coarse blocks as block LU
+    (latgen.ring_cell(14), (2, 2), 0),       # 440 remaining DOFs: panels of 128, the last one of 40 after 16
+    (latgen.solid_cell(6, 3), (1, 2, 2), 0), # 1005 remaining DOFs, split at 375 inside a 128-row tile
 ])
 def test_symmetric_inverse_by_size(L, cell, dims, lu):
     """Local and coarse inverses by sweeps: K^-rom K~ = I on the force-all path, whose every local
