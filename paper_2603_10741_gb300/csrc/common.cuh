@@ -125,6 +125,7 @@ struct lat_ctx {
   DBuf<int> lam_p, lam_m;             // [n_lambda] local entries of the +/- copies
   DBuf<int> dual_entry, dual_l1, dual_l2;  // dual copies and their multipliers (+-(l+1), 0 = none)
   DBuf<double> dual_scale;            // [n_dual] 1/multiplicity of the node
+  DBuf<double> lam_scale;             // [n_lambda] the same for the node a multiplier joins copies of
   DBuf<int2> dual_lk;                 // [n_D][n_cells] signed multipliers (l1, l2) of each dual copy
   DBuf<float> dual_lsc;               // [n_D][n_cells] its 1/multiplicity
   int64_t n_dual = 0;
@@ -236,11 +237,11 @@ struct lat_ctx {
   // launches of named kernels (lattice_set_timing / lattice_kernel_time)
   bool timing = false;
   bool timing_apply_only = false;       // time only the reduced / plain tangent action kernels
-  // interface PCG iteration captured as a CUDA graph (dropped whenever the solver is set up)
+  // interface PCG: a CUDA graph whose while node runs the iterations (dropped whenever the solver is
+  // set up)
   cudaGraphExec_t pcg_exec = nullptr;
   cudaStream_t cap_stream = nullptr;    // private stream the graph is captured on
-  int pcg_exec_check = -1;              // whether the captured iteration copies its scalars out
-  int64_t pcg_graph_kernels = 0;        // kernels in one replay (added to n_launch per replay)
+  int64_t pcg_graph_kernels = 0;        // kernels in one iteration (added to n_launch per iteration)
   bool graphs_ok = true;
   std::map<std::string, std::vector<std::pair<cudaEvent_t, cudaEvent_t>>> ev;
   std::vector<cudaEvent_t> ev_pool;

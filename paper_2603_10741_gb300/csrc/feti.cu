@@ -39,13 +39,20 @@ __global__ void k_axpby(int64_t n, double a, const double* __restrict__ x, doubl
     y[i] = a * x[i] + b * y[i];
 }
 
-// PCG scalars (see k_sum_part_pcg): sc[0] rz, sc[1] pq, sc[2] rz_new, sc[3] alpha, sc[4] beta,
-// sc[5] frozen (once p.q <= 0 or r.z <= 0 the iteration stops updating)
-// p = z + b[0] p  (p left unchanged when the iteration is frozen)
-__global__ void k_xpby_s(int64_t n, const double* __restrict__ z, const double* __restrict__ b,
-                         const double* __restrict__ frozen, double* __restrict__ p) {
-  if (frozen[0] != 0.0) return;
-  const double c = b[0];
+// Interface PCG.  Scalars of one solve on the device, so that iterations need no host: the two dot
+// products' kernels end with the step length, the direction coefficient and the decision to go on.
+struct PcgScalars {
+  double rz, pq, rz0, alpha, beta;
+  double frozen;      // set once p.q <= 0 or r.z <= 0: the iteration stops updating
+  double its;         // iterations done
+  double max_it, tol2; // limits of this solve: iterations, (r.z / r0.z0) to stop at (0: never)
+};
+
+// p = z + beta p  (p left unchanged when the iteration is frozen)
+__global__ void k_xpby_s(int64_t n, const double* __restrict__ z, const PcgScalars* __restrict__ sc,
+                         double* __restrict__ p) {
+  if (sc->frozen != 0.0) return;
+  const double c = sc->beta;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
     p[i] = z[i] + c * p[i];
 }
@@ -68,34 +75,10 @@ __global__ void k_sum_part(int n, const double* __restrict__ part, double* __res
   if (threadIdx.x == 0) out[0] = v;
 }
 
-// the same sum into the PCG scalars, followed by the step length (step = 0: sc[1] = p.q,
-// alpha = rz / pq) or the direction coefficient (step = 1: sc[2] = r.z, beta = rz_new / rz),
-// with the breakdown guard that freezes the iteration: one launch per PCG dot and scalar
-__global__ void k_sum_part_pcg(int n, const double* __restrict__ part, double* __restrict__ sc, int step) {
-  __shared__ double red[32];
-  double v = 0;
-  for (int i = threadIdx.x; i < n; i += blockDim.x) v += part[i];
-  v = block_sum(v, red);
-  if (threadIdx.x == 0) {
-    if (step == 0) {
-      sc[1] = v;
-      const bool ok = sc[5] == 0.0 && sc[1] > 0.0 && sc[0] > 0.0;
-      if (!ok) sc[5] = 1.0;
-      sc[3] = ok ? sc[0] / sc[1] : 0.0;
-    } else {
-      sc[2] = v;
-      const bool ok = sc[5] == 0.0 && sc[2] > 0.0 && sc[0] > 0.0;
-      if (!ok) sc[5] = 1.0;
-      sc[4] = ok ? sc[2] / sc[0] : 0.0;
-      sc[0] = sc[2];
-    }
-  }
-}
-
-// x += a[0] p and r -= a[0] q in one pass (the PCG updates of solution and residual)
-__global__ void k_axpy2_s(int64_t n, const double* __restrict__ a, const double* __restrict__ p,
+// x += alpha p and r -= alpha q in one pass (the PCG updates of solution and residual)
+__global__ void k_axpy2_s(int64_t n, const PcgScalars* __restrict__ sc, const double* __restrict__ p,
                           const double* __restrict__ q, double* __restrict__ x, double* __restrict__ r) {
-  const double c = a[0];
+  const double c = sc->alpha;
   if (c == 0.0) return;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
     x[i] += c * p[i];
@@ -173,34 +156,133 @@ __global__ void k_jump(int64_t L, const int* __restrict__ lp, const int* __restr
   lam[l] = accumulate ? lam[l] + v : v;
 }
 
-// y[dual entry] += a * (B^T lambda) (optionally scaled by 1/multiplicity)
+// y[dual entry] += a * (B^T lambda)
 __global__ void k_jump_t(int64_t nd, const int* __restrict__ de, const int* __restrict__ l1,
-                         const int* __restrict__ l2, const double* __restrict__ scale,
-                         const double* __restrict__ lam, double a, double* __restrict__ y) {
+                         const int* __restrict__ l2, const double* __restrict__ lam, double a,
+                         double* __restrict__ y) {
   int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (e >= nd) return;
   double v = 0;
   int c1 = l1[e], c2 = l2[e];
   if (c1) v += (c1 > 0 ? 1.0 : -1.0) * lam[abs(c1) - 1];
   if (c2) v += (c2 > 0 ? 1.0 : -1.0) * lam[abs(c2) - 1];
-  if (scale) v *= scale[e];
   y[de[e]] += a * v;
 }
 
-// scaled jump  lambda_l = (x[p] * s_p - x[m] * s_m)  with per-entry scaling gathered from a
-// dense scale array indexed like the local vector
-__global__ void k_jump_scaled(int64_t L, const int* __restrict__ lp, const int* __restrict__ lm,
-                              const double* __restrict__ x, const double* __restrict__ wloc,
-                              double* __restrict__ lam) {
-  int64_t l = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (l >= L) return;
-  lam[l] = x[lp[l]] * wloc[lp[l]] - x[lm[l]] * wloc[lm[l]];
+// The interface iteration on vectors outside the tensor-core path: y[dual entry] = B^T v (scaled by
+// 1/multiplicity when `scale` is given) with v formed on the fly, so that the vector updates need no
+// pass of their own:
+//   DIR: the new direction z + beta p (p when frozen);  else: the new residual y - alpha q
+// The other entries of y stay zero (cleared once per solve).
+template <bool DIR>
+__global__ void k_pcg_scatter(int64_t nd, const int* __restrict__ de, const int* __restrict__ l1,
+                              const int* __restrict__ l2, const double* __restrict__ scale,
+                              const PcgScalars* __restrict__ sc, const double* __restrict__ u,
+                              const double* __restrict__ w, double* __restrict__ y) {
+  const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (e >= nd) return;
+  const int c[2] = {l1[e], l2[e]};
+  const bool plain = DIR ? sc->frozen != 0.0 : sc->alpha == 0.0;
+  const double f = DIR ? sc->beta : -sc->alpha;
+  double v = 0;
+#pragma unroll
+  for (int q = 0; q < 2; ++q) {
+    if (!c[q]) continue;
+    const int l = abs(c[q]) - 1;
+    // DIR: u = z, w = p;  else u = the residual, w = q
+    const double x = plain ? (DIR ? w[l] : u[l]) : u[l] + f * w[l];
+    v += c[q] > 0 ? x : -x;
+  }
+  if (scale) v *= scale[e];
+  y[de[e]] = v;
 }
 
-__global__ void k_fill_dual_weights(int64_t nd, const int* __restrict__ de, const double* __restrict__ sc,
-                                    double* __restrict__ wloc) {
-  int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (e < nd) wloc[de[e]] = sc[e];
+// The jump of a local vector, the vector updates of the multiplier (FLY: the ones the scatter formed
+// on the fly; without it they ran before), the dot product, and in the block that ends last the PCG
+// scalars:
+//   DIR: p = z + beta p, q = B t2, p.q, alpha;  else: x += alpha p, r -= alpha q, z = B_D t2, r.z,
+//   beta, and whether the loop goes on (told to the graph's loop node when there is one).
+// A multiplier belongs to one thread.  Partial sums are added in block order: deterministic.
+constexpr int kPcgBlocks = 1216;
+
+template <bool DIR, bool FLY>
+__global__ void __launch_bounds__(256)
+    k_pcg_jump(int64_t L, const int* __restrict__ lp, const int* __restrict__ lm, const double* __restrict__ ls,
+               const double* __restrict__ t2, double* __restrict__ x, double* __restrict__ r, double* __restrict__ z,
+               double* __restrict__ p, double* __restrict__ q, PcgScalars* __restrict__ sc,
+               double* __restrict__ part, unsigned* __restrict__ ticket, cudaGraphConditionalHandle loop, int has_loop) {
+  __shared__ double red[32];
+  __shared__ bool last;
+  const double al = sc->alpha, be = sc->beta;
+  const bool frozen = sc->frozen != 0.0;
+  double v = 0;
+  for (int64_t l = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; l < L; l += (int64_t)gridDim.x * blockDim.x) {
+    const double j = t2[lp[l]] - t2[lm[l]];
+    if (DIR) {
+      double pl = p[l];
+      if (FLY && !frozen) {
+        pl = z[l] + be * pl;
+        p[l] = pl;
+      }
+      q[l] = j;
+      v += pl * j;
+    } else {
+      double rl = r[l];
+      if (FLY && al != 0.0) {
+        x[l] += al * p[l];
+        rl = rl - al * q[l];
+        r[l] = rl;
+      }
+      const double zl = j * ls[l];
+      z[l] = zl;
+      v += rl * zl;
+    }
+  }
+  v = block_sum(v, red);
+  if (threadIdx.x == 0) {
+    part[blockIdx.x] = v;
+    __threadfence();
+    last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+  }
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  v = 0;
+  for (int i = threadIdx.x; i < (int)gridDim.x; i += blockDim.x) v += __ldcg(part + i);
+  v = block_sum(v, red);
+  if (threadIdx.x != 0) return;
+  *ticket = 0;
+  if (DIR) {
+    sc->pq = v;
+    const bool ok = !frozen && v > 0.0 && sc->rz > 0.0;
+    if (!ok) sc->frozen = 1.0;
+    sc->alpha = ok ? sc->rz / v : 0.0;
+  } else {
+    const bool ok = !frozen && v > 0.0 && sc->rz > 0.0;
+    if (!ok) sc->frozen = 1.0;
+    sc->beta = ok ? v / sc->rz : 0.0;
+    sc->rz = v;
+    sc->its += 1.0;
+    const bool go = sc->its < sc->max_it &&
+                    (sc->tol2 == 0.0 || (ok && sc->rz0 > 0.0 && !(v <= sc->tol2 * sc->rz0)));
+    if (has_loop) cudaGraphSetConditional(loop, go ? 1u : 0u);
+  }
+}
+
+// scalars at the start of a solve, after r0.z0 is in sc->rz
+__global__ void k_pcg_start(PcgScalars* __restrict__ sc, unsigned* __restrict__ ticket, double max_it, double tol2) {
+  sc->pq = sc->alpha = sc->beta = sc->frozen = sc->its = 0.0;
+  sc->rz0 = sc->rz;
+  sc->max_it = max_it;
+  sc->tol2 = tol2;
+  *ticket = 0;
+}
+
+// z = B_D t2: the scaled jump (both copies of a multiplier carry their node's 1/multiplicity)
+__global__ void k_jump_scaled(int64_t L, const int* __restrict__ lp, const int* __restrict__ lm,
+                              const double* __restrict__ ls, const double* __restrict__ t2, double* __restrict__ z) {
+  const int64_t l = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (l < L) z[l] = (t2[lp[l]] - t2[lm[l]]) * ls[l];
 }
 
 // saddle-point vector -> global vector: corners from the primal part, other DOFs the mean of
@@ -1434,7 +1516,7 @@ void feti_operator(lat_ctx* h, const double* v, double* w, bool with_lambda, boo
   if (h->n_lambda) {
     if (with_lambda)
       LAT_LAUNCH(h, k_jump_t<<<div_up(h->n_dual, 256), 256, 0, h->stream>>>(h->n_dual, h->dual_entry.p, h->dual_l1.p,
-          h->dual_l2.p, nullptr, la_of(h, v), 1.0, w));
+          h->dual_l2.p, la_of(h, v), 1.0, w));
     LAT_LAUNCH(h, k_jump<<<div_up(h->n_lambda, 256), 256, 0, h->stream>>>(h->n_lambda, h->lam_p.p, h->lam_m.p, v, 1.0,
                                                               la_of(h, w), 0));
   }
@@ -1473,8 +1555,8 @@ void run_coarse_solve(lat_ctx* h, const double* g, double* x) {
 //   KINV_DUAL     the same, and only the dual and corner rows of w are formed (the interface
 //                 operator B K^-rom B^T reads no others): the trailing dual block,
 //                 (n_R - n_I + n_P) x (n_R - n_I) instead of (n_R + n_P) x n_R.
-//   lam (KINV_DUAL on the tensor-core path only): v is B^T lam on the dual DOFs and zero
-//                 elsewhere, formed by the product's operand packing (v is not read).
+//   lam (KINV_DUAL and KINV_DUAL_IN on the tensor-core path only): v is B^T lam on the dual DOFs and
+//                 zero elsewhere, formed by the product's operand packing (v is not read).
 void kinv(lat_ctx* h, const double* v, double* w, KinvMode mode = KINV_FULL, const double* lam = nullptr) {
   const int ns = h->n_cells, nR = h->n_R, nP = h->n_P;
   const int lo_r = mode == KINV_DUAL ? h->n_I : 0;   // first row and column of the view
@@ -1548,43 +1630,32 @@ void kinv(lat_ctx* h, const double* v, double* w, KinvMode mode = KINV_FULL, con
   }
 }
 
-// S_op p = B K^-rom B^T p (multiplier vectors); uses tmp (saddle sized) as scratch
 // the tensor-core path forms B^T lambda inside its operand packing (no zeroed local vector, no
 // scatter): BF16 mode with the segmented products (few keys)
 bool fused_dual(const lat_ctx* h) { return h->prec == LAT_MIXED_BF16 && (int64_t)h->n_keys * 8 <= h->n_cells; }
+// the Dirichlet preconditioner's products take the same path; the lumped one reads a local vector
+bool fused_schur(const lat_ctx* h) { return h->iface == 0 && fused_dual(h); }
 
-void dual_op(lat_ctx* h, const double* p, double* q, double* t1, double* t2) {
-  const int64_t nloc = (int64_t)h->n_loc * h->n_cells;
-  if (fused_dual(h)) {
-    kinv(h, nullptr, t2, KINV_DUAL, p);
-  } else {
-    LAT_CUDA(cudaMemsetAsync(t1, 0, (nloc + h->n_primal) * sizeof(double), h->stream));
-    LAT_LAUNCH(h, k_jump_t<<<div_up(h->n_dual, 256), 256, 0, h->stream>>>(h->n_dual, h->dual_entry.p, h->dual_l1.p,
-                                                            h->dual_l2.p, nullptr, p, 1.0, t1));
-    LAT_CHECK_LAUNCH();
-    kinv(h, t1, t2, KINV_DUAL);   // t1 vanishes off the dual DOFs; only dual rows of t2 are read
-  }
-  LAT_LAUNCH(h, k_jump<<<div_up(h->n_lambda, 256), 256, 0, h->stream>>>(h->n_lambda, h->lam_p.p, h->lam_m.p, t2, 1.0, q, 0));
+// B^T of the direction (or of the residual, scaled) into the local vector t1
+template <bool DIR>
+void pcg_scatter(lat_ctx* h, const double* u, const double* w, const PcgScalars* sc, double* t1) {
+  LAT_LAUNCH(h, k_pcg_scatter<DIR><<<div_up(h->n_dual, 256), 256, 0, h->stream>>>(
+                    h->n_dual, h->dual_entry.p, h->dual_l1.p, h->dual_l2.p, DIR ? nullptr : h->dual_scale.p, sc, u, w,
+                    t1));
   LAT_CHECK_LAUNCH();
 }
 
-// lumped preconditioner z = B_D K~_dd B_D^T r
-void dual_precond(lat_ctx* h, const double* r, double* z, double* t1, double* t2, double* wloc) {
+// local part of the interface preconditioner M = B_D S B_D^T: t2 = S B_D^T r, from the multiplier
+// vector r (tensor-core path) or from t1 = B_D^T r
+void dual_precond_local(lat_ctx* h, const double* r, double* t1, double* t2) {
   const int64_t nloc = (int64_t)h->n_loc * h->n_cells;
-  const bool fused = h->iface == 0 && fused_dual(h);
-  if (!fused) {
-    LAT_CUDA(cudaMemsetAsync(t1, 0, (nloc + h->n_primal) * sizeof(double), h->stream));
-    LAT_LAUNCH(h, k_jump_t<<<div_up(h->n_dual, 256), 256, 0, h->stream>>>(h->n_dual, h->dual_entry.p, h->dual_l1.p,
-                                                            h->dual_l2.p, h->dual_scale.p, r, 1.0, t1));
-    LAT_CHECK_LAUNCH();
-  }
   if (h->iface == 0) {
     // Dirichlet: local dual Schur complements of the cells' principals, c_s S_DD^{slot(s)} x_D;
     // with few keys as a segmented product over the key-ordered cells (as the local inverses)
     const int nD = h->n_R - h->n_I;
     const size_t shm = (size_t)nD * sizeof(double);
     const bool seg = (int64_t)h->n_keys * 8 <= h->n_cells;
-    if (fused) {
+    if (fused_schur(h)) {
       run_sdd_tc(h, r, t2);   // tcgen05, BF16 operand pairs, FP32 accumulation; operand B_D^T r
     } else if (h->oz) {
       KernelTimer kt(h, "dual_schur");
@@ -1619,8 +1690,53 @@ void dual_precond(lat_ctx* h, const double* r, double* z, double* t1, double* t2
     run_apply(h, h->x32.p, h->y32.p, 1, pr_of(h, t1), true);
     run_f2d(h, nloc, h->y32.p, t2);
   }
-  LAT_LAUNCH(h, k_jump_scaled<<<div_up(h->n_lambda, 256), 256, 0, h->stream>>>(h->n_lambda, h->lam_p.p, h->lam_m.p, t2, wloc, z));
   LAT_CHECK_LAUNCH();
+}
+
+// the loop node's graph: one iteration captured as the body of a while node on the handle's private
+// stream (the caller's may be the legacy default stream, which cannot be captured)
+template <typename Body>
+bool capture_pcg_loop(lat_ctx* h, Body&& body) {
+  drop_pcg_graph(h);
+  const int64_t n0 = h->n_launch;
+  if (!h->cap_stream) LAT_CUDA(cudaStreamCreateWithFlags(&h->cap_stream, cudaStreamNonBlocking));
+  cudaStream_t user = h->stream;
+  cudaGraph_t g = nullptr;
+  bool ok = cudaGraphCreate(&g, 0) == cudaSuccess;
+  cudaGraphConditionalHandle loop = 0;
+  ok = ok && cudaGraphConditionalHandleCreate(&loop, g, 1, cudaGraphCondAssignDefault) == cudaSuccess;
+  cudaGraphNodeParams np = {};
+  np.type = cudaGraphNodeTypeConditional;
+  np.conditional.handle = loop;
+  np.conditional.type = cudaGraphCondTypeWhile;
+  np.conditional.size = 1;
+  cudaGraphNode_t node;
+  ok = ok && cudaGraphAddNode(&node, g, nullptr, nullptr, 0, &np) == cudaSuccess;
+  if (ok && cudaStreamBeginCaptureToGraph(h->cap_stream, np.conditional.phGraph_out[0], nullptr, nullptr, 0,
+                                          cudaStreamCaptureModeRelaxed) == cudaSuccess) {
+    h->stream = h->cap_stream;
+    try {
+      body(loop, 1);
+    } catch (const LatError&) {
+      ok = false;
+    }
+    h->stream = user;
+    cudaGraph_t out = nullptr;
+    ok = cudaStreamEndCapture(h->cap_stream, &out) == cudaSuccess && ok;
+    ok = ok && cudaGraphInstantiate(&h->pcg_exec, g, 0) == cudaSuccess;
+  } else {
+    ok = false;
+  }
+  if (ok) {
+    h->pcg_graph_kernels = h->n_launch - n0;
+  } else {
+    h->graphs_ok = false;   // this handle keeps the launch-by-launch path from now on
+    h->pcg_exec = nullptr;
+  }
+  if (g) cudaGraphDestroy(g);
+  h->n_launch = n0;
+  cudaGetLastError();
+  return ok;
 }
 
 }  // namespace
@@ -1636,7 +1752,7 @@ void run_kinv(lat_ctx* h, const double* v, double* w) {
 
 void run_block_precond(lat_ctx* h, const double* v, double* w, int pcg_iters, double pcg_rtol) {
   const int64_t L = h->n_lambda;
-  double* t = h->kv_tmp[2].p;   // K^-rom v_u, later v_u - B^T z
+  double* t = h->kv_tmp[2].p;   // K^-rom v_u
   double* t1 = h->kv_tmp[3].p;
   double* t2 = h->kv_tmp[4].p;
   double* pv = h->pcg_ws.p;     // five multiplier-sized work vectors
@@ -1650,108 +1766,99 @@ void run_block_precond(lat_ctx* h, const double* v, double* w, int pcg_iters, do
   double* z = pv + 2 * L;
   double* p = pv + 3 * L;
   double* q = pv + 4 * L;
-  double* wloc = h->kv_tmp[1].p;  // dual weights (1/multiplicity) as a dense local array
   LAT_REQUIRE((size_t)5 * L <= h->pcg_ws.n, LAT_EINVAL, "multiplier work space too small");
   const int64_t nloc = (int64_t)h->n_loc * h->n_cells;
-  LAT_CUDA(cudaMemsetAsync(wloc, 0, nloc * sizeof(double), h->stream));
-  LAT_LAUNCH(h, k_fill_dual_weights<<<div_up(h->n_dual, 256), 256, 0, h->stream>>>(h->n_dual, h->dual_entry.p, h->dual_scale.p, wloc));
+  const bool tc = fused_dual(h), tcs = fused_schur(h);
   // y = v_l - B t
   LAT_CUDA(cudaMemcpyAsync(y, la_of(h, v), L * sizeof(double), cudaMemcpyDeviceToDevice, h->stream));
   LAT_LAUNCH(h, k_jump<<<div_up(L, 256), 256, 0, h->stream>>>(L, h->lam_p.p, h->lam_m.p, t, -1.0, y, 1));
   LAT_CHECK_LAUNCH();
   // PCG on S x = y from x = 0
   LAT_CUDA(cudaMemsetAsync(x, 0, L * sizeof(double), h->stream));
-  double* sc = h->red_part.p + 3000;  // PCG scalars, see k_sum_part_pcg
+  // the local vector of the scatters: zero off the dual entries, which every scatter rewrites
+  if (!tc || !tcs) LAT_CUDA(cudaMemsetAsync(t1, 0, (nloc + h->n_primal) * sizeof(double), h->stream));
+  auto* sc = reinterpret_cast<PcgScalars*>(h->red_part.p + 3000);
+  auto* ticket = reinterpret_cast<unsigned*>(h->red_part.p + 3020);
+  double* part = h->red_part.p + 1024;
   if (pcg_iters > 0) {
-    // PCG until the preconditioned residual r^T M r has dropped by pcg_rtol^2 (checked on the
-    // host after every iteration), at most pcg_iters iterations, or until breakdown.  One
-    // iteration updates the search direction first (p = z + beta p; p = z on the first pass, from
-    // p = 0 and beta = 0), so that every iteration is the same sequence of launches: outside the
-    // kernel-timing mode it is captured once per preconditioner setup as a CUDA graph and replayed.
-    LAT_CUDA(cudaMemsetAsync(sc, 0, 8 * sizeof(double), h->stream));
-    dual_precond(h, y, z, t1, t2, wloc);
+    // PCG until the preconditioned residual r^T M r has dropped by pcg_rtol^2 (0: never), at most
+    // pcg_iters iterations, or until breakdown.  An iteration updates the search direction first (p =
+    // z + beta p; p = z on the first pass, from p = 0 and beta = 0), so that every one is the same
+    // sequence of launches.  Outside the kernel-timing mode it is the body of a graph's while node,
+    // captured once per preconditioner setup: the loop runs on the device, and the host, which used
+    // to read the residual after every iteration (about 15 us of an iteration of 60 to 300), waits
+    // once per solve.  The two dot products share the jump kernels' pass and their last block leaves
+    // the scalars; outside the tensor-core path, whose packing reads the vectors at random, the
+    // updates of p, x and r ride along as well.  An iteration was 18 graph nodes (15 with the
+    // packing), now 9 (11).
+    LAT_CUDA(cudaMemsetAsync(sc, 0, sizeof(PcgScalars), h->stream));
     LAT_CUDA(cudaMemsetAsync(p, 0, L * sizeof(double), h->stream));
-    dev_dot(h, L, y, z, sc);
-    double rz0 = -1.0;
-    if (pcg_rtol > 0) {
-      LAT_CUDA(cudaMemcpyAsync(h->h_pinned + 8, sc, sizeof(double), cudaMemcpyDeviceToHost, h->stream));
-      LAT_CUDA(cudaStreamSynchronize(h->stream));
-      rz0 = h->h_pinned[8];
-    }
+    if (!tcs) pcg_scatter<false>(h, y, q, sc, t1);   // alpha = 0: B_D^T y
+    dual_precond_local(h, y, t1, t2);
+    LAT_LAUNCH(h, k_jump_scaled<<<div_up(L, 256), 256, 0, h->stream>>>(L, h->lam_p.p, h->lam_m.p, h->lam_scale.p, t2, z));
+    dev_dot(h, L, y, z, &sc->rz);
+    LAT_LAUNCH(h, k_pcg_start<<<1, 1, 0, h->stream>>>(sc, ticket, (double)pcg_iters, pcg_rtol * pcg_rtol));
+    LAT_CHECK_LAUNCH();
     const int nb = ew_blocks(h, L);
-    const bool check = pcg_rtol > 0;
-    auto body = [&]() {
-      LAT_LAUNCH(h, k_xpby_s<<<nb, 256, 0, h->stream>>>(L, z, sc + 4, sc + 5, p));
-      dual_op(h, p, q, t1, t2);
-      const int rb = red_blocks(L);
-      LAT_LAUNCH(h, k_dot_part<<<rb, 256, 0, h->stream>>>(L, p, q, h->red_part.p + 1024));
-      LAT_LAUNCH(h, k_sum_part_pcg<<<1, 512, 0, h->stream>>>(rb, h->red_part.p + 1024, sc, 0));   // alpha
-      LAT_LAUNCH(h, k_axpy2_s<<<nb, 256, 0, h->stream>>>(L, sc + 3, p, q, x, y));
-      dual_precond(h, y, z, t1, t2, wloc);
-      LAT_LAUNCH(h, k_dot_part<<<rb, 256, 0, h->stream>>>(L, y, z, h->red_part.p + 1024));
-      LAT_LAUNCH(h, k_sum_part_pcg<<<1, 512, 0, h->stream>>>(rb, h->red_part.p + 1024, sc, 1));   // beta
-      if (check)
-        LAT_CUDA(cudaMemcpyAsync(h->h_pinned + 8, sc, 6 * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
+    const int jb = (int)std::min<int64_t>(kPcgBlocks, div_up(L, 256));
+    auto jump = [&](auto kern, cudaGraphConditionalHandle loop, int has_loop) {
+      LAT_LAUNCH(h, kern<<<jb, 256, 0, h->stream>>>(L, h->lam_p.p, h->lam_m.p, h->lam_scale.p, t2, x, y, z, p, q, sc, part,
+                                                    ticket, loop, has_loop));
+    };
+    auto body = [&](cudaGraphConditionalHandle loop, int has_loop) {
+      if (tc) {
+        LAT_LAUNCH(h, k_xpby_s<<<nb, 256, 0, h->stream>>>(L, z, sc, p));
+        kinv(h, nullptr, t2, KINV_DUAL, p);
+        jump(k_pcg_jump<true, false>, loop, 0);
+      } else {
+        pcg_scatter<true>(h, z, p, sc, t1);
+        kinv(h, t1, t2, KINV_DUAL);   // t1 vanishes off the dual DOFs; only dual rows of t2 are read
+        jump(k_pcg_jump<true, true>, loop, 0);
+      }
+      if (tcs) {
+        LAT_LAUNCH(h, k_axpy2_s<<<nb, 256, 0, h->stream>>>(L, sc, p, q, x, y));
+        dual_precond_local(h, y, t1, t2);
+        jump(k_pcg_jump<false, false>, loop, has_loop);
+      } else {
+        pcg_scatter<false>(h, y, q, sc, t1);
+        dual_precond_local(h, y, t1, t2);
+        jump(k_pcg_jump<false, true>, loop, has_loop);
+      }
       LAT_CHECK_LAUNCH();
     };
     bool graph = (!h->timing || h->timing_apply_only) && h->graphs_ok;
-    if (graph && (!h->pcg_exec || h->pcg_exec_check != (int)check)) {
-      if (h->pcg_exec) {
-        cudaGraphExecDestroy(h->pcg_exec);
-        h->pcg_exec = nullptr;
+    if (graph && !h->pcg_exec) graph = capture_pcg_loop(h, body);
+    auto* hs = reinterpret_cast<PcgScalars*>(h->h_pinned + 8);
+    auto read = [&] {
+      LAT_CUDA(cudaMemcpyAsync(hs, sc, sizeof(PcgScalars), cudaMemcpyDeviceToHost, h->stream));
+      LAT_CUDA(cudaStreamSynchronize(h->stream));
+    };
+    if (graph) {
+      LAT_CUDA(cudaGraphLaunch(h->pcg_exec, h->stream));
+      read();
+      h->n_launch += (int64_t)hs->its * h->pcg_graph_kernels;
+    } else {
+      for (int it = 0; it < pcg_iters; ++it) {
+        body(0, 0);
+        if (pcg_rtol == 0) continue;
+        read();
+        if (hs->frozen != 0.0 || !(hs->rz0 > 0) || hs->rz <= hs->tol2 * hs->rz0) break;
       }
-      // captured on a private stream (the caller's may be the legacy default stream, which
-      // cannot be captured); replays are ordered on the handle's stream
-      const int64_t n0 = h->n_launch;
-      if (!h->cap_stream) LAT_CUDA(cudaStreamCreateWithFlags(&h->cap_stream, cudaStreamNonBlocking));
-      cudaStream_t user = h->stream;
-      cudaGraph_t g = nullptr;
-      cudaError_t e1 = cudaStreamBeginCapture(h->cap_stream, cudaStreamCaptureModeRelaxed);
-      if (e1 == cudaSuccess) {
-        h->stream = h->cap_stream;
-        try {
-          body();
-        } catch (const LatError&) {
-          graph = false;
-        }
-        h->stream = user;
-        e1 = cudaStreamEndCapture(h->cap_stream, &g);
-      }
-      if (graph && e1 == cudaSuccess && g && cudaGraphInstantiate(&h->pcg_exec, g, 0) == cudaSuccess) {
-        h->pcg_graph_kernels = h->n_launch - n0;
-        h->pcg_exec_check = (int)check;
-      } else {
-        graph = false;
-        h->graphs_ok = false;   // this handle keeps the launch-by-launch path from now on
-        h->pcg_exec = nullptr;
-      }
-      if (g) cudaGraphDestroy(g);
-      h->n_launch = n0;
-      cudaGetLastError();
+      read();
     }
-    int it = 0;
-    for (; it < pcg_iters; ++it) {
-      if (graph) {
-        LAT_CUDA(cudaGraphLaunch(h->pcg_exec, h->stream));
-        h->n_launch += h->pcg_graph_kernels;
-      } else {
-        body();
-      }
-      if (check) {
-        LAT_CUDA(cudaStreamSynchronize(h->stream));
-        const double rz = h->h_pinned[8], frozen = h->h_pinned[13];
-        if (frozen != 0.0 || !(rz0 > 0) || rz <= pcg_rtol * pcg_rtol * rz0) break;
-      }
-    }
-    h->pcg_its_total += std::min(it + 1, pcg_iters);
+    h->pcg_its_total += (int64_t)hs->its;
   }
   // z_l = -x ;  w_u = K^-rom (v_u - B^T z_l) = K^-rom v_u + K^-rom B^T x, the first term kept in t
   // from above and the second with the dual columns only (B^T x vanishes off the dual DOFs)
-  LAT_CUDA(cudaMemsetAsync(t1, 0, (nloc + h->n_primal) * sizeof(double), h->stream));
-  LAT_LAUNCH(h, k_jump_t<<<div_up(h->n_dual, 256), 256, 0, h->stream>>>(h->n_dual, h->dual_entry.p, h->dual_l1.p,
-                                                          h->dual_l2.p, nullptr, x, 1.0, t1));
-  LAT_CHECK_LAUNCH();
-  kinv(h, t1, w, KINV_DUAL_IN);
+  if (tc) {
+    kinv(h, nullptr, w, KINV_DUAL_IN, x);
+  } else {
+    LAT_CUDA(cudaMemsetAsync(t1, 0, (nloc + h->n_primal) * sizeof(double), h->stream));
+    LAT_LAUNCH(h, k_jump_t<<<div_up(h->n_dual, 256), 256, 0, h->stream>>>(h->n_dual, h->dual_entry.p, h->dual_l1.p,
+                                                                          h->dual_l2.p, x, 1.0, t1));
+    LAT_CHECK_LAUNCH();
+    kinv(h, t1, w, KINV_DUAL_IN);
+  }
   LAT_LAUNCH(h, k_axpby<<<ew_blocks(h, nloc + h->n_primal), 256, 0, h->stream>>>(nloc + h->n_primal, 1.0, t, 1.0, w));
   LAT_LAUNCH(h, k_axpby<<<ew_blocks(h, L), 256, 0, h->stream>>>(L, -1.0, x, 0.0, la_of(h, w)));
   LAT_CHECK_LAUNCH();

@@ -420,6 +420,9 @@ void build_feti_impl(lat_ctx* h, int level) {
   h->n_lambda = (int64_t)lp.size();
   h->lam_p.upload(lp, h->stream);
   h->lam_m.upload(lm, h->stream);
+  std::vector<double> lsc_l(pairs.size());
+  for (size_t l = 0; l < pairs.size(); ++l) lsc_l[l] = 1.0 / mult[pairs[l].first];
+  h->lam_scale.upload(lsc_l, h->stream);
   std::vector<int> de, d1, d2;
   std::vector<double> dsc;
   for (auto& kv : dual) {
@@ -647,7 +650,7 @@ extern "C" lat_status lattice_destroy(lat_handle h) {
   rel(h->copy_ptr); rel(h->copy_idx); rel(h->dof_fixed); rel(h->dir_unit); rel(h->aff_unit);
   rel(h->corner_of_node); rel(h->rdofs); rel(h->pdofs); rel(h->rpos); rel(h->pidx);
   rel(h->p_copy_ptr); rel(h->p_copy); rel(h->loc_fixed); rel(h->lam_p); rel(h->lam_m);
-  rel(h->dual_entry); rel(h->dual_l1); rel(h->dual_l2); rel(h->dual_scale); rel(h->dual_lk); rel(h->dual_lsc); rel(h->cell_class);
+  rel(h->dual_entry); rel(h->dual_l1); rel(h->dual_l2); rel(h->dual_scale); rel(h->lam_scale); rel(h->dual_lk); rel(h->dual_lsc); rel(h->cell_class);
   rel(h->coarse_ptr); rel(h->coarse_src); rel(h->cb_dest); rel(h->cb_perm); rel(h->cb_A);
   rel(h->cb_Dinv); rel(h->cb_Einv); rel(h->cb_U); rel(h->cb_V); rel(h->cb_T); rel(h->cb_X); rel(h->cb_Ut); rel(h->cb_y); rel(h->cb_w); rel(h->coarse_row); rel(h->coarse_col);
   rel(h->S); rel(h->alpha); rel(h->alpha32); rel(h->Kp); rel(h->Kp32); rel(h->Kg);
