@@ -175,9 +175,8 @@ struct lat_ctx {
   int64_t sel_version = 0, kg_version = -1;   // principal-set changes / the group-order copy's
   int kg_gr = 0;
   // greedy workspaces
-  DBuf<double> g_delta, g_Z, g_beta, g_inf, g_nrm2, g_norms, g_part, g_maxres;
-  DBuf<int> g_state;                  // [0] done, [1] n_r, [2] s_next
-  DBuf<double> g_scale;
+  DBuf<double> g_delta, g_Z, g_beta, g_inf, g_norms, g_part, g_maxres;
+  DBuf<int> g_state;                  // [0] done, [1] n_r, [2] s_next, [3] blocks done
   // assembly workspaces
   DBuf<double> f_cells, r_glob, minJ_cell, T;
   DBuf<int> negJ;

@@ -3,11 +3,18 @@
 //
 // The snapshot matrix is stored column-major, one cell per contiguous column (T^s = data of the
 // reduced-rule tangent of cell s, Eq. snapshots).  Per greedy iteration i:
-//   select : one CTA reduces (max ||Delta^s||_inf, argmax) over the columns (ties -> lowest s),
-//            records it and decides termination (device flag, no host round trip);
+//   select : argmax of ||Delta^s||_inf over the columns (ties -> lowest s), recorded, and the decision
+//            to end (device flag, no host round trip), by the block of the pass before that ends last;
+//   norm   : partial sums of ||Delta^{s_i}||_2^2, the selected column's alone;
 //   zeta   : zeta_i = Delta^{s_i} / ||Delta^{s_i}||_2 copied into Z (grid over rows);
 //   update : one CTA per column: beta_i^s = Delta^s . zeta_i, Delta^s -= beta_i^s zeta_i, and the
-//            new ||Delta^s||_inf, ||Delta^s||_2 of the column (one read + one write of Delta).
+//            new ||Delta^s||_inf of the column.
+// The update is bound by the FP64 pipe (two lanes per clock per SM) as much as by memory, so an
+// entry costs two multiply-adds and nothing else there: the maximum is taken on the bits of |v| by
+// integer compares, and the norm is left to the one column that needs it.  1024 ring columns of 9880
+// rows: 67 us (and no launch of 10 us to select) against 75 us with an FP64 maximum and a norm per column.  (Keeping the column
+// in shared memory between the dot product and the update, two CTAs per SM, took 99 us: the second
+// read costs less than the warps that room takes.)
 // Every kernel returns at once when the device flag says the loop has ended, so the host can
 // launch iterations in chunks and look at the flag once per chunk.
 #include <algorithm>
@@ -19,44 +26,53 @@ namespace {
 
 constexpr int kColThreads = 256;
 
-__global__ void __launch_bounds__(kColThreads)
-    k_g_init(int64_t n_rows, const double* __restrict__ T, double* __restrict__ Delta,
-             double* __restrict__ norms, double* __restrict__ inf, double* __restrict__ nrm2) {
-  __shared__ double red[32];
-  const int s = blockIdx.x;
-  const double* t = T + (size_t)s * n_rows;
-  double* dl = Delta + (size_t)s * n_rows;
-  double ss = 0;
-  for (int64_t r = threadIdx.x; r < n_rows; r += blockDim.x) ss += t[r] * t[r];
-  const double nrm = sqrt(block_sum(ss, red));
-  const double inv = nrm > 0 ? 1.0 / nrm : 0.0;
-  double mx = 0, s2 = 0;
-  for (int64_t r = threadIdx.x; r < n_rows; r += blockDim.x) {
-    double v = t[r] * inv;
-    dl[r] = v;
-    mx = fmax(mx, fabs(v));
-    s2 += v * v;
-  }
-  mx = block_max(mx, red);
-  s2 = block_sum(s2, red);
-  if (threadIdx.x == 0) {
-    norms[s] = nrm;
-    inf[s] = mx;
-    nrm2[s] = s2;
-  }
+constexpr int kNormBlocks = 32;
+
+// |v| as ordered bits, NaN as 0 (a NaN entry does not count for the maximum)
+__device__ __forceinline__ unsigned long long mag_bits(double v) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(v) & 0x7fffffffffffffffull;
+  return b > 0x7ff0000000000000ull ? 0ull : b;
 }
 
-// state[0] = done, state[1] = n_r, state[2] = selected column of this iteration
-__global__ void k_g_select(int it, int n_cols, int limit, double eps, const double* __restrict__ inf,
-                           const double* __restrict__ nrm2, int* __restrict__ state,
-                           int* __restrict__ S, double* __restrict__ maxres, double* __restrict__ scale) {
-  if (state[0]) return;
+__device__ __forceinline__ unsigned long long block_max_bits(unsigned long long v, unsigned long long* sh) {
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v = max(v, __shfl_xor_sync(0xffffffffu, v, o));
+  __syncthreads();
+  if (lane == 0) sh[wid] = v;
+  __syncthreads();
+  v = sh[lane < nw ? lane : 0];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v = max(v, __shfl_xor_sync(0xffffffffu, v, o));
+  return v;
+}
+
+struct SelectArgs {
+  int it, n_cols, limit;
+  double eps;
+  double* inf;        // [n_cols] largest magnitude of every column
+  int* state;         // [0] = done, [1] = n_r, [2] = selected column of this iteration, [3] = ticket
+  int* S;
+  double* maxres;
+};
+
+// the block that ends last selects iteration A.it's column
+__device__ void select_last(const SelectArgs& A) {
+  __shared__ bool last;
   __shared__ double bv[32];
   __shared__ int bi[32];
+  if (threadIdx.x == 0) {
+    __threadfence();
+    last = atomicAdd(A.state + 3, 1) == (int)gridDim.x - 1;
+  }
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
   double best = -1.0;
   int bidx = 0x7fffffff;
-  for (int s = threadIdx.x; s < n_cols; s += blockDim.x) {
-    double v = inf[s];
+#pragma unroll 4
+  for (int s = threadIdx.x; s < A.n_cols; s += blockDim.x) {
+    const double v = __ldcg(A.inf + s);
     if (v > best || (v == best && s < bidx)) {
       best = v;
       bidx = s;
@@ -64,8 +80,8 @@ __global__ void k_g_select(int it, int n_cols, int limit, double eps, const doub
   }
   // warp then block argmax, ties to the lowest index
   for (int o = 16; o > 0; o >>= 1) {
-    double ov = __shfl_xor_sync(0xffffffffu, best, o);
-    int oi = __shfl_xor_sync(0xffffffffu, bidx, o);
+    const double ov = __shfl_xor_sync(0xffffffffu, best, o);
+    const int oi = __shfl_xor_sync(0xffffffffu, bidx, o);
     if (ov > best || (ov == best && oi < bidx)) {
       best = ov;
       bidx = oi;
@@ -77,62 +93,126 @@ __global__ void k_g_select(int it, int n_cols, int limit, double eps, const doub
     bi[wid] = bidx;
   }
   __syncthreads();
-  if (threadIdx.x == 0) {
-    for (int w = 1; w < (int)(blockDim.x >> 5); ++w)
-      if (bv[w] > best || (bv[w] == best && bi[w] < bidx)) {
-        best = bv[w];
-        bidx = bi[w];
-      }
-    maxres[it] = best;
-    if (!(best > eps) || it >= limit) {
-      state[0] = 1;
-      state[1] = it;
-    } else {
-      S[it] = bidx;
-      state[1] = it + 1;
-      state[2] = bidx;
-      scale[0] = 1.0 / sqrt(nrm2[bidx]);
+  if (threadIdx.x != 0) return;
+  for (int w = 1; w < (int)(blockDim.x >> 5); ++w)
+    if (bv[w] > best || (bv[w] == best && bi[w] < bidx)) {
+      best = bv[w];
+      bidx = bi[w];
     }
+  A.state[3] = 0;
+  A.maxres[A.it] = best;
+  if (!(best > A.eps) || A.it >= A.limit) {
+    A.state[0] = 1;
+    A.state[1] = A.it;
+  } else {
+    A.S[A.it] = bidx;
+    A.state[1] = A.it + 1;
+    A.state[2] = bidx;
   }
 }
 
+// normalised columns, their norms and largest magnitudes; then the first selection
+__global__ void __launch_bounds__(kColThreads)
+    k_g_init(int64_t n_rows, const double* __restrict__ T, double* __restrict__ Delta,
+             double* __restrict__ norms, SelectArgs A) {
+  __shared__ double red[32];
+  __shared__ unsigned long long redm[32];
+  const int s = blockIdx.x;
+  const double* t = T + (size_t)s * n_rows;
+  double* dl = Delta + (size_t)s * n_rows;
+  double ss = 0;
+#pragma unroll 4
+  for (int64_t r = threadIdx.x; r < n_rows; r += kColThreads) {
+    const double v = t[r];
+    ss += v * v;
+  }
+  const double nrm = sqrt(block_sum(ss, red));
+  const double inv = nrm > 0 ? 1.0 / nrm : 0.0;
+  unsigned long long mx = 0;
+#pragma unroll 4
+  for (int64_t r = threadIdx.x; r < n_rows; r += kColThreads) {
+    const double v = t[r] * inv;
+    dl[r] = v;
+    mx = max(mx, mag_bits(v));
+  }
+  mx = block_max_bits(mx, redm);
+  if (threadIdx.x == 0) {
+    norms[s] = nrm;
+    A.inf[s] = __longlong_as_double((long long)mx);
+  }
+  select_last(A);
+}
+
+// partial sums of the selected column's squares
+__global__ void __launch_bounds__(256)
+    k_g_norm(int64_t n_rows, const double* __restrict__ Delta, const int* __restrict__ state,
+             double* __restrict__ part) {
+  if (state[0]) return;
+  __shared__ double red[32];
+  const double* dl = Delta + (size_t)state[2] * n_rows;
+  double v = 0;
+#pragma unroll 4
+  for (int64_t r = blockIdx.x * (int64_t)256 + threadIdx.x; r < n_rows; r += (int64_t)kNormBlocks * 256)
+    v += dl[r] * dl[r];
+  v = block_sum(v, red);
+  if (threadIdx.x == 0) part[blockIdx.x] = v;
+}
+
 __global__ void k_g_zeta(int it, int64_t n_rows, const double* __restrict__ Delta,
-                         const int* __restrict__ state, const double* __restrict__ scale,
+                         const int* __restrict__ state, const double* __restrict__ part,
                          double* __restrict__ Z) {
   if (state[0]) return;
   const int s = state[2];
-  const double sc = scale[0];
+  const double sc = 1.0 / sqrt(warp_sum(part[threadIdx.x & 31]));   // kNormBlocks = 32 partial sums
   double* z = Z + (size_t)it * n_rows;
   const double* dl = Delta + (size_t)s * n_rows;
   for (int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; r < n_rows; r += (int64_t)gridDim.x * blockDim.x)
     z[r] = dl[r] * sc;
 }
 
+// iteration `it`'s projection, then the selection of the next (A.it = it + 1)
 __global__ void __launch_bounds__(kColThreads)
-    k_g_update(int it, int64_t n_rows, int n_cols, double* __restrict__ Delta,
-               const double* __restrict__ Z, const int* __restrict__ state, double* __restrict__ beta,
-               double* __restrict__ inf, double* __restrict__ nrm2) {
-  if (state[0]) return;
+    k_g_update(int it, int64_t n_rows, double* __restrict__ Delta, const double* __restrict__ Z,
+               double* __restrict__ beta, SelectArgs A) {
+  if (A.state[0]) return;
   __shared__ double red[32];
+  __shared__ unsigned long long redm[32];
   const int s = blockIdx.x;
   double* dl = Delta + (size_t)s * n_rows;
   const double* z = Z + (size_t)it * n_rows;
   double b = 0;
-  for (int64_t r = threadIdx.x; r < n_rows; r += blockDim.x) b += dl[r] * z[r];
-  b = block_sum(b, red);
-  double mx = 0, s2 = 0;
-  for (int64_t r = threadIdx.x; r < n_rows; r += blockDim.x) {
-    double v = dl[r] - b * z[r];
-    dl[r] = v;
-    mx = fmax(mx, fabs(v));
-    s2 += v * v;
+#pragma unroll 4
+  for (int64_t r = threadIdx.x; r < n_rows; r += kColThreads) {
+    b += dl[r] * z[r];
   }
-  mx = block_max(mx, red);
-  s2 = block_sum(s2, red);
+  b = block_sum(b, red);
+  unsigned long long mx = 0;
+#pragma unroll 4
+  for (int64_t r = threadIdx.x; r < n_rows; r += kColThreads) {
+    const double v = dl[r] - b * z[r];
+    dl[r] = v;
+    mx = max(mx, mag_bits(v));
+  }
+  mx = block_max_bits(mx, redm);
   if (threadIdx.x == 0) {
-    beta[(size_t)it * n_cols + s] = b;
-    inf[s] = mx;
-    nrm2[s] = s2;
+    beta[(size_t)it * A.n_cols + s] = b;
+    A.inf[s] = __longlong_as_double((long long)mx);
+  }
+  select_last(A);
+}
+
+// Algorithm 1 on the workspaces given: the launches of one chunk of iterations [it0, it1).  The
+// selection of iteration it runs at the end of the pass before (init for it = 0), so the update of
+// the last iteration a chunk can reach also decides the end.
+void launch_greedy(cudaStream_t st, int n_sm, int it0, int it1, int64_t n_rows, int n_cols, double* delta, double* Z,
+                   double* part, double* beta, const SelectArgs& base) {
+  const int zgrid = std::min(div_up(n_rows, 256), 4 * n_sm);
+  for (int it = it0; it < it1; ++it) {
+    k_g_norm<<<kNormBlocks, 256, 0, st>>>(n_rows, delta, base.state, part);
+    k_g_zeta<<<zgrid, 256, 0, st>>>(it, n_rows, delta, base.state, part, Z);
+    SelectArgs A = base;
+    A.it = it + 1;
+    k_g_update<<<n_cols, kColThreads, 0, st>>>(it, n_rows, delta, Z, beta, A);
   }
 }
 
@@ -180,27 +260,23 @@ void run_greedy(lat_ctx* h, const double* T, int64_t n_rows, int n_cols, double 
   h->g_Z.ensure((size_t)limit * n_rows);
   h->g_beta.ensure((size_t)limit * n_cols);
   h->g_inf.ensure(n_cols);
-  h->g_nrm2.ensure(n_cols);
   h->g_norms.ensure(n_cols);
+  h->g_part.ensure(kNormBlocks);
   h->g_maxres.ensure(limit + 1);
   h->g_state.ensure(4);
-  h->g_scale.ensure(2);
   h->S.ensure(std::max(limit, h->n_cells));
   LAT_CUDA(cudaMemsetAsync(h->g_state.p, 0, 4 * sizeof(int), h->stream));
-  LAT_LAUNCH(h, k_g_init<<<n_cols, kColThreads, 0, h->stream>>>(n_rows, T, h->g_delta.p, h->g_norms.p, h->g_inf.p,
-                                                  h->g_nrm2.p));
+  const SelectArgs base{0, n_cols, limit, eps, h->g_inf.p, h->g_state.p, h->S.p, h->g_maxres.p};
+  LAT_LAUNCH(h, k_g_init<<<n_cols, kColThreads, 0, h->stream>>>(n_rows, T, h->g_delta.p, h->g_norms.p, base));
   LAT_CHECK_LAUNCH();
-  const int zgrid = std::min(div_up(n_rows, 256), 4 * h->n_sm);
   int* hp = reinterpret_cast<int*>(h->h_pinned);
   const int chunk = 8;
-  for (int it0 = 0; it0 <= limit; it0 += chunk) {
-    for (int it = it0; it < std::min(it0 + chunk, limit + 1); ++it) {
-      LAT_LAUNCH(h, k_g_select<<<1, 1024, 0, h->stream>>>(it, n_cols, limit, eps, h->g_inf.p, h->g_nrm2.p,
-                                            h->g_state.p, h->S.p, h->g_maxres.p, h->g_scale.p));
-      LAT_LAUNCH(h, k_g_zeta<<<zgrid, 256, 0, h->stream>>>(it, n_rows, h->g_delta.p, h->g_state.p, h->g_scale.p, h->g_Z.p));
+  for (int it0 = 0; it0 < limit; it0 += chunk) {
+    const int it1 = std::min(it0 + chunk, limit);
+    {
       KernelTimer kt(h, "greedy_update");
-      LAT_LAUNCH(h, k_g_update<<<n_cols, kColThreads, 0, h->stream>>>(it, n_rows, n_cols, h->g_delta.p, h->g_Z.p,
-                                                        h->g_state.p, h->g_beta.p, h->g_inf.p, h->g_nrm2.p));
+      launch_greedy(h->stream, h->n_sm, it0, it1, n_rows, n_cols, h->g_delta.p, h->g_Z.p, h->g_part.p, h->g_beta.p, base);
+      h->n_launch += 3 * (it1 - it0);
     }
     LAT_CHECK_LAUNCH();
     LAT_CUDA(cudaMemcpyAsync(hp, h->g_state.p, 2 * sizeof(int), cudaMemcpyDeviceToHost, h->stream));
@@ -370,7 +446,7 @@ __device__ __align__(256) double g_static_greedy[kStaticGreedyDoubles];
 double* g_static_ptr[kStaticMaxDevices] = {nullptr};
 
 struct StaticLayout {
-  double *delta, *Z, *beta, *norms, *inf, *nrm2, *maxres, *scale;
+  double *delta, *Z, *beta, *norms, *inf, *part, *maxres;
   int* state;
   int* S;
   size_t doubles;
@@ -389,9 +465,8 @@ StaticLayout static_layout(double* base, int64_t n_rows, int n_cols, int limit) 
   L.beta = take((size_t)limit * n_cols);
   L.norms = take(n_cols);
   L.inf = take(n_cols);
-  L.nrm2 = take(n_cols);
   L.maxres = take(limit + 1);
-  L.scale = take(2);
+  L.part = take(kNormBlocks);
   L.state = reinterpret_cast<int*>(take(2));          // 4 ints
   L.S = reinterpret_cast<int*>(take((limit + 1) / 2 + 1));
   L.doubles = off;
@@ -420,16 +495,12 @@ extern "C" lat_status greedy_select_static(const double* T, int64_t n_rows, int3
   int n_sm = 0;
   if (cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return LAT_ECUDA;
   if (cudaMemsetAsync(W.state, 0, 4 * sizeof(int), st) != cudaSuccess) return LAT_ECUDA;
-  k_g_init<<<n_cols, kColThreads, 0, st>>>(n_rows, T, W.delta, W.norms, W.inf, W.nrm2);
-  const int zgrid = std::min(div_up(n_rows, 256), 4 * n_sm);
+  const SelectArgs base{0, n_cols, limit, eps, W.inf, W.state, W.S, W.maxres};
+  k_g_init<<<n_cols, kColThreads, 0, st>>>(n_rows, T, W.delta, W.norms, base);
   int hstate[2] = {0, 0};
   const int chunk = 8;
-  for (int it0 = 0; it0 <= limit; it0 += chunk) {
-    for (int it = it0; it < std::min(it0 + chunk, limit + 1); ++it) {
-      k_g_select<<<1, 1024, 0, st>>>(it, n_cols, limit, eps, W.inf, W.nrm2, W.state, W.S, W.maxres, W.scale);
-      k_g_zeta<<<zgrid, 256, 0, st>>>(it, n_rows, W.delta, W.state, W.scale, W.Z);
-      k_g_update<<<n_cols, kColThreads, 0, st>>>(it, n_rows, n_cols, W.delta, W.Z, W.state, W.beta, W.inf, W.nrm2);
-    }
+  for (int it0 = 0; it0 < limit; it0 += chunk) {
+    launch_greedy(st, n_sm, it0, std::min(it0 + chunk, limit), n_rows, n_cols, W.delta, W.Z, W.part, W.beta, base);
     if (cudaGetLastError() != cudaSuccess) return LAT_ECUDA;
     if (cudaMemcpyAsync(hstate, W.state, 2 * sizeof(int), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
         cudaStreamSynchronize(st) != cudaSuccess)

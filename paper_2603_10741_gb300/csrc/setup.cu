@@ -655,8 +655,8 @@ extern "C" lat_status lattice_destroy(lat_handle h) {
   rel(h->cb_Dinv); rel(h->cb_Einv); rel(h->cb_U); rel(h->cb_V); rel(h->cb_T); rel(h->cb_X); rel(h->cb_Ut); rel(h->cb_y); rel(h->cb_w); rel(h->coarse_row); rel(h->coarse_col);
   rel(h->S); rel(h->alpha); rel(h->alpha32); rel(h->Kp); rel(h->Kp32); rel(h->Kg);
   for (auto& g : h->ng) { rel(g.rows); rel(g.ucptr); rel(g.ucol); rel(g.pp); rel(g.pair_u); rel(g.perm); }
-  rel(h->g_delta); rel(h->g_Z); rel(h->g_beta); rel(h->g_inf); rel(h->g_nrm2); rel(h->g_norms);
-  rel(h->g_part); rel(h->g_maxres); rel(h->g_state); rel(h->g_scale);
+  rel(h->g_delta); rel(h->g_Z); rel(h->g_beta); rel(h->g_inf); rel(h->g_norms);
+  rel(h->g_part); rel(h->g_maxres); rel(h->g_state);
   rel(h->f_cells); rel(h->r_glob); rel(h->minJ_cell); rel(h->T); rel(h->negJ);
   rel(h->key_of_cell); rel(h->key_slot); rel(h->perm); rel(h->seg_ptr); rel(h->tile_seg);
   rel(h->tile_c0); rel(h->key_list); rel(h->solver_int); rel(h->delta_cell); rel(h->c_cell);
