@@ -129,8 +129,8 @@ __global__ void __launch_bounds__(256)
   store_ya<T, D, FETI>(A, Y, s, a, y);
 }
 
-// Shared-memory staged form.  A CTA is 8 warps; warp w owns local node a = 8 blockIdx.y + w and
-// its lanes own CPT x 32 consecutive cells (the same cells for all 8 warps).  Per chunk of RCH
+// Shared-memory staged form.  A CTA is W warps; warp w owns local node a = W blockIdx.y + w and
+// its lanes own CPT x 32 consecutive cells (the same cells for all W warps).  Per chunk of RCH
 // principals the CTA stages the alpha values of its cells once, and each warp its node's
 // principal blocks K^r_{a,:} into its own slice of shared memory; the warp keeps the neighbour
 // values x_b of its cells in registers and for every principal forms z = K^r_{a,:} x
@@ -141,6 +141,12 @@ struct StageCfg {
   static constexpr int MAXNB = D == 2 ? 9 : 27;  // node blocks per row of a Q1 pattern
   static constexpr int CPT = D == 2 ? 2 : 1;     // cells per thread
 };
+
+// Warps per CTA: 8; in FP64 3D 4, so that two CTAs share an SM (203 registers a thread) and one
+// stages while the other multiplies.  Small lattices take 2 warps of one cell per lane: the FP64 pipe
+// of an SM issues a warp's multiply-add in 16 clocks, so 16 ring cells on 10 CTAs of 8 warps, half
+// their lanes without a cell, took 39 us where 40 CTAs take 18 us.  567 strut cells, four
+// principals: 698 us with 8 warps, 621 us with 4.
 
 template <typename T, int D>
 __host__ __device__ constexpr int stage_rch() {
@@ -154,16 +160,16 @@ __host__ __device__ constexpr int stage_min_blocks() {
   return D == 2 && sizeof(T) == 4 && !FETI ? 4 : 1;
 }
 
-template <typename T, int D, bool FETI>
-__global__ void __launch_bounds__(256, stage_min_blocks<T, D, FETI>())
+template <typename T, int D, bool FETI, int W, int CPT>
+__global__ void __launch_bounds__(32 * W, stage_min_blocks<T, D, FETI>())
     k_apply_staged(ApplyArgs A, int n_r, const T* __restrict__ Kp, const T* __restrict__ alpha,
                    const T* __restrict__ X, T* __restrict__ Y) {
-  constexpr int MAXNB = StageCfg<D>::MAXNB, CPT = StageCfg<D>::CPT, RCH = stage_rch<T, D>();
+  constexpr int MAXNB = StageCfg<D>::MAXNB, RCH = stage_rch<T, D>();
   constexpr int DD = D * D;
-  constexpr int NC = 32 * CPT;                   // cells of the CTA (the same for its 8 warps)
+  constexpr int NC = 32 * CPT;                   // cells of the CTA (the same for its warps)
   extern __shared__ __align__(16) unsigned char sm_raw[];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int a = blockIdx.y * 8 + warp;
+  const int a = blockIdx.y * W + warp;
   const bool active = a < A.nn;                  // idle warps still join the CTA barriers
   T* als = reinterpret_cast<T*>(sm_raw);                                  // alpha chunk [RCH][NC]
   T* ks = als + RCH * NC + (size_t)warp * MAXNB * RCH * DD;              // this warp's K blocks
@@ -474,11 +480,18 @@ void launch(lat_ctx* h, const ApplyArgs& A, const T* Kp, const T* alpha, const T
       dim3 grid(div_up(h->n_cells, 32), div_up(h->n_nodes_cell, 8));
       LAT_LAUNCH(h, k_apply_reduced<T, D, FETI><<<grid, blk, 0, h->stream>>>(A, h->n_r, Kp, alpha, X, Y));
     } else {
-      constexpr int MAXNB = StageCfg<D>::MAXNB, CPT = StageCfg<D>::CPT, RCH = stage_rch<T, D>();
-      const size_t shm = ((size_t)RCH * 32 * CPT + (size_t)8 * MAXNB * RCH * D * D) * sizeof(T);
-      LAT_CUDA(cudaFuncSetAttribute(k_apply_staged<T, D, FETI>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm));
-      dim3 grid(div_up(h->n_cells, 32 * CPT), div_up(h->n_nodes_cell, 8));
-      LAT_LAUNCH(h, k_apply_staged<T, D, FETI><<<grid, 256, shm, h->stream>>>(A, h->n_r, Kp, alpha, X, Y));
+      auto go = [&](auto kern, int W, int CPT) {
+        const size_t shm = ((size_t)stage_rch<T, D>() * 32 * CPT + (size_t)W * StageCfg<D>::MAXNB * stage_rch<T, D>() * D * D) * sizeof(T);
+        LAT_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm));
+        const dim3 grid(div_up(h->n_cells, 32 * CPT), div_up(h->n_nodes_cell, W));
+        LAT_LAUNCH(h, kern<<<grid, 32 * W, shm, h->stream>>>(A, h->n_r, Kp, alpha, X, Y));
+      };
+      constexpr int W = D == 3 && sizeof(T) == 8 ? 4 : 8, CPT = StageCfg<D>::CPT;
+      // fewer CTAs than SMs: smaller ones
+      if ((int64_t)div_up(h->n_cells, 32 * CPT) * div_up(h->n_nodes_cell, W) < h->n_sm)
+        go(k_apply_staged<T, D, FETI, 2, 1>, 2, 1);
+      else
+        go(k_apply_staged<T, D, FETI, W, CPT>, W, CPT);
     }
   }
   LAT_CHECK_LAUNCH();

@@ -174,3 +174,45 @@ def test_fp64_digit_products(L, dims):
     Kv[s.n_cells * (s.n_loc // 2) + 1] = float("nan")
     assert torch.isnan(lat.feti_apply(1, Kv)[:nd]).any()
     lat.close()
+
+
+@pytest.mark.parametrize("cell,dims,n_r", [
+    (latgen.ring_cell(8), (4, 4), 17),           # small CTAs, two chunks of principals
+    (latgen.ring_cell(8), (25, 39), 2),          # 975 cells: 16 tiles of 64 x 10 CTAs of 8 nodes, one more than the SMs
+    (latgen.strut_cell(6, 0.2), (1, 2, 1), 5),   # small CTAs in 3D, two chunks
+    (latgen.strut_cell(12, 0.15), (3, 3, 4), 1), # 36 cells: CTAs of 4 warps, last tile of 4 cells
+])
+def test_fp64_action_by_cta_form(L, cell, dims, n_r):
+    """FP64 reduced action against the oracle (1e-10 as in test_gpu_kernels.py)."""
+    from oracle import rom as OR
+    case = _case(cell, dims)
+    prob = Problem(case)
+    n = prob.lat.n_cells
+    n_r = min(n_r, n)
+    u = latgen.smooth_state(case.lattice, 0.01, 21).ravel()
+    S = np.arange(n_r, dtype=np.int32)
+    al = latgen.dirichlet_coefficients(n_r, n, 8)
+    X = latgen.uniform_field((prob.cell.n_nodes * prob.cell.d, n), 22)
+    ref = OR.reduced_apply(prob.cell, OC.tangent(prob.cell, prob.local(u)[S], prob.mu_cells[S], prob.lam), al, X)
+    lat = L.Lattice.from_case(case)
+    lat.set_principal_cells(torch.tensor(u, device="cuda"), torch.tensor(S), torch.tensor(al))
+    assert _rel(lat.apply_reduced_tangent(torch.tensor(X, device="cuda")).cpu(), ref) < 1e-10
+    lat.close()
+
+
+@pytest.mark.parametrize("n_rows,n_cols,max_nr", [(1, 1, 1), (31, 3, 8), (257, 40, 9), (4096, 5, 5)])
+def test_greedy_by_size(L, n_rows, n_cols, max_nr):
+    """Algorithm 1 against the oracle's at sizes off the blocks' multiples: identical selections, alpha
+    to 1e-9 (test_gpu_kernels.py); with the cap, and through the allocation-free entry point too."""
+    from oracle import greedy as OG
+    T = np.random.default_rng(n_rows).normal(size=(n_rows, n_cols))
+    g = OG.greedy(T, 1e-6, max_nr)
+    a_ref = OG.alpha_triangular(T, g)
+    lat = L.Lattice.from_case(latgen.make_case("ring2"))
+    Td = torch.tensor(T.T.copy(), device="cuda")
+    out = lat.greedy_select(Td, 1e-6, max_nr)
+    S, al = L.greedy_select_static(Td, 1e-6, max_nr)
+    for s_got, a_got in ((out["S"], out["alpha"]), (S, al)):
+        assert s_got.cpu().numpy().tolist() == g.S.tolist()
+        assert np.abs(a_got.cpu().numpy() - a_ref).max() <= 1e-9 * max(1.0, np.abs(a_ref).max())
+    lat.close()
