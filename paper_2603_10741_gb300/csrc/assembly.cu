@@ -36,6 +36,7 @@ struct GeomArgs {
   const int* elems;      // [n_el][nen]
   const int* color_elems;
   int nq;
+  const double* gram;    // [n_el][pairs a <= b, a-major] sum_q W g_a.g_b
 };
 
 __device__ __forceinline__ void load_cell_u(const double* __restrict__ u_glob,
@@ -228,23 +229,24 @@ __global__ void __launch_bounds__(kCellThreads)
 // ---------------------------------------------------------------------------------------------
 // tangent: K^s on the shared pattern for a list of cells, [n_sel][nnz].  Per batch of a colour's
 // elements (EB at most), a thread per quadrature point leaves h_a = F^{-T} grad phi_a of all its
-// nodes and the three weights in shared memory; then a thread per (element, node pair a <= b) sums
-// its block over the points and writes K_ab and K_ba = K_ab^T.  The first element to touch a block
+// nodes in shared memory, once as it is and once times each of its two weights; then a thread per
+// (element, node pair a <= b) sums its block over the points and writes K_ab and K_ba = K_ab^T.  The
+// mu term's sum_q W g_a.g_b does not depend on the state: one table entry per pair (gram).  The first element to touch a block
 // (in colour order; kFirst in elem_blk) stores it, later ones add, so K is not cleared first.  A
 // cell is worked on by a cluster of CL CTAs that share each colour's batches and meet at a cluster
 // barrier between colours: with few cells (the principals) one CTA each would leave the GPU idle
 // (3 strut cells took 3.4 ms).
 //
-// Bound by the FP64 pipe (24 operations per pair and point in 3D, 8.5k per element against 29k
-// when a thread per element row repeated the kinematics).  1024 ring cells: 0.51 ms, before 1.35;
-// one strut principal: 0.3 ms, before 3.4.
+// Bound by the FP64 pipe (18 operations per pair and point in 3D, 8 in 2D).  1024 ring cells: 0.45 ms,
+// 0.51 with the weights and g_a.g_b applied per pair and point, 1.35 when a thread per element row
+// also repeated the kinematics; one strut principal: 0.3 ms, before 3.4.
 // ---------------------------------------------------------------------------------------------
 constexpr int kFirst = 1 << 30;
 
-// smem of one element of a batch: h [nq][NEN * D + 1] (padded: a thread's row, conflict-free
-// stores), weights [nq][3]
+// smem of one element of a batch: [nq] rows of h, lam w h, (mu - lam ln J) w h (an odd length: a
+// thread's row, conflict-free stores)
 template <int D>
-__host__ __device__ constexpr int tangent_el_doubles(int nq) { return nq * ((1 << D) * D + 1 + 3); }
+__host__ __device__ constexpr int tangent_row() { return 3 * (1 << D) * D + 1; }
 
 template <int D>
 __global__ void __launch_bounds__(kCellThreads)
@@ -253,12 +255,11 @@ __global__ void __launch_bounds__(kCellThreads)
               const double* __restrict__ mu_cell, double lam, const double* __restrict__ u_glob,
               int64_t nnz, double* __restrict__ K_out, double* __restrict__ minJ_out, int geo, int EB, int CL,
               int staged) {
-  constexpr int NEN = 1 << D, NP = NEN * (NEN + 1) / 2, HS = NEN * D + 1;
+  constexpr int NEN = 1 << D, NP = NEN * (NEN + 1) / 2, ND = NEN * D, HS = tangent_row<D>();
   extern __shared__ double sm[];
   const int nq = g.nq;
   double* hs = sm;                          // [EB][nq][HS]
-  double* ws = hs + (size_t)EB * nq * HS;   // [EB][nq][3]
-  double* u_loc = ws + (size_t)EB * nq * 3; // [nn * D] when staged
+  double* u_loc = hs + (size_t)EB * nq * HS; // [nn * D] when staged
   __shared__ double red[32];
   __shared__ unsigned char pa[NP], pb[NP];
   const int si = blockIdx.x / CL, rank = blockIdx.x % CL;
@@ -300,10 +301,7 @@ __global__ void __launch_bounds__(kCellThreads)
         minJ = fmin(minJ, J);
         const double lnJ = J > 0 ? log(J) : 0.0;
         const double w = g.W[e * nq + q];
-        double* wt = ws + (size_t)t * 3;
-        wt[0] = w * mu;
-        wt[1] = w * lam;
-        wt[2] = w * (mu - lam * lnJ);
+        const double cl = w * lam, cg = w * (mu - lam * lnJ);
         double* ht = hs + (size_t)t * HS;
 #pragma unroll
         for (int a = 0; a < NEN; ++a)
@@ -313,6 +311,8 @@ __global__ void __launch_bounds__(kCellThreads)
 #pragma unroll
             for (int k = 0; k < D; ++k) v = fma(Fi[k][i], gq[a * D + k], v);
             ht[a * D + i] = v;
+            ht[ND + a * D + i] = cl * v;
+            ht[2 * ND + a * D + i] = cg * v;
           }
       }
       __syncthreads();
@@ -325,39 +325,30 @@ __global__ void __launch_bounds__(kCellThreads)
         for (int i = 0; i < D; ++i)
 #pragma unroll
           for (int j = 0; j < D; ++j) acc[i][j] = 0.0;
+        double dg = 0.0;
         for (int q = 0; q < nq; ++q) {
           const double* ht = hs + (size_t)(el * nq + q) * HS;
-          const double* wt = ws + (size_t)(el * nq + q) * 3;
-          const double cl = wt[1], cg = wt[2];
-          double ha[D], hb[D], la[D], ga[D];
+          double la[D], ga[D], hb[D];
 #pragma unroll
           for (int i = 0; i < D; ++i) {
-            ha[i] = ht[a * D + i];
+            la[i] = ht[ND + a * D + i];
+            ga[i] = ht[2 * ND + a * D + i];
             hb[i] = ht[b * D + i];
-            la[i] = cl * ha[i];
-            ga[i] = cg * ha[i];
-          }
-          // diagonal term: mu g_a.g_b holds the geometric part delta_ij J h_a^T sigma h_b =
-          // mu (g_a.g_b - h_a.h_b) + lam ln J h_a.h_b; without it (geo = 0) what remains is the
-          // material part, the contraction of C_ikjl alone: (mu - lam ln J) h_a.h_b
-          double dg = 0.0;
-          if (geo) {
-            const double* gq = g.gradX + ((size_t)(e * nq + q) * NEN) * D;
-#pragma unroll
-            for (int k = 0; k < D; ++k) dg = fma(gq[a * D + k], gq[b * D + k], dg);
-            dg *= wt[0];
-          } else {
-#pragma unroll
-            for (int k = 0; k < D; ++k) dg = fma(ga[k], hb[k], dg);
           }
 #pragma unroll
           for (int i = 0; i < D; ++i)
 #pragma unroll
-            for (int j = 0; j < D; ++j) {
-              acc[i][j] = fma(la[i], hb[j], fma(hb[i], ga[j], acc[i][j]));
-              if (i == j) acc[i][j] += dg;
-            }
+            for (int j = 0; j < D; ++j) acc[i][j] = fma(la[i], hb[j], fma(hb[i], ga[j], acc[i][j]));
+          if (!geo)
+#pragma unroll
+            for (int k = 0; k < D; ++k) dg = fma(ga[k], hb[k], dg);
         }
+        // diagonal term: mu g_a.g_b holds the geometric part delta_ij J h_a^T sigma h_b =
+        // mu (g_a.g_b - h_a.h_b) + lam ln J h_a.h_b; without it (geo = 0) what remains is the
+        // material part, the contraction of C_ikjl alone: (mu - lam ln J) h_a.h_b
+        if (geo) dg = mu * g.gram[(size_t)e * NP + pr];
+#pragma unroll
+        for (int i = 0; i < D; ++i) acc[i][i] += dg;
         const int ab = elem_blk[(e * NEN + a) * NEN + b], ba = elem_blk[(e * NEN + b) * NEN + a];
         double* Kab = K + (size_t)(ab & (kFirst - 1)) * D * D;
         double* Kba = K + (size_t)(ba & (kFirst - 1)) * D * D;
@@ -674,7 +665,7 @@ ColorTable colors(lat_ctx* h) {
 }
 
 GeomArgs geom(lat_ctx* h, int quad) {
-  return GeomArgs{h->gradX[quad].p, h->W[quad].p, h->elems.p, h->color_elems.p, h->nq[quad]};
+  return GeomArgs{h->gradX[quad].p, h->W[quad].p, h->elems.p, h->color_elems.p, h->nq[quad], h->gram[quad].p};
 }
 
 // Shared memory of the lane kernels: `vecs` cell vectors and the staged element forces.  All
@@ -745,9 +736,10 @@ void run_tangent(lat_ctx* h, const double* u_glob, int quad, const int* cells, i
   // elements of a batch: about one quadrature point per thread, no more than a colour's share
   int widest = 1;
   for (int c = 0; c < ct.n; ++c) widest = std::max(widest, ct.start[c + 1] - ct.start[c]);
-  const size_t per = sizeof(double) * (h->dim == 2 ? tangent_el_doubles<2>(g.nq) : tangent_el_doubles<3>(g.nq));
-  const int EB = std::max(1, std::min(kCellThreads / g.nq, div_up(widest, CL)));
+  const size_t per = sizeof(double) * g.nq * (h->dim == 2 ? tangent_row<2>() : tangent_row<3>());
   const size_t ub = (size_t)h->n_loc * sizeof(double);
+  const size_t room = ub < 64 * 1024 ? 104 * 1024 - ub : 80 * 1024;   // two CTAs per SM where u allows
+  const int EB = (int)std::max<size_t>(1, std::min<size_t>({(size_t)(kCellThreads / g.nq), (size_t)div_up(widest, CL), room / per}));
   const int staged = EB * per + ub <= 200 * 1024;
   const size_t shm = EB * per + (staged ? ub : 0);
   KernelTimer kt(h, quad ? "tangent_reduced" : (geometric ? "tangent_full" : "tangent_material"));

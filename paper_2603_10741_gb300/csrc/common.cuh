@@ -90,6 +90,7 @@ struct lat_ctx {
 
   // reference cell
   DBuf<double> gradX[2], W[2];  // [n_el][nq][nen][dim], [n_el][nq]
+  DBuf<double> gram[2];         // [n_el][nen (nen + 1) / 2] sum_q W g_a.g_b, pairs a <= b
   DBuf<int> elems;              // [n_el][nen]
   DBuf<int> elem_blk;           // [n_el][nen][nen] block index of (a, b); bit 30: the first element, in
                                 // colour order, to touch the block

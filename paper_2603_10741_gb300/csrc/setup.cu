@@ -107,6 +107,21 @@ void build_geometry(lat_ctx* h, const double* X, const int* E) {
       }
     }
     if (!red) h->Jinv.upload(Ji, h->stream);
+    std::vector<double> gram;
+    gram.reserve((size_t)h->n_el * nen * (nen + 1) / 2);
+    for (int e = 0; e < h->n_el; ++e)
+      for (int a = 0; a < nen; ++a)
+        for (int b = a; b < nen; ++b) {
+          double v = 0;
+          for (int q = 0; q < nq; ++q) {
+            const double* gq = gX.data() + ((size_t)e * nq + q) * nen * d;
+            double s = 0;
+            for (int k = 0; k < d; ++k) s += gq[a * d + k] * gq[b * d + k];
+            v += Wv[(size_t)e * nq + q] * s;
+          }
+          gram.push_back(v);
+        }
+    h->gram[red].upload(gram, h->stream);
     h->gradX[red].upload(gX, h->stream);
     h->W[red].upload(Wv, h->stream);
   }
@@ -645,7 +660,7 @@ extern "C" lat_status lattice_destroy(lat_handle h) {
   if (h->cap_stream) cudaStreamDestroy(h->cap_stream);
   // DBuf members free themselves through release(); walk them explicitly
   auto rel = [](auto& b) { b.release(); };
-  rel(h->gradX[0]); rel(h->gradX[1]); rel(h->W[0]); rel(h->W[1]); rel(h->elems); rel(h->elem_blk); rel(h->Jinv); rel(h->node_el_ptr); rel(h->node_el);
+  rel(h->gradX[0]); rel(h->gradX[1]); rel(h->W[0]); rel(h->W[1]); rel(h->gram[0]); rel(h->gram[1]); rel(h->elems); rel(h->elem_blk); rel(h->Jinv); rel(h->node_el_ptr); rel(h->node_el);
   rel(h->color_elems); rel(h->blk_ptr); rel(h->blk_col); rel(h->cell_nodes); rel(h->mu_cell);
   rel(h->copy_ptr); rel(h->copy_idx); rel(h->dof_fixed); rel(h->dir_unit); rel(h->aff_unit);
   rel(h->corner_of_node); rel(h->rdofs); rel(h->pdofs); rel(h->rpos); rel(h->pidx);
