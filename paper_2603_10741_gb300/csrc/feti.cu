@@ -86,30 +86,117 @@ __global__ void k_axpy2_s(int64_t n, const PcgScalars* __restrict__ sc, const do
   }
 }
 
-// partial dots of w against the first m vectors of V (stride n): part[i][block]
-__global__ void k_multidot_part(int64_t n, int m, const double* __restrict__ V, const double* __restrict__ w,
-                                double* __restrict__ part) {
-  __shared__ double red[32];
-  for (int i = 0; i < m; ++i) {
-    const double* vi = V + (size_t)i * n;
+// --- one Arnoldi step: two passes of classical Gram-Schmidt, norm, Givens rotation, scaling ------
+// Three launches instead of eleven: the block of a pass that ends last adds the partial sums (in block
+// order: deterministic) and does the scalar work, and the second pass's dot products follow the
+// first's update in the same kernel, a thread working on the same entries in both.  What is saved is
+// launches and their gaps (3 us each on small lattices) and a pass over w.
+struct ArnoldiArgs {
+  int64_t n;
+  int j, m;                 // column (vectors V_0 .. V_j), restart length
+  const double* V;
+  double* w;
+  double* part;             // [j + 2][blocks] partial sums
+  double* h1;               // [j + 1] first pass's coefficients, then the column of H
+  double* h2;               // [j + 1] second pass's
+  double* sc;               // [0] ||w||^2, [1] residual estimate
+  double* H;                // [m][m + 1]
+  double* small;            // cs [m], sn [m], g [m + 1]
+  unsigned* ticket;
+};
+
+// the block that ends last adds the partial sums of `cnt` dots into out
+__device__ __forceinline__ bool last_block_sums(const ArnoldiArgs& A, int cnt, double* out, double* red) {
+  __shared__ bool last;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    last = atomicAdd(A.ticket, 1u) == gridDim.x - 1;
+  }
+  __syncthreads();
+  if (!last) return false;
+  __threadfence();
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  for (int i = warp; i < cnt; i += nw) {
     double v = 0;
-    for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n; k += (int64_t)gridDim.x * blockDim.x)
-      v += vi[k] * w[k];
+    for (int b = lane; b < (int)gridDim.x; b += 32) v += __ldcg(A.part + (size_t)i * gridDim.x + b);
+    v = warp_sum(v);
+    if (lane == 0) out[i] = v;
+  }
+  if (threadIdx.x == 0) *A.ticket = 0;
+  (void)red;
+  return true;
+}
+
+__device__ __forceinline__ void partial_dots(const ArnoldiArgs& A, double* red) {
+  const int64_t t0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, st = (int64_t)gridDim.x * blockDim.x;
+  for (int i = 0; i <= A.j; ++i) {
+    const double* vi = A.V + (size_t)i * A.n;
+    double v = 0;
+    for (int64_t k = t0; k < A.n; k += st) v += vi[k] * A.w[k];
     v = block_sum(v, red);
-    if (threadIdx.x == 0) part[(size_t)i * gridDim.x + blockIdx.x] = v;
+    if (threadIdx.x == 0) A.part[(size_t)i * gridDim.x + blockIdx.x] = v;
   }
 }
 
-__global__ void k_multidot_final(int nb, const double* __restrict__ part, double* __restrict__ out) {
+// h1 = V^T w
+__global__ void __launch_bounds__(256) k_arnoldi_dots(ArnoldiArgs A) {
   __shared__ double red[32];
-  const int i = blockIdx.x;
-  double v = 0;
-  for (int b = threadIdx.x; b < nb; b += blockDim.x) v += part[(size_t)i * nb + b];
-  v = block_sum(v, red);
-  if (threadIdx.x == 0) out[i] = v;
+  partial_dots(A, red);
+  last_block_sums(A, A.j + 1, A.h1, red);
 }
 
-// w -= sum_i h[i] V_i  (and accumulate into hacc when given)
+// w -= V h1, h2 = V^T w
+__global__ void __launch_bounds__(256) k_arnoldi_pass(ArnoldiArgs A) {
+  __shared__ double red[32];
+  const int64_t t0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, st = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t k = t0; k < A.n; k += st) {
+    double v = A.w[k];
+    for (int i = 0; i <= A.j; ++i) v -= A.h1[i] * A.V[(size_t)i * A.n + k];
+    A.w[k] = v;
+  }
+  partial_dots(A, red);
+  last_block_sums(A, A.j + 1, A.h2, red);
+}
+
+// w -= V h2, ||w||^2; then H's column h1 + h2, its rotations and the residual estimate
+__global__ void __launch_bounds__(256) k_arnoldi_finish(ArnoldiArgs A) {
+  __shared__ double red[32];
+  const int64_t t0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, st = (int64_t)gridDim.x * blockDim.x;
+  double nrm = 0;
+  for (int64_t k = t0; k < A.n; k += st) {
+    double v = A.w[k];
+    for (int i = 0; i <= A.j; ++i) v -= A.h2[i] * A.V[(size_t)i * A.n + k];
+    A.w[k] = v;
+    nrm += v * v;
+  }
+  nrm = block_sum(nrm, red);
+  if (threadIdx.x == 0) A.part[blockIdx.x] = nrm;
+  if (!last_block_sums(A, 1, A.sc, red)) return;
+  __syncthreads();
+  if (threadIdx.x != 0) return;
+  // Givens rotations on one thread (Hessenberg column j, column major)
+  const int j = A.j, m = A.m;
+  double *cs = A.small, *sn = A.small + m, *g = A.small + 2 * m, *col = A.H + (size_t)j * (m + 1);
+  for (int i = 0; i <= j; ++i) col[i] = A.h1[i] + A.h2[i];
+  col[j + 1] = sqrt(A.sc[0]);
+  for (int i = 0; i < j; ++i) {
+    const double t = cs[i] * col[i] + sn[i] * col[i + 1];
+    col[i + 1] = -sn[i] * col[i] + cs[i] * col[i + 1];
+    col[i] = t;
+  }
+  const double a = col[j], b = col[j + 1];
+  const double r = hypot(a, b);
+  cs[j] = r > 0 ? a / r : 1.0;
+  sn[j] = r > 0 ? b / r : 0.0;
+  col[j] = r;
+  col[j + 1] = 0.0;
+  g[j + 1] = -sn[j] * g[j];
+  g[j] = cs[j] * g[j];
+  A.sc[1] = fabs(g[j + 1]);
+}
+
+// w += sgn * sum_i h[i] V_i
 __global__ void k_multi_axpy(int64_t n, int m, const double* __restrict__ V, const double* __restrict__ hcoef,
                              double sgn, double* __restrict__ w) {
   for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n; k += (int64_t)gridDim.x * blockDim.x) {
@@ -140,6 +227,32 @@ __global__ void k_primal_assemble(int64_t n_primal, const int* __restrict__ pptr
   yP[p] = v;
 }
 
+// The operator's index work after the primal assembly, in one launch over three independent sets of
+// entries: the corner rows of w cleared, w += B^T lambda on the dual entries (lam null: not), and the
+// multiplier part B v
+__global__ void k_operator_jumps(int n_cells, int n_P, int64_t nd, int64_t L, const int* __restrict__ pdofs,
+                                 const int* __restrict__ de, const int* __restrict__ l1, const int* __restrict__ l2,
+                                 const int* __restrict__ lp, const int* __restrict__ lm, const double* __restrict__ lam,
+                                 const double* __restrict__ v, double* __restrict__ w, double* __restrict__ wl) {
+  int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (t < L) {
+    wl[t] = v[lp[t]] - v[lm[t]];
+    return;
+  }
+  t -= L;
+  if (t < nd) {
+    if (!lam) return;
+    double s = 0;
+    const int c1 = l1[t], c2 = l2[t];
+    if (c1) s += (c1 > 0 ? 1.0 : -1.0) * lam[abs(c1) - 1];
+    if (c2) s += (c2 > 0 ? 1.0 : -1.0) * lam[abs(c2) - 1];
+    w[de[t]] += s;
+    return;
+  }
+  t -= nd;
+  if (t < (int64_t)n_cells * n_P) w[(size_t)pdofs[t / n_cells] * n_cells + t % n_cells] = 0.0;
+}
+
 // zero the corner rows of a local vector (entries listed per primal dof) -- all corner rows
 __global__ void k_zero_rows(int n_cells, int n_P, const int* __restrict__ pdofs, double* __restrict__ loc) {
   int s = blockIdx.x * blockDim.x + threadIdx.x;
@@ -147,33 +260,11 @@ __global__ void k_zero_rows(int n_cells, int n_P, const int* __restrict__ pdofs,
   for (int j = 0; j < n_P; ++j) loc[(size_t)pdofs[j] * n_cells + s] = 0.0;
 }
 
-// lambda_l = x[p_l] - x[m_l]  (B x), or lambda += ...
-__global__ void k_jump(int64_t L, const int* __restrict__ lp, const int* __restrict__ lm,
-                       const double* __restrict__ x, double a, double* __restrict__ lam, int accumulate) {
-  int64_t l = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (l >= L) return;
-  double v = a * (x[lp[l]] - x[lm[l]]);
-  lam[l] = accumulate ? lam[l] + v : v;
-}
-
-// y[dual entry] += a * (B^T lambda)
-__global__ void k_jump_t(int64_t nd, const int* __restrict__ de, const int* __restrict__ l1,
-                         const int* __restrict__ l2, const double* __restrict__ lam, double a,
-                         double* __restrict__ y) {
-  int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (e >= nd) return;
-  double v = 0;
-  int c1 = l1[e], c2 = l2[e];
-  if (c1) v += (c1 > 0 ? 1.0 : -1.0) * lam[abs(c1) - 1];
-  if (c2) v += (c2 > 0 ? 1.0 : -1.0) * lam[abs(c2) - 1];
-  y[de[e]] += a * v;
-}
-
 // The interface iteration on vectors outside the tensor-core path: y[dual entry] = B^T v (scaled by
 // 1/multiplicity when `scale` is given) with v formed on the fly, so that the vector updates need no
 // pass of their own:
 //   DIR: the new direction z + beta p (p when frozen);  else: the new residual y - alpha q
-// The other entries of y stay zero (cleared once per solve).
+// The other entries of y stay zero (cleared at setup).
 template <bool DIR>
 __global__ void k_pcg_scatter(int64_t nd, const int* __restrict__ de, const int* __restrict__ l1,
                               const int* __restrict__ l2, const double* __restrict__ scale,
@@ -201,16 +292,18 @@ __global__ void k_pcg_scatter(int64_t nd, const int* __restrict__ de, const int*
 // on the fly; without it they ran before), the dot product, and in the block that ends last the PCG
 // scalars:
 //   DIR: p = z + beta p, q = B t2, p.q, alpha;  else: x += alpha p, r -= alpha q, z = B_D t2, r.z,
-//   beta, and whether the loop goes on (told to the graph's loop node when there is one).
+//   beta, and whether the loop goes on (told to the graph's loop node when there is one); before the
+//   first iteration (kPcgFirst) z and r.z alone.
 // A multiplier belongs to one thread.  Partial sums are added in block order: deterministic.
 constexpr int kPcgBlocks = 1216;
+enum { kPcgHost = 0, kPcgLoop = 1, kPcgFirst = 2 };
 
 template <bool DIR, bool FLY>
 __global__ void __launch_bounds__(256)
     k_pcg_jump(int64_t L, const int* __restrict__ lp, const int* __restrict__ lm, const double* __restrict__ ls,
                const double* __restrict__ t2, double* __restrict__ x, double* __restrict__ r, double* __restrict__ z,
                double* __restrict__ p, double* __restrict__ q, PcgScalars* __restrict__ sc,
-               double* __restrict__ part, unsigned* __restrict__ ticket, cudaGraphConditionalHandle loop, int has_loop) {
+               double* __restrict__ part, unsigned* __restrict__ ticket, cudaGraphConditionalHandle loop, int mode) {
   __shared__ double red[32];
   __shared__ bool last;
   const double al = sc->alpha, be = sc->beta;
@@ -257,6 +350,8 @@ __global__ void __launch_bounds__(256)
     const bool ok = !frozen && v > 0.0 && sc->rz > 0.0;
     if (!ok) sc->frozen = 1.0;
     sc->alpha = ok ? sc->rz / v : 0.0;
+  } else if (mode == kPcgFirst) {
+    sc->rz = sc->rz0 = v;
   } else {
     const bool ok = !frozen && v > 0.0 && sc->rz > 0.0;
     if (!ok) sc->frozen = 1.0;
@@ -265,24 +360,45 @@ __global__ void __launch_bounds__(256)
     sc->its += 1.0;
     const bool go = sc->its < sc->max_it &&
                     (sc->tol2 == 0.0 || (ok && sc->rz0 > 0.0 && !(v <= sc->tol2 * sc->rz0)));
-    if (has_loop) cudaGraphSetConditional(loop, go ? 1u : 0u);
+    if (mode == kPcgLoop) cudaGraphSetConditional(loop, go ? 1u : 0u);
   }
 }
 
-// scalars at the start of a solve, after r0.z0 is in sc->rz
-__global__ void k_pcg_start(PcgScalars* __restrict__ sc, unsigned* __restrict__ ticket, double max_it, double tol2) {
-  sc->pq = sc->alpha = sc->beta = sc->frozen = sc->its = 0.0;
-  sc->rz0 = sc->rz;
-  sc->max_it = max_it;
-  sc->tol2 = tol2;
-  *ticket = 0;
+// the start of a solve: r = v_l - B t, x = p = 0, cleared scalars
+__global__ void k_pcg_start(int64_t L, const int* __restrict__ lp, const int* __restrict__ lm,
+                            const double* __restrict__ vl, const double* __restrict__ t, double* __restrict__ r,
+                            double* __restrict__ x, double* __restrict__ p, PcgScalars* __restrict__ sc,
+                            unsigned* __restrict__ ticket, double max_it, double tol2) {
+  const int64_t l = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (l == 0) {
+    *sc = PcgScalars{};
+    sc->max_it = max_it;
+    sc->tol2 = tol2;
+    *ticket = 0;
+  }
+  if (l >= L) return;
+  r[l] = vl[l] - (t[lp[l]] - t[lm[l]]);
+  x[l] = 0.0;
+  p[l] = 0.0;
 }
 
-// z = B_D t2: the scaled jump (both copies of a multiplier carry their node's 1/multiplicity)
-__global__ void k_jump_scaled(int64_t L, const int* __restrict__ lp, const int* __restrict__ lm,
-                              const double* __restrict__ ls, const double* __restrict__ t2, double* __restrict__ z) {
-  const int64_t l = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (l < L) z[l] = (t2[lp[l]] - t2[lm[l]]) * ls[l];
+// y[dual entry] = B^T x
+__global__ void k_scatter_dual(int64_t nd, const int* __restrict__ de, const int* __restrict__ l1,
+                               const int* __restrict__ l2, const double* __restrict__ x, double* __restrict__ y) {
+  const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (e >= nd) return;
+  double v = 0;
+  const int c1 = l1[e], c2 = l2[e];
+  if (c1) v += (c1 > 0 ? 1.0 : -1.0) * x[abs(c1) - 1];
+  if (c2) v += (c2 > 0 ? 1.0 : -1.0) * x[abs(c2) - 1];
+  y[de[e]] = v;
+}
+
+// w_u += t, w_l = -x
+__global__ void k_precond_finish(int64_t nu, int64_t L, const double* __restrict__ t, const double* __restrict__ x,
+                                 double* __restrict__ w) {
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < nu + L; i += (int64_t)gridDim.x * blockDim.x)
+    w[i] = i < nu ? w[i] + t[i] : -x[i - nu];
 }
 
 // saddle-point vector -> global vector: corners from the primal part, other DOFs the mean of
@@ -1136,32 +1252,6 @@ __global__ void __launch_bounds__(512) k_gemv_xs_f32(int n, int ld, const float*
   }
 }
 
-// FGMRES small dense work on one thread: Hessenberg column j (in Hh[(m+1) x m], column major)
-// after the Arnoldi step; Givens rotations in small[0..m) cs, [m..2m) sn, g in [2m..3m+1)
-__global__ void k_givens(int j, int m, double* __restrict__ H, double* __restrict__ small,
-                         const double* __restrict__ hcol, const double* __restrict__ nrm2, double* __restrict__ est) {
-  double* cs = small;
-  double* sn = small + m;
-  double* g = small + 2 * m;
-  double* col = H + (size_t)j * (m + 1);
-  for (int i = 0; i <= j; ++i) col[i] = hcol[i];
-  col[j + 1] = sqrt(nrm2[0]);
-  for (int i = 0; i < j; ++i) {
-    const double t = cs[i] * col[i] + sn[i] * col[i + 1];
-    col[i + 1] = -sn[i] * col[i] + cs[i] * col[i + 1];
-    col[i] = t;
-  }
-  const double a = col[j], b = col[j + 1];
-  const double r = hypot(a, b);
-  cs[j] = r > 0 ? a / r : 1.0;
-  sn[j] = r > 0 ? b / r : 0.0;
-  col[j] = r;
-  col[j + 1] = 0.0;
-  g[j + 1] = -sn[j] * g[j];
-  g[j] = cs[j] * g[j];
-  est[0] = fabs(g[j + 1]);
-}
-
 __global__ void k_gmres_init(int m, double* __restrict__ small, const double* __restrict__ nrm2) {
   for (int i = 0; i < 3 * m + 1; ++i) small[i] = 0.0;
   small[2 * m] = sqrt(nrm2[0]);
@@ -1472,6 +1562,8 @@ void run_prepare_solver(lat_ctx* h, const lat_newton_opts* o, const double* u_gl
   }
   // temporaries
   for (int i = 0; i < 6; ++i) h->kv_tmp[i].ensure(h->n_krylov);
+  // the interface scatters' vector: they rewrite its dual entries and leave the rest at zero
+  LAT_CUDA(cudaMemsetAsync(h->kv_tmp[3].p, 0, h->n_krylov * sizeof(double), h->stream));
   h->pcg_ws.ensure(std::max<size_t>(1, (size_t)5 * h->n_lambda));
   h->gP.ensure(std::max<int64_t>(np, 1));
   h->xP.ensure(std::max<int64_t>(np, 1));
@@ -1512,14 +1604,10 @@ void feti_operator(lat_ctx* h, const double* v, double* w, bool with_lambda, boo
   if (h->n_primal)
     LAT_LAUNCH(h, k_primal_assemble<<<div_up(h->n_primal, 256), 256, 0, h->stream>>>(h->n_primal, h->p_copy_ptr.p,
         h->p_copy.p, w, pr_of(h, w), 0));
-  LAT_LAUNCH(h, k_zero_rows<<<div_up(h->n_cells, 256), 256, 0, h->stream>>>(h->n_cells, h->n_P, h->pdofs.p, w));
-  if (h->n_lambda) {
-    if (with_lambda)
-      LAT_LAUNCH(h, k_jump_t<<<div_up(h->n_dual, 256), 256, 0, h->stream>>>(h->n_dual, h->dual_entry.p, h->dual_l1.p,
-          h->dual_l2.p, la_of(h, v), 1.0, w));
-    LAT_LAUNCH(h, k_jump<<<div_up(h->n_lambda, 256), 256, 0, h->stream>>>(h->n_lambda, h->lam_p.p, h->lam_m.p, v, 1.0,
-                                                              la_of(h, w), 0));
-  }
+  const int64_t tot = h->n_lambda + h->n_dual + (int64_t)h->n_cells * h->n_P;
+  LAT_LAUNCH(h, k_operator_jumps<<<div_up(tot, 256), 256, 0, h->stream>>>(
+                    h->n_cells, h->n_P, h->n_dual, h->n_lambda, h->pdofs.p, h->dual_entry.p, h->dual_l1.p, h->dual_l2.p,
+                    h->lam_p.p, h->lam_m.p, with_lambda ? la_of(h, v) : nullptr, v, w, la_of(h, w)));
   LAT_CHECK_LAUNCH();
 }
 
@@ -1716,7 +1804,7 @@ bool capture_pcg_loop(lat_ctx* h, Body&& body) {
                                           cudaStreamCaptureModeRelaxed) == cudaSuccess) {
     h->stream = h->cap_stream;
     try {
-      body(loop, 1);
+      body(loop, kPcgLoop);
     } catch (const LatError&) {
       ok = false;
     }
@@ -1753,7 +1841,7 @@ void run_kinv(lat_ctx* h, const double* v, double* w) {
 void run_block_precond(lat_ctx* h, const double* v, double* w, int pcg_iters, double pcg_rtol) {
   const int64_t L = h->n_lambda;
   double* t = h->kv_tmp[2].p;   // K^-rom v_u
-  double* t1 = h->kv_tmp[3].p;
+  double* t1 = h->kv_tmp[3].p;  // zero off the dual entries (cleared at setup, written by the scatters alone)
   double* t2 = h->kv_tmp[4].p;
   double* pv = h->pcg_ws.p;     // five multiplier-sized work vectors
   if (L == 0) {
@@ -1769,17 +1857,13 @@ void run_block_precond(lat_ctx* h, const double* v, double* w, int pcg_iters, do
   LAT_REQUIRE((size_t)5 * L <= h->pcg_ws.n, LAT_EINVAL, "multiplier work space too small");
   const int64_t nloc = (int64_t)h->n_loc * h->n_cells;
   const bool tc = fused_dual(h), tcs = fused_schur(h);
-  // y = v_l - B t
-  LAT_CUDA(cudaMemcpyAsync(y, la_of(h, v), L * sizeof(double), cudaMemcpyDeviceToDevice, h->stream));
-  LAT_LAUNCH(h, k_jump<<<div_up(L, 256), 256, 0, h->stream>>>(L, h->lam_p.p, h->lam_m.p, t, -1.0, y, 1));
-  LAT_CHECK_LAUNCH();
-  // PCG on S x = y from x = 0
-  LAT_CUDA(cudaMemsetAsync(x, 0, L * sizeof(double), h->stream));
-  // the local vector of the scatters: zero off the dual entries, which every scatter rewrites
-  if (!tc || !tcs) LAT_CUDA(cudaMemsetAsync(t1, 0, (nloc + h->n_primal) * sizeof(double), h->stream));
   auto* sc = reinterpret_cast<PcgScalars*>(h->red_part.p + 3000);
   auto* ticket = reinterpret_cast<unsigned*>(h->red_part.p + 3020);
   double* part = h->red_part.p + 1024;
+  // PCG on S x = y = v_l - B t from x = 0
+  LAT_LAUNCH(h, k_pcg_start<<<div_up(L, 256), 256, 0, h->stream>>>(L, h->lam_p.p, h->lam_m.p, la_of(h, v), t, y, x, p, sc,
+                                                                   ticket, (double)pcg_iters, pcg_rtol * pcg_rtol));
+  LAT_CHECK_LAUNCH();
   if (pcg_iters > 0) {
     // PCG until the preconditioned residual r^T M r has dropped by pcg_rtol^2 (0: never), at most
     // pcg_iters iterations, or until breakdown.  An iteration updates the search direction first (p =
@@ -1791,38 +1875,34 @@ void run_block_precond(lat_ctx* h, const double* v, double* w, int pcg_iters, do
     // the scalars; outside the tensor-core path, whose packing reads the vectors at random, the
     // updates of p, x and r ride along as well.  An iteration was 18 graph nodes (15 with the
     // packing), now 9 (11).
-    LAT_CUDA(cudaMemsetAsync(sc, 0, sizeof(PcgScalars), h->stream));
-    LAT_CUDA(cudaMemsetAsync(p, 0, L * sizeof(double), h->stream));
-    if (!tcs) pcg_scatter<false>(h, y, q, sc, t1);   // alpha = 0: B_D^T y
-    dual_precond_local(h, y, t1, t2);
-    LAT_LAUNCH(h, k_jump_scaled<<<div_up(L, 256), 256, 0, h->stream>>>(L, h->lam_p.p, h->lam_m.p, h->lam_scale.p, t2, z));
-    dev_dot(h, L, y, z, &sc->rz);
-    LAT_LAUNCH(h, k_pcg_start<<<1, 1, 0, h->stream>>>(sc, ticket, (double)pcg_iters, pcg_rtol * pcg_rtol));
-    LAT_CHECK_LAUNCH();
     const int nb = ew_blocks(h, L);
     const int jb = (int)std::min<int64_t>(kPcgBlocks, div_up(L, 256));
-    auto jump = [&](auto kern, cudaGraphConditionalHandle loop, int has_loop) {
+    auto jump = [&](auto kern, cudaGraphConditionalHandle loop, int mode) {
       LAT_LAUNCH(h, kern<<<jb, 256, 0, h->stream>>>(L, h->lam_p.p, h->lam_m.p, h->lam_scale.p, t2, x, y, z, p, q, sc, part,
-                                                    ticket, loop, has_loop));
+                                                    ticket, loop, mode));
     };
-    auto body = [&](cudaGraphConditionalHandle loop, int has_loop) {
+    if (!tcs) pcg_scatter<false>(h, y, q, sc, t1);   // alpha = 0: B_D^T y
+    dual_precond_local(h, y, t1, t2);
+    jump(k_pcg_jump<false, false>, 0, kPcgFirst);
+    LAT_CHECK_LAUNCH();
+    auto body = [&](cudaGraphConditionalHandle loop, int mode) {
       if (tc) {
         LAT_LAUNCH(h, k_xpby_s<<<nb, 256, 0, h->stream>>>(L, z, sc, p));
         kinv(h, nullptr, t2, KINV_DUAL, p);
-        jump(k_pcg_jump<true, false>, loop, 0);
+        jump(k_pcg_jump<true, false>, loop, mode);
       } else {
         pcg_scatter<true>(h, z, p, sc, t1);
         kinv(h, t1, t2, KINV_DUAL);   // t1 vanishes off the dual DOFs; only dual rows of t2 are read
-        jump(k_pcg_jump<true, true>, loop, 0);
+        jump(k_pcg_jump<true, true>, loop, mode);
       }
       if (tcs) {
         LAT_LAUNCH(h, k_axpy2_s<<<nb, 256, 0, h->stream>>>(L, sc, p, q, x, y));
         dual_precond_local(h, y, t1, t2);
-        jump(k_pcg_jump<false, false>, loop, has_loop);
+        jump(k_pcg_jump<false, false>, loop, mode);
       } else {
         pcg_scatter<false>(h, y, q, sc, t1);
         dual_precond_local(h, y, t1, t2);
-        jump(k_pcg_jump<false, true>, loop, has_loop);
+        jump(k_pcg_jump<false, true>, loop, mode);
       }
       LAT_CHECK_LAUNCH();
     };
@@ -1839,7 +1919,7 @@ void run_block_precond(lat_ctx* h, const double* v, double* w, int pcg_iters, do
       h->n_launch += (int64_t)hs->its * h->pcg_graph_kernels;
     } else {
       for (int it = 0; it < pcg_iters; ++it) {
-        body(0, 0);
+        body(0, kPcgHost);
         if (pcg_rtol == 0) continue;
         read();
         if (hs->frozen != 0.0 || !(hs->rz0 > 0) || hs->rz <= hs->tol2 * hs->rz0) break;
@@ -1853,14 +1933,13 @@ void run_block_precond(lat_ctx* h, const double* v, double* w, int pcg_iters, do
   if (tc) {
     kinv(h, nullptr, w, KINV_DUAL_IN, x);
   } else {
-    LAT_CUDA(cudaMemsetAsync(t1, 0, (nloc + h->n_primal) * sizeof(double), h->stream));
-    LAT_LAUNCH(h, k_jump_t<<<div_up(h->n_dual, 256), 256, 0, h->stream>>>(h->n_dual, h->dual_entry.p, h->dual_l1.p,
-                                                                          h->dual_l2.p, x, 1.0, t1));
+    LAT_LAUNCH(h, k_scatter_dual<<<div_up(h->n_dual, 256), 256, 0, h->stream>>>(h->n_dual, h->dual_entry.p,
+                                                                                h->dual_l1.p, h->dual_l2.p, x, t1));
     LAT_CHECK_LAUNCH();
     kinv(h, t1, w, KINV_DUAL_IN);
   }
-  LAT_LAUNCH(h, k_axpby<<<ew_blocks(h, nloc + h->n_primal), 256, 0, h->stream>>>(nloc + h->n_primal, 1.0, t, 1.0, w));
-  LAT_LAUNCH(h, k_axpby<<<ew_blocks(h, L), 256, 0, h->stream>>>(L, -1.0, x, 0.0, la_of(h, w)));
+  const int64_t nu = nloc + h->n_primal;
+  LAT_LAUNCH(h, k_precond_finish<<<ew_blocks(h, nu + L), 256, 0, h->stream>>>(nu, L, t, x, w));
   LAT_CHECK_LAUNCH();
 }
 
@@ -1890,8 +1969,9 @@ int fgmres_core(lat_ctx* h, const GmresLevel& L, const double* b, double* x, boo
   L.H->ensure((size_t)(m + 1) * m + 4 * (m + 1));
   L.small->ensure(3 * m + 8);
   L.scal->ensure(8 + 4 * (m + 2));
-  const int nb = red_blocks(n);
-  h->dots_part.ensure((size_t)(m + 1) * nb);
+  const int nb = (int)std::min<int64_t>(kPcgBlocks, div_up(n, 256));
+  h->dots_part.ensure((size_t)(m + 2) * nb);
+  LAT_CUDA(cudaMemsetAsync(h->red_part.p + 3024, 0, sizeof(double), h->stream));   // the Arnoldi ticket
   double* sc = L.scal->p;              // [0] nrm2, [1] estimate
   double* hcol = sc + 8;
   double* h2 = hcol + (m + 2);
@@ -1937,14 +2017,11 @@ int fgmres_core(lat_ctx* h, const GmresLevel& L, const double* b, double* x, boo
       feti_operator(h, zj, w, true, op32);
       // CGS with one re-orthogonalisation
       KernelTimer kt(h, "krylov_orth");
-      for (int pass = 0; pass < 2; ++pass) {
-        LAT_LAUNCH(h, k_multidot_part<<<nb, 256, 0, h->stream>>>(n, j + 1, L.V->p, w, h->dots_part.p));
-        LAT_LAUNCH(h, k_multidot_final<<<j + 1, 256, 0, h->stream>>>(nb, h->dots_part.p, pass == 0 ? hcol : h2));
-        LAT_LAUNCH(h, k_multi_axpy<<<eb, 256, 0, h->stream>>>(n, j + 1, L.V->p, pass == 0 ? hcol : h2, -1.0, w));
-      }
-      LAT_LAUNCH(h, k_axpby<<<1, 256, 0, h->stream>>>(j + 1, 1.0, h2, 1.0, hcol));
-      dev_dot(h, n, w, w, sc);
-      LAT_LAUNCH(h, k_givens<<<1, 1, 0, h->stream>>>(j, m, L.H->p, L.small->p, hcol, sc, sc + 1));
+      const ArnoldiArgs A{n, j, m, L.V->p, w, h->dots_part.p, hcol, h2, sc, L.H->p, L.small->p,
+                          reinterpret_cast<unsigned*>(h->red_part.p + 3024)};
+      LAT_LAUNCH(h, k_arnoldi_dots<<<nb, 256, 0, h->stream>>>(A));
+      LAT_LAUNCH(h, k_arnoldi_pass<<<nb, 256, 0, h->stream>>>(A));
+      LAT_LAUNCH(h, k_arnoldi_finish<<<nb, 256, 0, h->stream>>>(A));
       LAT_LAUNCH(h, k_scale_dev<<<eb, 256, 0, h->stream>>>(n, w, sc, L.V->p + (size_t)(j + 1) * n));
       LAT_CHECK_LAUNCH();
       LAT_CUDA(cudaMemcpyAsync(hp, sc, 2 * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
