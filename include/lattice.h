@@ -228,8 +228,10 @@ typedef struct {
                               block LU with the cluster sweeps in the forms taken when larger
                               blocks do not fit (8-CTA clusters, block rows read from global
                               memory instead of prefetched), 0 the
-                              explicit inverse (N^2 m^3 to build, one dense product per solve;
-                              FP32 copy in the mixed modes), -1 (default) block LU when the
+                              explicit inverse by block recurrences (N^2 m^3 to build, one dense
+                              product per solve; FP32 copy in the mixed modes), -1 (default) the
+                              explicit inverse, built as a whole or by the recurrences, whichever
+                              chain of steps is shorter, and block LU when the
                               explicit inverse would hold more than 8192^2 entries (N blocks of
                               size m, N m > 8192) */
   int32_t precond_tangent; /* principal tangents the preconditioner's local blocks are built from:
@@ -337,7 +339,7 @@ lat_status feti_from_global(lat_handle h, const double* u_glob, double* v);
  * "tangent_reduced", "greedy_update", "apply_reduced" / "apply_reduced_fp32", "apply_percell" /
  * "apply_percell_fp32", "local_segmm", "local_gemv", "local_tc" and their "_dual" / "_dual_in"
  * variants inside the interface solve, "dual_schur" / "dual_schur_tc", "gj_update", "gj_pivot", "densify",
- * "phi_schur", "coarse_blocked", "coarse_gemv", "coarse_solve", "krylov_orth").  enable = 1
+ * "phi_schur", "coarse_blocked", "coarse_dense", "coarse_gemv", "coarse_solve", "krylov_orth").  enable = 1
  * times every named kernel; the interface PCG iteration then runs launch by launch instead of
  * as a CUDA-graph replay, so that every launch is timed.  enable = 2 times only the tangent
  * action kernels ("apply_*") and keeps the graph replays.  lattice_set_timing clears the

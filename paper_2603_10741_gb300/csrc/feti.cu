@@ -1382,6 +1382,21 @@ bool precond_material(const lat_ctx* h, const lat_newton_opts* o) {
   return pt == 1 || (pt < 0 && h->dim == 3);
 }
 
+// Whether inverting the coarse matrix as a whole beats the recurrences over its blocks.  Both are
+// chains: a sweep's of pivot blocks (150 us per panel of 128 columns, 26 us per 32 in a small matrix)
+// and the recurrences' of N block inversions and products (12 us each while they fit one wave), and
+// only beyond a few thousand primal DOFs does the dense update's work (n^2 entries per panel) or, for
+// wide blocks, the products' m^3 show.  Measured, as a whole against by blocks: 510 primal DOFs in 15
+// blocks 3.1 and 3.7 ms, 1701 in 7 3.6 and 4.8, 3267 in 9 9.0 and 15.3, 5460 in 10 22 and 51; 6142 in 32
+// (the enriched 32x32 ring lattice) stay with the recurrences, 21 ms.
+bool coarse_dense_faster(const lat_ctx* h) {
+  auto sweep = [](double n) {
+    return n >= kSweepLarge ? std::ceil(n / kSweepPanel) * (150.0 + 4e-6 * n * n) : 26.0 * std::ceil(n / 32.0);
+  };
+  const double np = (double)h->n_primal, m = h->cb_m;
+  return sweep(np) < h->cb_n * (sweep(m) + 45.0 + 6.4e-6 * m * m * m);
+}
+
 void run_prepare_solver(lat_ctx* h, const lat_newton_opts* o, const double* u_glob) {
   LAT_REQUIRE(h->n_r > 0, LAT_EINVAL, "select principal cells first");
   const double* Kpre = h->Kp.p;
@@ -1522,10 +1537,11 @@ void run_prepare_solver(lat_ctx* h, const lat_newton_opts* o, const double* u_gl
   } else if (np > 0) {
     h->CoarseInv.ensure((size_t)np * np);
     LAT_CUDA(cudaMemsetAsync(h->CoarseInv.p, 0, (size_t)np * np * sizeof(double), h->stream));
-    if (h->coarse_blocked) {
+    if (h->coarse_blocked && (want == 0 || !coarse_dense_faster(h))) {
       KernelTimer kt(h, "coarse_blocked");
       run_coarse_blocked(h, h->Sloc.p, np, true);
     } else {
+      KernelTimer kt(h, "coarse_dense");
       const int64_t n_ent = (int64_t)h->coarse_row.n;
       LAT_LAUNCH(h, k_coarse<<<div_up(n_ent, 256), 256, 0, h->stream>>>(n_ent, np, nP, h->coarse_row.p,
           h->coarse_col.p, h->coarse_ptr.p, h->coarse_src.p, h->key_slot.p, h->c_cell.p, h->Sloc.p, h->CoarseInv.p));
