@@ -417,14 +417,14 @@ struct GroupPlan {
   size_t shm = 0;
 };
 
-// Groups of 16 nodes read fewer union rows per output row and win when the action is one
-// principal over many waves of CTAs (measured 1.3x faster on 8000 strut cells); groups of 8 keep
-// more CTAs in flight and win otherwise.  False when no group size fits in shared memory (the
-// per-(cell, node) kernel runs then).
+// Groups of 16 nodes read fewer union rows per output row and win when the action is one principal
+// and they fill the SMs (8000 strut cells 1.3x, 1728 cells 29.7 -> 26.1 us, 1000 and 512 cells the
+// same); groups of 8 keep more CTAs in flight and win otherwise.  False when no group size fits in
+// shared memory (the per-(cell, node) kernel runs then).
 bool group_plan(lat_ctx* h, GroupPlan* p) {
   if (h->ng[0].n_grp == 0) return false;
   const int64_t tiles = div_up(h->n_cells, 128);
-  const bool wide = h->n_r == 1 && tiles * h->ng[1].n_grp >= 8LL * h->n_sm;
+  const bool wide = h->n_r == 1 && tiles * h->ng[1].n_grp >= h->n_sm;
   for (int k : {wide ? 1 : 0, 0}) {
     p->G = &h->ng[k];
     p->shm = group_smem(*p->G, h->n_r, &p->rch);
