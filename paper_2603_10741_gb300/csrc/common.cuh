@@ -201,6 +201,7 @@ struct lat_ctx {
   DBuf<double> gP, xP;                // primal vectors
   DBuf<float> Phi32;                  // FP32 copy of Phi (mixed modes)
   DBuf<float> x32, y32;               // mixed-precision local vectors
+  DBuf<float> xf32;                   // FP32 cell values in key order (segmented products)
   DBuf<double> kv_tmp[6];             // saddle-point sized temporaries
   DBuf<double> pcg_ws;                // interface PCG vectors (5 x n_lambda)
   DBuf<double> V, Zk, Hh, gmres_small, dots_part;

@@ -948,75 +948,92 @@ __global__ void __launch_bounds__(256)
   }
 }
 
-// few keys: segmented GEMM over 64 rows x BN cells of one key, cells in key order (perm);
-// FP32 operands accumulate in FP32 (TG = float), FP64 in FP64 (BN a multiple of 16).
-template <typename TG, int BN>
-__global__ void __launch_bounds__(256)
-    k_local_segmm(int n_cells, int n_Kr, int n_Kc, int n_P, int ldg, int64_t kstride, int scale_mul,
-                  const TG* __restrict__ G,
-                  const int* __restrict__ tile_seg,
-                  const int* __restrict__ tile_c0, const int* __restrict__ seg_ptr, const int* __restrict__ perm,
-                  const double* __restrict__ cscale, const int* __restrict__ rr, const int* __restrict__ rc,
-                  const int* __restrict__ pdofs,
-                  const double* __restrict__ X, double* __restrict__ Y) {
-  constexpr int NV = BN / 16;
-  const int tile = blockIdx.x;
-  const int k = tile_seg[tile];
-  const int c0 = tile_c0[tile];
-  const int c_end = seg_ptr[k + 1];
-  const int rows = n_Kr + n_P;
-  const int i0 = blockIdx.y * 64;
-  const TG* g = G + (size_t)k * kstride;
-  __shared__ TG Gs[64][33];
-  __shared__ TG Xs[32][BN + 1];
-  __shared__ int cells[BN];
-  const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
-  if (threadIdx.x < BN) {
-    const int c = c0 + threadIdx.x;
-    cells[threadIdx.x] = c < c_end ? perm[c] : -1;
+// few keys, FP32: the cells' values in key order, [k][position], converted once (every row tile of
+// the product reads them, and the conversion runs on the narrow FP64 pipe)
+__global__ void k_pack_f32(int n_cells, int n_K, const int* __restrict__ rc, const int* __restrict__ perm,
+                           const double* __restrict__ X, float* __restrict__ Xf) {
+  const int pos = blockIdx.x * blockDim.x + threadIdx.x, k = blockIdx.y;
+  if (pos < n_cells) Xf[(size_t)k * n_cells + pos] = (float)X[(size_t)rc[k] * n_cells + perm[pos]];
+}
+
+// Segmented GEMM over 64 rows x 32 cells of one key, FP32 products and sums in K order.  128 threads
+// of 4 x 4 outputs: two 16-byte shared loads per 16 multiply-adds, the next K chunk's global loads in
+// flight during the current one, tiles of 32 cells because the segments are short (25 keys of 1024
+// ring cells average 41).  The 108 products of a 32x32 ring load step outside the interface loop
+// (blocks of 576 x 568, 576 x 56 and 56 x 56): 2.7 ms against 6.2 ms with scalar shared loads, no
+// prefetch, 64-cell tiles and the FP64 conversion of every operand in every row tile.
+constexpr int kSegCells = 32;
+
+__global__ void __launch_bounds__(128)
+    k_local_segmm32(int n_cells, int n_Kr, int n_Kc, int n_P, int ldg, int64_t kstride, int scale_mul,
+                    const float* __restrict__ G, const int* __restrict__ tile_seg, const int* __restrict__ tile_c0,
+                    const int* __restrict__ seg_ptr, const int* __restrict__ perm, const double* __restrict__ cscale,
+                    const int* __restrict__ rr, const int* __restrict__ pdofs, const float* __restrict__ Xf,
+                    double* __restrict__ Y) {
+  constexpr int KC = 32, LD = 68;
+  __shared__ __align__(16) float As[KC][LD];        // [k][row]
+  __shared__ __align__(16) float Xs[KC][kSegCells];
+  __shared__ int cells[kSegCells];
+  __shared__ double fac[kSegCells];
+  const int key = tile_seg[blockIdx.x], c0 = tile_c0[blockIdx.x], nc = min(kSegCells, seg_ptr[key + 1] - c0);
+  const int rows = n_Kr + n_P, i0 = blockIdx.y * 64, t = threadIdx.x;
+  const float* g = G + (size_t)key * kstride;
+  if (t < kSegCells) {
+    const int s = t < nc ? perm[c0 + t] : -1;
+    const double c = s >= 0 ? cscale[s] : 1.0;
+    cells[t] = s;
+    fac[t] = scale_mul ? c : 1.0 / c;
   }
-  TG acc[4][NV];
+  const int lk = t & 31, lr = t >> 5;               // loads: a lane per k of A, per cell of X
+  float a[16], x[8];
+  auto fetch = [&](int l0) {
+#pragma unroll
+    for (int q = 0; q < 16; ++q) {
+      const int r = i0 + lr + 4 * q;
+      a[q] = r < rows && l0 + lk < n_Kc ? g[(size_t)r * ldg + l0 + lk] : 0.f;
+    }
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      const int k = l0 + lr + 4 * q;
+      x[q] = lk < nc && k < n_Kc ? Xf[(size_t)k * n_cells + c0 + lk] : 0.f;
+    }
+  };
+  const int tx = t & 7, ty = t >> 3;                // cells 4 tx .., rows 4 ty ..
+  float acc[4][4];
 #pragma unroll
   for (int u = 0; u < 4; ++u)
 #pragma unroll
-    for (int v = 0; v < NV; ++v) acc[u][v] = TG(0);
-  for (int l0 = 0; l0 < n_Kc; l0 += 32) {
+    for (int v = 0; v < 4; ++v) acc[u][v] = 0.f;
+  fetch(0);
+  for (int l0 = 0; l0 < n_Kc; l0 += KC) {
     __syncthreads();
-    for (int t = threadIdx.x; t < 64 * 32; t += blockDim.x) {
-      const int r = t / 32, c = t % 32;
-      const int gi = i0 + r, gl = l0 + c;
-      Gs[r][c] = (gi < rows && gl < n_Kc) ? g[(size_t)gi * ldg + gl] : TG(0);
-    }
-    for (int t = threadIdx.x; t < 32 * BN; t += blockDim.x) {
-      const int r = t / BN, c = t % BN;
-      const int gl = l0 + r, s = cells[c];
-      Xs[r][c] = (gl < n_Kc && s >= 0) ? (TG)X[(size_t)rc[gl] * n_cells + s] : TG(0);
-    }
+#pragma unroll
+    for (int q = 0; q < 16; ++q) As[lk][lr + 4 * q] = a[q];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) Xs[lr + 4 * q][lk] = x[q];
     __syncthreads();
-    const int lim = min(32, n_Kc - l0);   // no multiply-adds on the padding of the last chunk
+    if (l0 + KC < n_Kc) fetch(l0 + KC);
+    const int lim = min(KC, n_Kc - l0);
 #pragma unroll 8
     for (int l = 0; l < lim; ++l) {
-      TG gv[4], xv[NV];
-#pragma unroll
-      for (int u = 0; u < 4; ++u) gv[u] = Gs[ty + 16 * u][l];
-#pragma unroll
-      for (int v = 0; v < NV; ++v) xv[v] = Xs[l][tx + 16 * v];
+      const float4 av = *reinterpret_cast<const float4*>(&As[l][4 * ty]);
+      const float4 xv = *reinterpret_cast<const float4*>(&Xs[l][4 * tx]);
+      const float ar[4] = {av.x, av.y, av.z, av.w}, xr[4] = {xv.x, xv.y, xv.z, xv.w};
 #pragma unroll
       for (int u = 0; u < 4; ++u)
 #pragma unroll
-        for (int v = 0; v < NV; ++v) acc[u][v] = fma(gv[u], xv[v], acc[u][v]);
+        for (int v = 0; v < 4; ++v) acc[u][v] = fmaf(ar[u], xr[v], acc[u][v]);
     }
   }
 #pragma unroll
-  for (int v = 0; v < NV; ++v) {
-    const int s = cells[tx + 16 * v];
-    if (s < 0) continue;
-    const double inv = scale_mul ? cscale[s] : 1.0 / cscale[s];
+  for (int u = 0; u < 4; ++u) {
+    const int gi = i0 + 4 * ty + u;
+    if (gi >= rows) continue;
+    double* y = Y + out_row(gi, n_Kr, rr, pdofs) * n_cells;
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int gi = i0 + ty + 16 * u;
-      if (gi < rows) Y[out_row(gi, n_Kr, rr, pdofs) * n_cells + s] = gi < n_Kr ? (double)acc[u][v] * inv
-                                                                            : (double)acc[u][v];
+    for (int v = 0; v < 4; ++v) {
+      const int s = cells[4 * tx + v];
+      if (s >= 0) y[s] = gi < n_Kr ? (double)acc[u][v] * fac[4 * tx + v] : (double)acc[u][v];
     }
   }
 }
@@ -1275,8 +1292,21 @@ int split_rows(const lat_ctx* h, int n_cells, int rows) {
   return std::max(1, std::min(want, (int)div_up(rows, 64)));
 }
 
-// cells per segmented-GEMM tile: 4 in FP64, 64 in the mixed modes
-int seg_bn(lat_ctx* h) { return h->prec == LAT_FP64 ? 4 : 64; }
+// cells per segmented-GEMM tile
+int seg_bn(lat_ctx* h) { return h->prec == LAT_FP64 ? 4 : kSegCells; }
+
+// FP32 segmented product of a view (n_Kr + n_P rows, n_Kc columns from the DOFs rc) of the key matrices
+void run_segmm32(lat_ctx* h, const float* G, int n_Kr, int n_Kc, int n_P, int ldg, int64_t kstride, int scale_mul,
+                 const int* rr, const int* rc, const double* X, double* Y) {
+  h->xf32.ensure((size_t)std::max(1, h->n_R) * h->n_cells);
+  if (n_Kc > 0)
+    LAT_LAUNCH(h, k_pack_f32<<<dim3(div_up(h->n_cells, 128), n_Kc), 128, 0, h->stream>>>(h->n_cells, n_Kc, rc, h->perm.p, X,
+                                                                                        h->xf32.p));
+  LAT_LAUNCH(h, k_local_segmm32<<<dim3(h->max_tiles, div_up(n_Kr + n_P, 64)), 128, 0, h->stream>>>(
+                    h->n_cells, n_Kr, n_Kc, n_P, ldg, kstride, scale_mul, G, h->tile_seg.p, h->tile_c0.p, h->seg_ptr.p,
+                    h->perm.p, h->c_cell.p, rr, h->pdofs.p, h->xf32.p, Y));
+  LAT_CHECK_LAUNCH();
+}
 
 int red_blocks(int64_t n) { return (int)std::min<int64_t>(kRed, std::max<int64_t>(1, (n + 255) / 256)); }
 int ew_blocks(lat_ctx* h, int64_t n) {
@@ -1697,13 +1727,12 @@ void kinv(lat_ctx* h, const double* v, double* w, KinvMode mode = KINV_FULL, con
     run_local_oz(h, v, wl, mode);
   } else {
     KernelTimer kt(h, tg_segmm[mode]);
-    dim3 grid(h->max_tiles, div_up(nKr + nP, 64));
     if (lo)
-      LAT_LAUNCH(h, k_local_segmm<float, 64><<<grid, 256, 0, h->stream>>>(ns, nKr, nKc, nP, nR, kstride, 0,
-          h->G32.p + off, h->tile_seg.p, h->tile_c0.p, h->seg_ptr.p, h->perm.p, h->c_cell.p, rr, rc, h->pdofs.p, v, wl));
+      run_segmm32(h, h->G32.p + off, nKr, nKc, nP, nR, kstride, 0, rr, rc, v, wl);
     else
-      LAT_LAUNCH(h, k_local_segmm_n4<<<grid, 256, 0, h->stream>>>(ns, nKr, nKc, nP, nR, kstride, 0, h->G.p + off,
-          h->tile_seg.p, h->tile_c0.p, h->seg_ptr.p, h->perm.p, h->c_cell.p, rr, rc, h->pdofs.p, v, wl));
+      LAT_LAUNCH(h, k_local_segmm_n4<<<dim3(h->max_tiles, div_up(nKr + nP, 64)), 256, 0, h->stream>>>(
+                        ns, nKr, nKc, nP, nR, kstride, 0, h->G.p + off, h->tile_seg.p, h->tile_c0.p, h->seg_ptr.p,
+                        h->perm.p, h->c_cell.p, rr, rc, h->pdofs.p, v, wl));
   }
   LAT_CHECK_LAUNCH();
   if (h->n_primal) {
@@ -1772,9 +1801,7 @@ void dual_precond_local(lat_ctx* h, const double* r, double* t1, double* t2) {
         LAT_LAUNCH(h, k_local_segmm_n4<<<grid, 256, 0, h->stream>>>(h->n_cells, nD, nD, 0, nD, (int64_t)nD * nD, 1,
             h->SDD.p, h->tile_seg.p, h->tile_c0.p, h->seg_ptr.p, h->perm.p, h->c_cell.p, rd, rd, h->pdofs.p, t1, t2));
       else
-        LAT_LAUNCH(h, k_local_segmm<float, 64><<<grid, 256, 0, h->stream>>>(h->n_cells, nD, nD, 0, nD,
-            (int64_t)nD * nD, 1, h->SDD32.p, h->tile_seg.p, h->tile_c0.p, h->seg_ptr.p, h->perm.p, h->c_cell.p, rd,
-            rd, h->pdofs.p, t1, t2));
+        run_segmm32(h, h->SDD32.p, nD, nD, 0, nD, (int64_t)nD * nD, 1, rd, rd, t1, t2);
     } else if (h->prec == LAT_FP64) {
       LAT_CUDA(cudaFuncSetAttribute(k_dual_schur<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm));
       LAT_LAUNCH(h, k_dual_schur<double><<<dim3(h->n_cells, split_rows(h, h->n_cells, nD)), 256, shm, h->stream>>>(h->n_cells, h->n_I, nD, h->SDD.p,

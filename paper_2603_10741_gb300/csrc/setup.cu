@@ -676,7 +676,7 @@ extern "C" lat_status lattice_destroy(lat_handle h) {
   rel(h->key_of_cell); rel(h->key_slot); rel(h->perm); rel(h->seg_ptr); rel(h->tile_seg);
   rel(h->tile_c0); rel(h->key_list); rel(h->solver_int); rel(h->delta_cell); rel(h->c_cell);
   rel(h->G); rel(h->G16[0]); rel(h->G16[1]); rel(h->G16[2]); rel(h->G16[3]); rel(h->cb_U32); rel(h->cb_Ut32); rel(h->cb_Dinv32); rel(h->tile_seg_tc); rel(h->tile_c0_tc); rel(h->tile_seg_oz); rel(h->tile_c0_oz); rel(h->oz_G); rel(h->oz_S); rel(h->oz_X); rel(h->oz_Gs); rel(h->oz_Ss); rel(h->oz_max); rel(h->sp_C); rel(h->sp_B); rel(h->sp_max); rel(h->sp_P); rel(h->sp_R); rel(h->Phi32); rel(h->SDD); rel(h->SDD32); rel(h->Phi); rel(h->Sloc); rel(h->G32); rel(h->Xb16); rel(h->KRP); rel(h->Coarse);
-  rel(h->CoarseInv); rel(h->CoarseInv32); rel(h->pcg_ws); rel(h->gP); rel(h->xP); rel(h->x32); rel(h->y32);
+  rel(h->CoarseInv); rel(h->CoarseInv32); rel(h->pcg_ws); rel(h->gP); rel(h->xP); rel(h->x32); rel(h->y32); rel(h->xf32);
   for (auto& b : h->kv_tmp) rel(b);
   rel(h->V); rel(h->Zk); rel(h->Hh); rel(h->gmres_small); rel(h->dots_part); rel(h->flag); rel(h->red_part);
   if (h->h_pinned) cudaFreeHost(h->h_pinned);

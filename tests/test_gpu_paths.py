@@ -216,3 +216,28 @@ def test_greedy_by_size(L, n_rows, n_cols, max_nr):
         assert s_got.cpu().numpy().tolist() == g.S.tolist()
         assert np.abs(a_got.cpu().numpy() - a_ref).max() <= 1e-9 * max(1.0, np.abs(a_ref).max())
     lat.close()
+
+
+@pytest.mark.parametrize("cell,dims", [
+    (latgen.ring_cell(8), (31, 9)),      # segments of 31 and 217 cells: tiles of 31 and 25, one tile less than full
+    (latgen.ring_cell(6), (8, 6)),       # 72 remaining DOFs: K chunks of 32, 32 and 8; 20 dual columns
+    (latgen.solid_cell(4, 2), (4, 16)),  # 32-row remainders: 50 rows of a 64-row tile
+])
+def test_fp32_segmented_product(L, cell, dims):
+    """K^-rom in the FP32 mode against the FP64 mode: FP32 blocks and sums on local problems of
+    condition below 1e3 (tolerance 1e-4 as for the BF16 pairs, which carry fewer bits)."""
+    case = _case(cell, dims)
+    outs = []
+    for prec in (0, 1):
+        lat = L.Lattice.from_case(case, prec)
+        u = lat.lattice_predictor(0.1 * case.top_displacement(1))
+        lat.select_principal_cells(u, 1e-3, 1)
+        lat.lattice_set_timing(True)
+        lat.lattice_prepare_solver(u, lat.lattice_default_opts(max_enrich=0, precond_tangent=1))
+        s = lat.sizes
+        v = lat.feti_from_global(torch.tensor(np.random.default_rng(7).uniform(-1, 1, s.n_dof), device="cuda"))
+        outs.append(lat.feti_apply(1, v)[: s.n_loc * s.n_cells + s.n_primal].cpu().numpy())
+        assert lat.lattice_kernel_time("local_segmm")[1] > 0
+        lat.close()
+    err = np.linalg.norm(outs[1] - outs[0]) / np.linalg.norm(outs[0])
+    assert err < 1e-4, err
