@@ -463,6 +463,7 @@ void gj_invert(lat_ctx* h, double* A, int n, int batch, int64_t bs, int neg_bit,
                double* snap = nullptr);
 void sweep_small(lat_ctx* h, double* A, int n, int batch, int64_t bs, int neg_bit);
 void run_sweep_panel(lat_ctx* h, double* A, int n, int batch, int64_t bs, int k0, int kw, int neg_bit);
+int sweep_panel_batch(int n);
 constexpr int kSweepPanel = 128;              // panel width of the large inversions
 constexpr int kSweepLarge = 384;              // matrices from this size on are swept in such panels
 void run_coarse_blocked(lat_ctx* h, const double* S, int64_t np, bool dense);

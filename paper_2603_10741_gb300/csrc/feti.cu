@@ -1387,13 +1387,24 @@ void sweep_small(lat_ctx* h, double* A, int n, int batch, int64_t bs, int neg_bi
 // us of update per 32 columns before, 102 us per 128 now).
 void gj_invert(lat_ctx* h, double* A, int n, int batch, int64_t bs, int neg_bit, int split,
                double* snap) {
+  const bool large = n >= kSweepLarge;
+  if (large) {
+    // the panels' workspace is several MB per matrix: no more matrices at a time than 2 GB of it
+    const int most = sweep_panel_batch(n);
+    if (batch > most) {
+      const int64_t m = n - std::max(split, 0);
+      for (int b = 0; b < batch; b += most)
+        gj_invert(h, A + (size_t)b * bs, n, std::min(most, batch - b), bs, neg_bit, split,
+                  snap ? snap + (size_t)b * m * m : nullptr);
+      return;
+    }
+  }
   auto snapshot = [&](int at) {
     const int64_t m = n - at;
     LAT_LAUNCH(h, k_gj_snapshot<<<dim3(div_up(m * m, 256), batch), 256, 0, h->stream>>>(n, bs, at, A, snap));
     LAT_CHECK_LAUNCH();
   };
   if (snap && split == 0) snapshot(0);
-  const bool large = n >= kSweepLarge;
   for (int k0 = 0; k0 < n;) {
     int kw = std::min(large ? kSweepPanel : GJB, n - k0);
     if (split > 0 && k0 < split) kw = std::min(kw, split - k0);
@@ -1848,7 +1859,7 @@ bool capture_pcg_loop(lat_ctx* h, Body&& body) {
     h->stream = h->cap_stream;
     try {
       body(loop, kPcgLoop);
-    } catch (const LatError&) {
+    } catch (...) {
       ok = false;
     }
     h->stream = user;

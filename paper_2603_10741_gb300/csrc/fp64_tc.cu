@@ -455,13 +455,18 @@ void product(lat_ctx* h, const OzShape& sh, int mt0, int kp0, const DBuf<__nv_bf
 // bytes per entry and the launches that split the cell vectors cost less than the FP64 pipe does
 // (36 cells of the strut cell's
 // dual block 50 us against 406, 512 cells of the whole block 0.40 ms against 6.0; the ring cells' dual
-// block is 56 columns, under 10 us either way), no more columns than the largest cluster sums exactly, and digits within 24 GB.
+// block is 56 columns, under 10 us either way), no more columns than the largest cluster sums exactly, and digits
+// within 24 GB and a quarter of the free memory.
 bool oz_wanted(const lat_ctx* h) {
   if (h->prec != LAT_FP64 || (int64_t)h->n_keys * 8 > h->n_cells) return false;
   const OzShape g = g_shape(h), s = s_shape(h);
   if (h->n_R - h->n_I < 512 || g.KP > MAX_SPLIT * MAX_PANELS) return false;
-  const double bytes = 2.0 * h->n_keys * A_ELEMS * ((double)g.MT * g.KP + (double)s.MT * s.KP);
-  return bytes <= 24e9;
+  const double nG = (double)h->n_keys * A_ELEMS * g.MT * g.KP, nS = (double)h->n_keys * A_ELEMS * s.MT * s.KP;
+  if (2 * (nG + nS) > 24e9) return false;
+  if ((double)h->oz_G.n >= nG && (double)h->oz_S.n >= nS) return true;
+  // room for them beside what the Krylov solves will still allocate
+  size_t free_b = 0, total_b = 0;
+  return cudaMemGetInfo(&free_b, &total_b) == cudaSuccess && 2 * (nG + nS) <= 0.25 * (double)free_b;
 }
 
 // digits of the augmented local matrices and of the dual Schur complements (after the inversions)
@@ -712,6 +717,13 @@ __global__ void __launch_bounds__(128, 2)
 }
 
 }  // namespace
+
+// matrices of one size whose panels' workspace (run_sweep_panel) stays within 2 GB
+int sweep_panel_batch(int n) {
+  const double per = 2.0 * div_up(n, TM) * SP * A_ELEMS + 2.0 * (div_up(n, SN) + SW / SN) * SP * SB_ELEMS +
+                     8.0 * n * SW + 8.0 * SW * SW;
+  return std::max(1, (int)(2e9 / per));
+}
 
 // one panel [k0, k0 + kw) of the sweep of `batch` n x n matrices (lower triangles)
 void run_sweep_panel(lat_ctx* h, double* A, int n, int batch, int64_t bs, int k0, int kw, int neg_bit) {
