@@ -1120,14 +1120,15 @@ __global__ void __launch_bounds__(256)
 // Dirichlet primal DOF); rows n_K.. of the grid clear the corner rows (their values went to g_P).
 // A CTA owns 32 consecutive cells and kPhiRows rows: it gathers the cells' corner values (kPhiCols
 // at a time: 8 or 24 without enrichment, hundreds with a deep one) into shared memory ([j][cell],
-// conflict free), then every warp takes its two rows together with a lane per cell, so that a row's read-modify-write is one coalesced 256-byte segment, both
-// in flight, and the Phi row is a broadcast VEC-wide load (cells of a layer share their key).
+// conflict free), then every warp takes its two rows together with a lane per cell, so that a row's
+// read-modify-write is one coalesced 256-byte segment, both in flight, and the Phi row is a
+// broadcast VEC-wide load (cells of a layer share their key).
 // Bound by the 17 bytes per entry of Y and its mask.  The form before (a thread per cell walking
 // 32 rows one after the other, corner values gathered by a launch of its own) was a chain of
 // dependent loads: 72 us per launch on the 10^3 strut lattice and 44 us on 16 ring cells, where it
 // was 30 % of a load step.  16 rows per CTA: 10^3 strut solve (BF16) 520 ms, 36-cell strut solve (FP64)
-// 265, against 536 and 278 with 32 rows and 544 and 262 with 8.  T = FP32 in the mixed modes (an FP32 copy of Phi, part of their FP32
-// preconditioner).
+// 265, against 536 and 278 with 32 rows and 544 and 262 with 8.  T = FP32 in the mixed modes (an FP32
+// copy of Phi, part of their FP32 preconditioner).
 constexpr int kPhiRows = 16, kPhiCols = 96;
 
 template <typename T, int VEC>

@@ -435,17 +435,17 @@ void build_feti_impl(lat_ctx* h, int level) {
   h->n_lambda = (int64_t)lp.size();
   h->lam_p.upload(lp, h->stream);
   h->lam_m.upload(lm, h->stream);
-  std::vector<double> lsc_l(pairs.size());
-  for (size_t l = 0; l < pairs.size(); ++l) lsc_l[l] = 1.0 / mult[pairs[l].first];
-  h->lam_scale.upload(lsc_l, h->stream);
   std::vector<int> de, d1, d2;
-  std::vector<double> dsc;
+  std::vector<double> dsc, lsc_l(lp.size());
   for (auto& kv : dual) {
     de.push_back(kv.first);
     d1.push_back(kv.second.first);
     d2.push_back(kv.second.second);
     dsc.push_back(dscale[kv.first]);
+    lsc_l[std::abs(kv.second.first) - 1] = dsc.back();
+    if (kv.second.second) lsc_l[std::abs(kv.second.second) - 1] = dsc.back();
   }
+  h->lam_scale.upload(lsc_l, h->stream);
   h->n_dual = (int64_t)de.size();
   // per (dual DOF position, cell) the signed multipliers of the copy and its scale: the
   // interface products of the tensor-core path read B^T lambda from it directly
