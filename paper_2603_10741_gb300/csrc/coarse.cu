@@ -584,7 +584,7 @@ __global__ void __launch_bounds__(kCoopThreads, 1)
     __syncthreads();
     if (nr > 0 && !coop_wait(bar0 + 8 * (k & 1), (uint32_t)((k >> 1) & 1))) {
       late[k & 1] = true;
-      if (threadIdx.x == 0) atomicOr(err, 8);
+      if (threadIdx.x == 0) atomicOr(err, kFlagCopyWait);
     }
     const T* Mb = buf + (k & 1) * bstride;
     for (int lr = warp; lr < nr; lr += nwarp_cta) {
@@ -683,12 +683,12 @@ void run_coarse_blocked(lat_ctx* h, const double* S, int64_t np, bool dense) {
   if (!dense) {
     // forward recurrence only: D_i^{-1} in place, U_{i-1} = D_{i-1}^{-1} B_{i-1}
     cpy(blk(DE, 0), blk(A, 0));
-    gj_invert(h, DE, m, 1, (int64_t)mm, 8);
+    gj_invert(h, DE, m, 1, (int64_t)mm, kFlagCoarseNegative);
     for (int i = 1; i < N; ++i) {
       bgemm<false, false>(h, m, {blk(DE, i - 1)}, {blk(Bk, i - 1)}, {blk(U, i - 1)}, 1.0, 0.0);
       cpy(blk(DE, i), blk(A, i));
       bgemm<false, false>(h, m, {blk(Bt, i - 1)}, {blk(U, i - 1)}, {blk(DE, i)}, -1.0, 1.0);
-      gj_invert(h, blk(DE, i), m, 1, (int64_t)mm, 8);
+      gj_invert(h, blk(DE, i), m, 1, (int64_t)mm, kFlagCoarseNegative);
     }
     // U_i^T for the forward sweep, and the sweep buffers
     h->cb_Ut.ensure((size_t)N1 * mm);
@@ -719,7 +719,7 @@ void run_coarse_blocked(lat_ctx* h, const double* S, int64_t np, bool dense) {
   cpy(xb(0, 0), blk(A, 0));
   cpy(blk(DE, 0), blk(A, 0));
   cpy(erev(0), blk(A, N - 1));
-  gj_invert(h, DE, m, 2, half, 8);
+  gj_invert(h, DE, m, 2, half, kFlagCoarseNegative);
   // step k: forward i = k and backward e = N-1-k, each pair in one batched launch
   for (int k = 1; k < N; ++k) {
     const int i = k, e = N - 1 - k;
@@ -729,7 +729,7 @@ void run_coarse_blocked(lat_ctx* h, const double* S, int64_t np, bool dense) {
     cpy(erev(k), blk(A, e));
     bgemm<false, false>(h, m, {blk(Bt, i - 1), blk(Bk, e)}, {blk(U, i - 1), blk(T, e)}, {xb(i, i), erev(k)}, -1.0, 1.0);
     cpy(blk(DE, i), xb(i, i));
-    gj_invert(h, blk(DE, k), m, 2, half, 8);
+    gj_invert(h, blk(DE, k), m, 2, half, kFlagCoarseNegative);
   }
   // X_ii <- D_i - B_i E_{i+1}^{-1} B_i^T, then the diagonal blocks of the inverse
   if (N > 1) {
@@ -742,7 +742,7 @@ void run_coarse_blocked(lat_ctx* h, const double* S, int64_t np, bool dense) {
     }
     bgemm<false, false>(h, m, a, b, c, -1.0, 1.0);
   }
-  gj_invert(h, X, m, N, (int64_t)(N + 1) * mm, 8);
+  gj_invert(h, X, m, N, (int64_t)(N + 1) * mm, kFlagCoarseNegative);
   // upper blocks, wave by wave in d = j - i:  X_ij = U_i X_{i+1,j} = -(D_i^-1 B_i) X_{i+1,j}
   for (int d = 1; d < N; ++d) {
     std::vector<const double*> a, b;

@@ -292,6 +292,16 @@ static lat_status guard(lat_ctx* h, F&& f) {
   }
 }
 
+// Bits of the handle's flag word.  The setup reads and clears the pivot bits, so that a solve that
+// looks at the word sees its own waits alone.
+enum {
+  kFlagSingular = 1,       // a zero or non-finite pivot
+  kFlagLocalNegative = 2,  // a principal's remaining block has a negative pivot
+  kFlagProductWait = 4,    // a wait of a tensor-core product gave up
+  kFlagCoarseNegative = 8, // the coarse matrix has a negative pivot
+  kFlagCopyWait = 16       // a block-row copy of the cooperative coarse solve did not land
+};
+
 // element colours passed by value to the per-cell kernels
 struct ColorTable {
   int n;

@@ -591,7 +591,7 @@ __device__ void sweep_pivot(int kw, double (&M)[GJB][GJB + 1], double (&col)[2][
   }
   auto check = [&](double piv) {
     if (t != 0 || !flag) return;
-    if (!(fabs(piv) > 0.0) || !isfinite(piv)) atomicOr(flag, 1);
+    if (!(fabs(piv) > 0.0) || !isfinite(piv)) atomicOr(flag, kFlagSingular);
     else if (piv < 0.0) atomicOr(flag, neg_bit);
   };
   if (t < 32) {
@@ -1545,7 +1545,7 @@ void run_prepare_solver(lat_ctx* h, const lat_newton_opts* o, const double* u_gl
   }
   const int nD = nR - h->n_I;
   h->SDD.ensure((size_t)nk * nD * nD);
-  gj_invert(h, h->G.p, nR, nk, gstride, 2, h->n_I, h->SDD.p);
+  gj_invert(h, h->G.p, nR, nk, gstride, kFlagLocalNegative, h->n_I, h->SDD.p);
   h->iface = o ? o->interface_precond : 0;
   {
     KernelTimer kt(h, "phi_schur");
@@ -1589,16 +1589,17 @@ void run_prepare_solver(lat_ctx* h, const lat_newton_opts* o, const double* u_gl
       LAT_LAUNCH(h, k_coarse<<<div_up(n_ent, 256), 256, 0, h->stream>>>(n_ent, np, nP, h->coarse_row.p,
           h->coarse_col.p, h->coarse_ptr.p, h->coarse_src.p, h->key_slot.p, h->c_cell.p, h->Sloc.p, h->CoarseInv.p));
       LAT_CHECK_LAUNCH();
-      gj_invert(h, h->CoarseInv.p, (int)np, 1, np * np, 8);
+      gj_invert(h, h->CoarseInv.p, (int)np, 1, np * np, kFlagCoarseNegative);
     }
   }
   int fl = 0;
   LAT_CUDA(cudaMemcpyAsync(&fl, h->flag.p, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
+  LAT_CUDA(cudaMemsetAsync(h->flag.p, 0, sizeof(int), h->stream));
   LAT_CUDA(cudaStreamSynchronize(h->stream));
-  LAT_REQUIRE(!(fl & 4), LAT_ETIMEOUT, "a tensor-core wait in a local inversion gave up");
-  LAT_REQUIRE(!(fl & 1), LAT_EINDEFINITE, "a local remaining-DOF matrix or the coarse matrix is singular");
-  h->indefinite = (fl & 2) != 0;          // a principal's remaining block has a negative pivot
-  h->coarse_indefinite = (fl & 8) != 0;   // the coarse matrix has a negative pivot
+  LAT_REQUIRE(!(fl & kFlagProductWait), LAT_ETIMEOUT, "a tensor-core wait in a local inversion gave up");
+  LAT_REQUIRE(!(fl & kFlagSingular), LAT_EINDEFINITE, "a local remaining-DOF matrix or the coarse matrix is singular");
+  h->indefinite = (fl & kFlagLocalNegative) != 0;
+  h->coarse_indefinite = (fl & kFlagCoarseNegative) != 0;
   if (h->oz) run_oz_split(h);
   if (h->prec == LAT_MIXED_BF16) run_g_to_bf16(h, gsz);
   if (h->prec != LAT_FP64) {
@@ -2137,8 +2138,8 @@ int run_fgmres(lat_ctx* h, const double* b, double* x, const lat_newton_opts* o,
     int fl = 0;
     LAT_CUDA(cudaMemcpyAsync(&fl, h->flag.p, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
     LAT_CUDA(cudaStreamSynchronize(h->stream));
-    LAT_REQUIRE(!(fl & 4), LAT_ETIMEOUT, "a tensor-core wait in the local product gave up");
-    LAT_REQUIRE(!(fl & 8), LAT_ETIMEOUT, "a block-row copy of the cooperative coarse solve did not land");
+    LAT_REQUIRE(!(fl & kFlagProductWait), LAT_ETIMEOUT, "a tensor-core wait in the local product gave up");
+    LAT_REQUIRE(!(fl & kFlagCopyWait), LAT_ETIMEOUT, "a block-row copy of the cooperative coarse solve did not land");
   }
   return total;
 }

@@ -339,7 +339,7 @@ __global__ void __launch_bounds__(128, 2)
   __syncthreads();
   const bool good = !fail;   // accumulators complete, every wait met
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  if (!good && tid == 0) atomicOr(err, 4);
+  if (!good && tid == 0) atomicOr(err, kFlagProductWait);
   // digit sums of the tile's row (this thread's) and each cell to one FP64 value, in shared memory
   double* part = reinterpret_cast<double*>(smem);   // [cell][129]
   if (good) {
@@ -676,7 +676,7 @@ __global__ void __launch_bounds__(128, 2)
   __syncthreads();
   const bool good = !fail;
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  if (!good && tid == 0) atomicOr(err, 4);
+  if (!good && tid == 0) atomicOr(err, kFlagProductWait);
   if (good) {
     const uint32_t base = tmem + ((uint32_t)(warp * 32) << 16);
     const int gi = mt * TM + tid, j0 = nt * SN;

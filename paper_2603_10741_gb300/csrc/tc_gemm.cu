@@ -201,7 +201,7 @@ __global__ void __launch_bounds__(128, 2)
   __syncthreads();
   const bool good = !fail;   // accumulators complete, every wait met
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  if (!good && tid == 0) atomicOr(err, 4);
+  if (!good && tid == 0) atomicOr(err, kFlagProductWait);
   // accumulators to shared memory (the stages are idle), [column][row] with a row of 129 floats:
   // warp w holds accumulator lanes 32w..32w+31 (tile rows)
   float* part = reinterpret_cast<float*>(smem);
