@@ -231,6 +231,7 @@ struct lat_ctx {
   int64_t pcg_its_total = 0;            // interface PCG iterations since the last reset
   int64_t n_launch = 0;                 // kernels launched through this handle
   int iface = 0;                        // interface preconditioner: 0 Dirichlet, 1 lumped
+  int wait_polls = 1 << 20;             // polls before a wait of a tensor-core product gives up
   bool verbose = false;                 // LATTICE_VERBOSE=1: per-iteration log on stderr
   double *h_pinned = nullptr;          // small pinned host scratch
 

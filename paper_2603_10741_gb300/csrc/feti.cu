@@ -2102,6 +2102,18 @@ int fgmres_core(lat_ctx* h, const GmresLevel& L, const double* b, double* x, boo
 
 }  // namespace
 
+// Reports a bounded device-side wait that gave up since the last check: the products of such a launch
+// are not written.  The word is cleared, so that one expired wait does not fail every later call.
+void check_waits(lat_ctx* h) {
+  if (h->prec != LAT_MIXED_BF16 && !h->oz && !(h->cb_solve && h->cb_wide && h->cb_coop_grid > 0)) return;
+  int fl = 0;
+  LAT_CUDA(cudaMemcpyAsync(&fl, h->flag.p, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
+  LAT_CUDA(cudaStreamSynchronize(h->stream));
+  if (fl) LAT_CUDA(cudaMemsetAsync(h->flag.p, 0, sizeof(int), h->stream));
+  LAT_REQUIRE(!(fl & kFlagProductWait), LAT_ETIMEOUT, "a tensor-core wait in the local product gave up");
+  LAT_REQUIRE(!(fl & kFlagCopyWait), LAT_ETIMEOUT, "a block-row copy of the cooperative coarse solve did not land");
+}
+
 // FGMRES on the saddle-point system (Section 3.3.1) with the FP64 reduced tangent action.  Its
 // preconditioner is the block preconditioner of Eq. (ifetidp_precond), or, in the mixed modes
 // with inner_its > 0, an inner flexible GMRES whose operator is the FP32 reduced tangent action
@@ -2134,13 +2146,7 @@ int run_fgmres(lat_ctx* h, const double* b, double* x, const lat_newton_opts* o,
     total = fgmres_core(h, outer, b, x, false, o->krylov_rtol, o->krylov_max_it, o->krylov_restart, false, block,
                         rel_out);
   }
-  if (h->prec == LAT_MIXED_BF16 || h->oz || (h->cb_solve && h->cb_wide && h->cb_coop_grid > 0)) {
-    int fl = 0;
-    LAT_CUDA(cudaMemcpyAsync(&fl, h->flag.p, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
-    LAT_CUDA(cudaStreamSynchronize(h->stream));
-    LAT_REQUIRE(!(fl & kFlagProductWait), LAT_ETIMEOUT, "a tensor-core wait in the local product gave up");
-    LAT_REQUIRE(!(fl & kFlagCopyWait), LAT_ETIMEOUT, "a block-row copy of the cooperative coarse solve did not land");
-  }
+  check_waits(h);
   return total;
 }
 
@@ -2378,6 +2384,15 @@ extern "C" lat_status lattice_prepare_solver(lat_handle h, const double* u, cons
   return guard(h, [&] {
     check_opts(o);
     prepare_enriched(h, o, u);
+  });
+}
+
+extern "C" lat_status lattice_set_wait_limit(lat_handle h, int32_t polls) {
+  if (!h) return LAT_EINVAL;
+  return guard(h, [&] {
+    LAT_REQUIRE(polls >= 0, LAT_EINVAL, "polls must not be negative");
+    drop_pcg_graph(h);   // its launches carry the limit
+    h->wait_polls = polls;
   });
 }
 

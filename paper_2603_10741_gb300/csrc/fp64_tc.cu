@@ -246,11 +246,12 @@ __global__ void __launch_bounds__(128, 2)
             const unsigned long long* __restrict__ cmax, const int* __restrict__ tile_seg,
             const int* __restrict__ tile_c0, const int* __restrict__ seg_ptr, const int* __restrict__ perm,
             const double* __restrict__ cscale, int n_R, int r_base, const int* __restrict__ rdofs,
-            const int* __restrict__ pdofs, double* __restrict__ Y, int* __restrict__ err, int mul_scale) {
+            const int* __restrict__ pdofs, double* __restrict__ Y, int* __restrict__ err, int mul_scale,
+            int polls) {
   extern __shared__ __align__(1024) unsigned char smem[];
   __shared__ __align__(8) uint64_t full[STAGES], empty[STAGES], done;
   __shared__ uint32_t tmem_slot;
-  __shared__ int fail;
+  __shared__ int fail, issued;   // a wait gave up; panels whose copies were issued
   __shared__ int cell[NC];
   __shared__ double cs1[NC], cs2[NC];      // factor of a column's scaled rows, and of its corner rows
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -278,11 +279,11 @@ __global__ void __launch_bounds__(128, 2)
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = tmem_slot;
   if (tid == 0) {
-    int issued = 0;
+    int n = 0;
     bool ok = true;
     for (int p = 0; p < np; ++p) {
       const int st = p % STAGES;
-      if (p >= STAGES && !mbar_wait(smem_u32(&empty[st]), (uint32_t)((p / STAGES - 1) & 1))) {
+      if (p >= STAGES && !mbar_wait(smem_u32(&empty[st]), (uint32_t)((p / STAGES - 1) & 1), polls)) {
         ok = false;
         break;
       }
@@ -290,19 +291,15 @@ __global__ void __launch_bounds__(128, 2)
       expect_tx(bar, (uint32_t)STAGE_BYTES);
       bulk_copy(dst, GT + (((size_t)key * sh.MT + mt) * sh.KP + kp0 + p0 + p) * A_ELEMS, 2 * A_ELEMS, bar);
       bulk_copy(dst + 2 * A_ELEMS, XT + ((size_t)tile * npan + p0 + p) * B_ELEMS, 2 * B_ELEMS, bar);
-      ++issued;
+      ++n;
     }
-    if (!ok) {
-      fail = 1;
-      // let copies in flight land (bounded) before the shared memory is released
-      for (int q = max(0, issued - STAGES); q < issued; ++q)
-        mbar_wait(smem_u32(&full[q % STAGES]), (uint32_t)((q / STAGES) & 1));
-    }
+    if (!ok) fail = 1;
+    issued = n;
   } else if (tid == 32) {
     bool ok = true;
     for (int p = 0; p < np; ++p) {
       const int st = p % STAGES;
-      if (!mbar_wait(smem_u32(&full[st]), (uint32_t)((p / STAGES) & 1))) {
+      if (!mbar_wait(smem_u32(&full[st]), (uint32_t)((p / STAGES) & 1), polls)) {
         ok = false;
         break;
       }
@@ -339,7 +336,13 @@ __global__ void __launch_bounds__(128, 2)
   __syncthreads();
   const bool good = !fail;   // accumulators complete, every wait met
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  if (!good && tid == 0) atomicOr(err, kFlagProductWait);
+  if (!good && tid == 0) {
+    atomicOr(err, kFlagProductWait);
+    // copies in flight land (bounded) before the shared memory is released
+    for (int q = max(0, issued - STAGES); q < issued; ++q)
+      mbar_wait(smem_u32(&full[q % STAGES]), (uint32_t)((q / STAGES) & 1));
+  }
+  __syncwarp();
   // digit sums of the tile's row (this thread's) and each cell to one FP64 value, in shared memory
   double* part = reinterpret_cast<double*>(smem);   // [cell][129]
   if (good) {
@@ -445,7 +448,7 @@ void product(lat_ctx* h, const OzShape& sh, int mt0, int kp0, const DBuf<__nv_bf
                                             (const __nv_bfloat16*)h->oz_X.p, (const unsigned long long*)h->oz_max.p, ts,
                                             tc, (const int*)h->seg_ptr.p, (const int*)h->perm.p,
                                             (const double*)h->c_cell.p, n_R, r_base, rdofs, (const int*)h->pdofs.p, Y,
-                                            h->flag.p, mul_scale)));
+                                            h->flag.p, mul_scale, h->wait_polls)));
   LAT_CHECK_LAUNCH();
 }
 
@@ -582,11 +585,11 @@ __global__ void __launch_bounds__(128, 2)
     k_sp_mm(int n, int64_t bs, int k0, int kw, int MT, int NT, const __nv_bfloat16* __restrict__ Cd,
             const unsigned long long* __restrict__ cmax, const __nv_bfloat16* __restrict__ Bd,
             const unsigned long long* __restrict__ bmax, const double* __restrict__ P, double* __restrict__ R,
-            double* __restrict__ A, int* __restrict__ err) {
+            double* __restrict__ A, int* __restrict__ err, int polls) {
   extern __shared__ __align__(1024) unsigned char smem[];
   __shared__ __align__(8) uint64_t full[SSTAGES], empty[SSTAGES], done;
   __shared__ uint32_t tmem_slot;
-  __shared__ int fail;
+  __shared__ int fail, issued;   // a wait gave up; panels whose copies were issued
   __shared__ double cs[SN];
   const int tid = threadIdx.x, warp = tid >> 5, b = blockIdx.y;
   int mt, nt;
@@ -622,11 +625,11 @@ __global__ void __launch_bounds__(128, 2)
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = tmem_slot;
   if (tid == 0) {
-    int issued = 0;
+    int n = 0;
     bool ok = true;
     for (int p = 0; p < np; ++p) {
       const int st = p % SSTAGES;
-      if (p >= SSTAGES && !mbar_wait(smem_u32(&empty[st]), (uint32_t)((p / SSTAGES - 1) & 1))) {
+      if (p >= SSTAGES && !mbar_wait(smem_u32(&empty[st]), (uint32_t)((p / SSTAGES - 1) & 1), polls)) {
         ok = false;
         break;
       }
@@ -634,18 +637,15 @@ __global__ void __launch_bounds__(128, 2)
       expect_tx(bar, (uint32_t)SSTAGE_BYTES);
       bulk_copy(dst, Cd + (((size_t)b * MT + mt) * SP + p) * A_ELEMS, 2 * A_ELEMS, bar);
       bulk_copy(dst + 2 * A_ELEMS, Bd + (((size_t)b * NT + nt) * SP + p) * SB_ELEMS, 2 * SB_ELEMS, bar);
-      ++issued;
+      ++n;
     }
-    if (!ok) {
-      fail = 1;
-      for (int q = max(0, issued - SSTAGES); q < issued; ++q)
-        mbar_wait(smem_u32(&full[q % SSTAGES]), (uint32_t)((q / SSTAGES) & 1));
-    }
+    if (!ok) fail = 1;
+    issued = n;
   } else if (tid == 32) {
     bool ok = true;
     for (int p = 0; p < np; ++p) {
       const int st = p % SSTAGES;
-      if (!mbar_wait(smem_u32(&full[st]), (uint32_t)((p / SSTAGES) & 1))) {
+      if (!mbar_wait(smem_u32(&full[st]), (uint32_t)((p / SSTAGES) & 1), polls)) {
         ok = false;
         break;
       }
@@ -676,7 +676,13 @@ __global__ void __launch_bounds__(128, 2)
   __syncthreads();
   const bool good = !fail;
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  if (!good && tid == 0) atomicOr(err, kFlagProductWait);
+  if (!good && tid == 0) {
+    atomicOr(err, kFlagProductWait);
+    // copies in flight land (bounded) before the shared memory is released
+    for (int q = max(0, issued - SSTAGES); q < issued; ++q)
+      mbar_wait(smem_u32(&full[q % SSTAGES]), (uint32_t)((q / SSTAGES) & 1));
+  }
+  __syncwarp();
   if (good) {
     const uint32_t base = tmem + ((uint32_t)(warp * 32) << 16);
     const int gi = mt * TM + tid, j0 = nt * SN;
@@ -747,10 +753,11 @@ void run_sweep_panel(lat_ctx* h, double* A, int n, int batch, int64_t bs, int k0
   LAT_LAUNCH(h, k_sp_rows<<<dim3(SW / 8, batch), 256, 0, h->stream>>>(kw, kw, (int64_t)SW * SW, kw, PT, h->sp_P.p, Pd,
                                                                       pmax));
   LAT_LAUNCH(h, k_sp_mm<false><<<dim3(MT * PT, batch), 128, shm, h->stream>>>(n, bs, k0, kw, MT, PT, h->sp_C.p, cmax, Pd,
-                                                                              pmax, h->sp_P.p, h->sp_R.p, A, h->flag.p));
+                                                                              pmax, h->sp_P.p, h->sp_R.p, A, h->flag.p,
+                                                                              h->wait_polls));
   LAT_LAUNCH(h, k_sp_rows<<<dim3(NT * SN / 8, batch), 256, 0, h->stream>>>(n, SW, (int64_t)n * SW, kw, NT, h->sp_R.p, Rd,
                                                                           rmax));
   LAT_LAUNCH(h, k_sp_mm<true><<<dim3(2 * MT * (MT + 1), batch), 128, shm, h->stream>>>(
-                    n, bs, k0, kw, MT, NT, h->sp_C.p, cmax, Rd, rmax, h->sp_P.p, h->sp_R.p, A, h->flag.p));
+                    n, bs, k0, kw, MT, NT, h->sp_C.p, cmax, Rd, rmax, h->sp_P.p, h->sp_R.p, A, h->flag.p, h->wait_polls));
   LAT_CHECK_LAUNCH();
 }

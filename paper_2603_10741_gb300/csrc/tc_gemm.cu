@@ -92,13 +92,13 @@ __global__ void __launch_bounds__(128, 2)
                const __nv_bfloat16* __restrict__ XT, const int* __restrict__ tile_seg,
                const int* __restrict__ tile_c0, const int* __restrict__ seg_ptr, const int* __restrict__ perm,
                const double* __restrict__ cscale, const int* __restrict__ rr, const int* __restrict__ pdofs,
-               double* __restrict__ Y, int* __restrict__ err, int mul_scale, int S) {
+               double* __restrict__ Y, int* __restrict__ err, int mul_scale, int S, int polls) {
   using C = TcCfg<TN>;
   constexpr int STAGES = C::STAGES;
   extern __shared__ __align__(1024) unsigned char smem[];
   __shared__ __align__(8) uint64_t full[STAGES], empty[STAGES], done;
   __shared__ uint32_t tmem_slot;
-  __shared__ int fail;
+  __shared__ int fail, issued;   // a wait gave up; panels whose copies were issued
   __shared__ int cell[TN], orow[TM];       // cell of a column (-1: past the segment), local row of a tile row
   __shared__ double fac[TN];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -129,11 +129,11 @@ __global__ void __launch_bounds__(128, 2)
 
   if (tid == 0) {
     // producer: panel p goes to stage p % STAGES once that stage's previous MMAs have read it
-    int issued = 0;
+    int n = 0;
     bool ok = true;
     for (int p = 0; p < np; ++p) {
       const int st = p % STAGES;
-      if (p >= STAGES && !mbar_wait(smem_u32(&empty[st]), (uint32_t)((p / STAGES - 1) & 1))) {
+      if (p >= STAGES && !mbar_wait(smem_u32(&empty[st]), (uint32_t)((p / STAGES - 1) & 1), polls)) {
         ok = false;
         break;
       }
@@ -141,19 +141,15 @@ __global__ void __launch_bounds__(128, 2)
       expect_tx(bar, (uint32_t)C::STAGE_BYTES);
       bulk_copy(dst, GT + (((size_t)key * MT + mt) * KP + p0 + p) * 2 * A_ELEMS, 2 * A_BYTES, bar);
       bulk_copy(dst + 2 * A_BYTES, XT + ((size_t)tile * KP + p0 + p) * 2 * C::B_ELEMS, 2 * C::B_BYTES, bar);
-      ++issued;
+      ++n;
     }
-    if (!ok) {
-      fail = 1;
-      // let copies in flight land (bounded) before the shared memory is released
-      for (int q = max(0, issued - STAGES); q < issued; ++q)
-        mbar_wait(smem_u32(&full[q % STAGES]), (uint32_t)((q / STAGES) & 1));
-    }
+    if (!ok) fail = 1;
+    issued = n;
   } else if (tid == 32) {
     bool ok = true;
     for (int p = 0; p < np; ++p) {
       const int st = p % STAGES;
-      if (!mbar_wait(smem_u32(&full[st]), (uint32_t)((p / STAGES) & 1))) {
+      if (!mbar_wait(smem_u32(&full[st]), (uint32_t)((p / STAGES) & 1), polls)) {
         ok = false;
         break;
       }
@@ -201,7 +197,13 @@ __global__ void __launch_bounds__(128, 2)
   __syncthreads();
   const bool good = !fail;   // accumulators complete, every wait met
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  if (!good && tid == 0) atomicOr(err, kFlagProductWait);
+  if (!good && tid == 0) {
+    atomicOr(err, kFlagProductWait);
+    // copies in flight land (bounded) before the shared memory is released
+    for (int q = max(0, issued - STAGES); q < issued; ++q)
+      mbar_wait(smem_u32(&full[q % STAGES]), (uint32_t)((q / STAGES) & 1));
+  }
+  __syncwarp();
   // accumulators to shared memory (the stages are idle), [column][row] with a row of 129 floats:
   // warp w holds accumulator lanes 32w..32w+31 (tile rows)
   float* part = reinterpret_cast<float*>(smem);
@@ -435,7 +437,7 @@ void launch_tc(lat_ctx* h, int n_Kr, int n_P, int MT, int KP, const __nv_bfloat1
                                             (const __nv_bfloat16*)h->Xb16.p, (const int*)h->tile_seg_tc.p,
                                             (const int*)h->tile_c0_tc.p, (const int*)h->seg_ptr.p,
                                             (const int*)h->perm.p, (const double*)h->c_cell.p, rr,
-                                            (const int*)h->pdofs.p, Y, h->flag.p, mul_scale, S)));
+                                            (const int*)h->pdofs.p, Y, h->flag.p, mul_scale, S, h->wait_polls)));
   LAT_CHECK_LAUNCH();
 }
 

@@ -9,8 +9,12 @@ __device__ __forceinline__ uint32_t smem_u32(const void* p) {
   return static_cast<uint32_t>(__cvta_generic_to_shared(p));
 }
 
-__device__ __forceinline__ bool mbar_wait(uint32_t addr, uint32_t parity) {
-  for (int i = 0; i < (1 << 20); ++i) {
+// Waits of a pipeline take the handle's limit (lattice_set_wait_limit); the waits for what is already
+// in flight, which a kernel that gives up still makes, keep this one.
+constexpr int kWaitPolls = 1 << 20;
+
+__device__ __forceinline__ bool mbar_wait(uint32_t addr, uint32_t parity, int polls = kWaitPolls) {
+  for (int i = 0; i < polls; ++i) {
     uint32_t done;
     asm volatile(
         "{\n\t.reg .pred p;\n\t"

@@ -25,7 +25,8 @@ EXPORTS = ["lattice_setup", "lattice_destroy", "lattice_sizes", "lattice_last_er
            "lattice_default_opts",
            "newton_step", "adjoint_gradient", "feti_apply", "lattice_prepare_solver", "feti_to_global",
            "feti_from_global", "lattice_checkpoint_save", "lattice_checkpoint_load", "tangent_solve",
-           "lattice_set_timing", "lattice_kernel_time", "lattice_launch_count", "greedy_select_static"]
+           "lattice_set_timing", "lattice_kernel_time", "lattice_launch_count", "lattice_set_wait_limit",
+           "greedy_select_static"]
 
 
 class LatticeError(RuntimeError):
@@ -99,6 +100,7 @@ def load_library(path: str = LIB_PATH):
         "feti_apply": [P, I32, P, P],
         "tangent_solve": [P, P, P, C.POINTER(NewtonOpts), P, P],
         "lattice_prepare_solver": [P, P, C.POINTER(NewtonOpts)],
+        "lattice_set_wait_limit": [P, I32],
         "feti_to_global": [P, P, P],
         "feti_from_global": [P, P, P],
         "lattice_checkpoint_save": [P, C.c_char_p, I32, D, P, P],
@@ -367,6 +369,10 @@ class Lattice:
         w = self.krylov_vector()
         self._check(self._lib.feti_apply(self.h, int(mode), _ptr(v), _ptr(w)))
         return w
+
+    def lattice_set_wait_limit(self, polls):
+        """Polls after which a wait of a tensor-core product gives up (LAT_ETIMEOUT)."""
+        self._check(self._lib.lattice_set_wait_limit(self.h, int(polls)))
 
     def feti_to_global(self, v):
         u = self.dof_vector()

@@ -40,3 +40,38 @@ def test_indefinite_coarse_matrix_is_not_a_timeout(L, prec):
     x, its, rel = lat.tangent_solve(rhs, opts)
     assert its == 4 and 0 < rel < 1 and bool(torch.isfinite(x).all())
     lat.close()
+
+
+@pytest.mark.parametrize("prec,cell,dims", [
+    (0, None, (2, 2, 6)),                         # FP64 products on digits, K over a cluster
+    (2, None, (2, 2, 6)),                         # BF16 pairs, K over a cluster of 4
+    (2, latgen.ring_cell(4), (8, 9)),             # fewer panels than stages
+])
+def test_wait_that_gives_up_is_reported(L, prec, cell, dims):
+    """With no polls every wait of a pipeline gives up at once (the copies in flight are still waited
+    for): each call that makes such products says so, and is itself again with the limit restored."""
+    case, lat = _strut(L, prec, dims, cell=cell)
+    u = lat.lattice_predictor(0.1 * case.top_displacement(1))
+    opts = lat.lattice_default_opts(max_enrich=0, precond_tangent=1, krylov_max_it=3, inner_its=2)
+    lat.select_principal_cells(u, 1e-9, 1)
+    lat.lattice_prepare_solver(u, opts)
+    rhs = torch.tensor(np.random.default_rng(1).uniform(-1, 1, lat.sizes.n_dof), device="cuda")
+    v = lat.feti_from_global(rhs)
+
+    def results():
+        return [lat.feti_apply(1, v), lat.feti_apply(2, v), lat.tangent_solve(rhs, opts)[0]]
+
+    ref = results()
+    lat.lattice_set_wait_limit(0)
+    with pytest.raises(L.LatticeError, match="LAT_ETIMEOUT"):
+        lat.tangent_solve(rhs, opts)
+    lat.feti_apply(0, v)                          # no product on the tensor cores
+    if lat.sizes.n_r_local >= 384:
+        with pytest.raises(L.LatticeError, match="LAT_ETIMEOUT"):
+            lat.lattice_prepare_solver(u, opts)
+    lat.lattice_set_wait_limit(1 << 20)
+    lat.lattice_prepare_solver(u, opts)
+    assert all(torch.equal(a, b) for a, b in zip(results(), ref))
+    with pytest.raises(L.LatticeError, match="LAT_EINVAL"):
+        lat.lattice_set_wait_limit(-1)
+    lat.close()
