@@ -2425,6 +2425,7 @@ extern "C" lat_status feti_apply(lat_handle h, int32_t mode, const double* v, do
     else if (mode == 2) run_block_precond(h, v, w, 5, 0.0);
     else throw LatError{LAT_EINVAL, "mode must be 0, 1 or 2"};
     LAT_CUDA(cudaStreamSynchronize(h->stream));
+    if (mode != 0) check_waits(h);
   });
 }
 

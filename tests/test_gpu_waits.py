@@ -63,8 +63,9 @@ def test_wait_that_gives_up_is_reported(L, prec, cell, dims):
 
     ref = results()
     lat.lattice_set_wait_limit(0)
-    with pytest.raises(L.LatticeError, match="LAT_ETIMEOUT"):
-        lat.tangent_solve(rhs, opts)
+    for call in (lambda: lat.feti_apply(1, v), lambda: lat.feti_apply(2, v), lambda: lat.tangent_solve(rhs, opts)):
+        with pytest.raises(L.LatticeError, match="LAT_ETIMEOUT"):
+            call()
     lat.feti_apply(0, v)                          # no product on the tensor cores
     if lat.sizes.n_r_local >= 384:
         with pytest.raises(L.LatticeError, match="LAT_ETIMEOUT"):
