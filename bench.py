@@ -258,7 +258,8 @@ KERNELS = ["residual", "tangent_full", "tangent_material", "tangent_reduced", "g
            "apply_reduced_fp32", "apply_percell", "apply_percell_fp32", "local_segmm", "local_gemv", "local_tc",
            "gj_update", "gj_pivot", "densify", "phi_schur", "coarse_blocked", "coarse_gemv", "coarse_solve",
            "local_segmm_dual", "local_gemv_dual", "local_tc_dual", "local_segmm_dual_in", "local_gemv_dual_in",
-           "local_tc_dual_in", "dual_schur", "dual_schur_tc", "krylov_orth"]
+           "local_tc_dual_in", "local_oz", "local_oz_dual", "local_oz_dual_in", "dual_schur", "dual_schur_tc",
+           "dual_schur_oz", "krylov_orth"]
 
 
 def kernel_work(name, s, n_r, mixed):

@@ -342,8 +342,9 @@ lat_status feti_from_global(lat_handle h, const double* u_glob, double* v);
 /* Kernel timing: while enabled, CUDA events are recorded on the handle's stream around every
  * launch of the named kernels ("residual", "tangent_full", "tangent_material",
  * "tangent_reduced", "greedy_update", "apply_reduced" / "apply_reduced_fp32", "apply_percell" /
- * "apply_percell_fp32", "local_segmm", "local_gemv", "local_tc" and their "_dual" / "_dual_in"
- * variants inside the interface solve, "dual_schur" / "dual_schur_tc", "gj_update", "gj_pivot", "densify",
+ * "apply_percell_fp32", "local_segmm", "local_gemv", "local_tc", "local_oz" (FP64 products on
+ * digits) and their "_dual" / "_dual_in" variants inside the interface solve, "dual_schur" /
+ * "dual_schur_tc" / "dual_schur_oz", "gj_update", "gj_pivot", "densify",
  * "phi_schur", "coarse_blocked", "coarse_dense", "coarse_gemv", "coarse_solve", "krylov_orth").  enable = 1
  * times every named kernel; the interface PCG iteration then runs launch by launch instead of
  * as a CUDA-graph replay, so that every launch is timed.  enable = 2 times only the tangent

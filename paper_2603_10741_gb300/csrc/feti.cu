@@ -1737,7 +1737,8 @@ void kinv(lat_ctx* h, const double* v, double* w, KinvMode mode = KINV_FULL, con
     run_local_tc(h, v, wl, mode, lam);
   } else if (h->oz) {
     // FP64 on the tensor cores: exact digit products
-    KernelTimer kt(h, tg_segmm[mode]);
+    static const char* const tg[3] = {"local_oz", "local_oz_dual", "local_oz_dual_in"};
+    KernelTimer kt(h, tg[mode]);
     run_local_oz(h, v, wl, mode);
   } else {
     KernelTimer kt(h, tg_segmm[mode]);
@@ -1805,7 +1806,7 @@ void dual_precond_local(lat_ctx* h, const double* r, double* t1, double* t2) {
     if (fused_schur(h)) {
       run_sdd_tc(h, r, t2);   // tcgen05, BF16 operand pairs, FP32 accumulation; operand B_D^T r
     } else if (h->oz) {
-      KernelTimer kt(h, "dual_schur");
+      KernelTimer kt(h, "dual_schur_oz");
       run_sdd_oz(h, t1, t2);
     } else if (seg) {
       KernelTimer kt(h, "dual_schur");

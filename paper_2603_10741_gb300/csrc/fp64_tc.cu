@@ -2,30 +2,40 @@
 // of K^-rom, Y[rows of cell s] = [G; Phi^T]_{key(s)} X_R^s, and the dual Schur complements of the
 // interface preconditioner, over cells grouped by key.
 //
-// FP64 runs at 1.2 TFLOP/s on this GPU, 1/1500 of its BF16 tensor rate, and these products are 80 %
+// FP64 runs at 1.2 TFLOP/s on this GPU, 1/1500 of its BF16 tensor rate, and these products were 80 %
 // of an FP64 3D solve.  They are formed without it, by an error-free splitting (the scheme of Ozaki,
 // Ogita, Oishi and Rump, "Error-free transformations of matrix multiplication by using fast routines
 // of matrix multiplication and its applications", 2012): each row of the matrix and each cell vector
-// is scaled by a power of two and split into 8 signed base-128 digits,
-//   x = 2^(e-6) sum_i s_i 2^(-7 i),  |s_i| <= 64   (|x| <= 2^e; the rest is below 2^(e-56)),
-// digits are exact in BF16, products of digits are integers below 2^12, and the tensor core adds
-// them in FP32 exactly while a sum stays below 2^24.  The 36 digit products with i + j <= 7 go to
-// eight accumulators by i + j (at most 8 products of 2^12 per column: 512 columns may be summed),
-// which the epilogue recombines as integers and converts to FP64 once.
+// is scaled by a power of two and split into 12 signed base-128 digits,
+//   x = 2^(e-6) sum_i s_i 2^(-7 i),  |s_i| <= 64   (|x| <= 2^e; the rest is below 2^(e-84)),
+// digits are exact in BF16, products of digits are integers up to 2^12, and the tensor core adds
+// them in FP32 exactly while a sum stays within 2^24.  The 78 digit products with i + j <= 11 go to
+// twelve accumulators by i + j (at most 12 products of 2^12 per column: 336 columns may be summed),
+// which the epilogue recombines as integers, four at a time, and converts to FP64.
 //
-// Precision.  What is dropped (digits beyond the eighth, products with i + j > 7) is about 2^-56 of
-// (row maximum) x (vector maximum) per term, with random signs; rounding in an FP64 dot product of
-// K terms is about 2^-53 of sqrt(K) times the rms product per term.  Measured: K^-rom K~ v - v on
-// lattices of equal strut cells (36, 216 and 225 cells, three vectors each) is 1.6e-13 to 1.0e-12 of
-// v, 0.91 (geometric mean) of what FP64 products with the same inverses leave.
+// Precision.  What is left out (digits beyond the twelfth, products with i + j > 11) is less than
+// 12.1 x 2^-82 of (row maximum) x (vector maximum) per term; the recombination and the sums over the
+// CTAs of a cluster round ten times at most.  An FP64 sum rounds relative to sum |g| |x| instead, so the
+// number of digits has to cover the spread of the operands as well: entries of either down to 2^-31 of
+// their maximum keep all their bits.  Error of the product in the 2-norm, and the largest error of an
+// entry against its sum |g| |x|, of the strut cell's dual Schur complement (1692 columns; its entries
+// fall to 1e-24 of their row's largest), emulated; FP64 sums, then 8 digits (not enough on graded
+// vectors) and 12:
+//   uniform in [-1, 1]             1.4e-15 2.2e-15    8.3e-16 9.6e-16    4.5e-17 5.2e-17
+//   magnitudes 1e-12 to 1          7.8e-16 3.2e-15    3.3e-15 2.4e-13    4.8e-17 9.1e-17
+//   20 entries over 1e-6           9.8e-16 5.5e-15    5.0e-15 1.0e-10    3.7e-17 1.0e-16
+//   one entry over 1e-8            7.5e-16 5.8e-15    1.3e-14 1.0e-07    6.5e-17 8.0e-16
+//   one entry over 1e-12           4.1e-16 7.4e-15    5.4e-15 3.5e-04    4.3e-17 5.9e-12
+// (G itself is denser: 1.0e-16 in every row of its dual block.)  Only entries whose terms all lie below
+// 2^-26 of row maximum x vector maximum come out less exact than an FP64 sum leaves them.
 //
-// One tensor-memory tile is 128 rows x (8 accumulators of 16 cells): for digit i of the matrix one
-// MMA multiplies the digits 0 .. 7-i of the 16 cells (N = 16 (8 - i), consecutive rows of the B
-// panel) into the accumulators i .. 7, consecutive columns from 16 i on.  K is split over a cluster
-// of CTAs (512 columns at most each, which the exactness needs) that add their FP64 tiles through
-// distributed shared memory.  Bound by streaming the digits, 16 bytes per matrix entry: the strut
-// cell's dual block (1716 x 1692) for 3 keys and 36 cells is 151 MB: 35 us,
-// and 15 us to split the vectors, against 406 us on the FP64 pipe (175 us at its full rate).
+// One tensor-memory tile is 128 rows x (12 accumulators of 16 cells): for digit i of the matrix one
+// MMA multiplies the digits 0 .. 11-i of the 16 cells (N = 16 (12 - i), consecutive rows of the B
+// panel) into the accumulators i .. 11, consecutive columns from 16 i on.  K is split over a cluster
+// of CTAs (336 columns at most each while eight CTAs suffice, which the exactness needs) that add their
+// FP64 tiles through distributed shared memory.  Bound by streaming the digits, 24 bytes per matrix
+// entry: the strut cell's dual block (1716 x 1692) for 3 keys and 36 cells is 227 MB: 67 us with
+// splitting the vectors (54 us with 8 digits) against 406 us on the FP64 pipe (175 us at its full rate).
 #include <algorithm>
 
 #include "common.cuh"
@@ -33,15 +43,16 @@
 
 namespace {
 
-constexpr int ND = 8;                     // digits
+constexpr int ND = 12;                    // digits
 constexpr int TM = 128, TK = 16, NC = kOzCells; // rows, K panel, cells of a tile
 constexpr int A_SLICE = TM * TK;          // elements of one digit of an A panel
-constexpr int A_ELEMS = ND * A_SLICE;     // 32 KiB
-constexpr int B_ELEMS = ND * NC * TK;     // 4 KiB
+constexpr int A_ELEMS = ND * A_SLICE;     // 48 KiB
+constexpr int B_ELEMS = ND * NC * TK;     // 6 KiB
 constexpr int STAGE_BYTES = 2 * (A_ELEMS + B_ELEMS);
-constexpr int STAGES = 3;                 // 108 KiB, two CTAs per SM
-constexpr int TMEM_COLS = ND * NC;        // 128
-constexpr int MAX_PANELS = 512 / TK;      // panels one CTA may sum exactly
+constexpr int STAGES = 2;                 // 108 KiB, two CTAs per SM
+constexpr int TMEM_COLS = 256;            // ND * NC = 192, allocated in powers of two
+constexpr int EXACT_PANELS = 336 / TK;    // panels one CTA sums exactly in every accumulator
+constexpr int MAX_PANELS = 512 / TK;      // and in the accumulators 0 .. 7
 constexpr int MAX_SPLIT = 8;              // portable cluster size
 constexpr int PART_LD = TM + 1;
 constexpr uint32_t LBO = 128, SBO = (TK / 8) * 128;
@@ -60,49 +71,73 @@ __device__ __forceinline__ unsigned long long abs_bits(double x) {
   return (unsigned long long)__double_as_longlong(x) & 0x7fffffffffffffffull;
 }
 
+// biased exponent of a magnitude's bits, subnormals with that of the smallest normal number
+__device__ __forceinline__ int biased_exponent(unsigned long long mag) { return max(1, (int)(mag >> 52)); }
 // e of a row or vector from the bits of its largest magnitude (every |x| <= 2^e), and the factor
 // 2^(e-6) of its digits: 0 for an all-zero row, NaN when an entry is infinite or NaN
-__device__ __forceinline__ int top_exponent(unsigned long long mx) { return (int)(mx >> 52) - 1022; }
+__device__ __forceinline__ int top_exponent(unsigned long long mx) { return biased_exponent(mx) - 1022; }
 __device__ __forceinline__ double digit_scale(unsigned long long mx) {
   if (mx >= 0x7ff0000000000000ull) return __longlong_as_double(0x7ff8000000000000ll);
-  if (mx < 0x0010000000000000ull) return 0.0;   // zero (subnormal magnitudes count as zero)
+  if (mx == 0) return 0.0;
   return scalbn(1.0, top_exponent(mx) - 6);
 }
 
-// the 8 base-2^DB digits of x for the top exponent e: q = round(x 2^(7 DB + 6 - e)), |q| <=
-// 2^(7 DB + 6), by integer operations (the FP64 pipe is the narrow one), lowest digit first
-template <int DB>
-__device__ __forceinline__ void digits(double x, unsigned long long mx, float (&s)[ND]) {
-  constexpr long long half = 1ll << (DB - 1), mask = (1ll << DB) - 1;
-  const long long b = __double_as_longlong(x);
-  const int ex = (int)((b >> 52) & 0x7ff);
-  const bool ok = ex > 0 && mx < 0x7ff0000000000000ull;
-  const unsigned long long m = (b & 0xfffffffffffffll) | 0x10000000000000ll;
-  const int sh = ex - 1022 - top_exponent(mx) + 7 * DB - 47;   // x = m 2^(ex - 1075); at most 7 DB - 47
-  unsigned long long mag = 0;
-  if (ok) mag = sh >= 0 ? m << sh : sh > -55 ? (m + (1ull << (-sh - 1))) >> -sh : 0;
-  long long q = b < 0 ? -(long long)mag : (long long)mag;
-#pragma unroll
-  for (int i = ND - 1; i >= 0; --i) {
-    const long long d = i ? ((q + half) & mask) - half : q;
-    s[i] = (float)(int)d;
-    q = (q - d) >> DB;
+// x 2^(P - e) for the top exponent e, P = BITS + 6 <= 83, rounded to a whole number hi 2^42 + lo of sign
+// and magnitude, by integer operations (the FP64 pipe is the narrow one); 0 when the row is not finite
+template <int BITS>
+__device__ __forceinline__ void fixed_point(double x, unsigned long long mx, long long& hi, long long& lo) {
+  constexpr unsigned long long low = (1ull << 42) - 1;
+  const unsigned long long b = abs_bits(x);
+  const unsigned long long m = (b & 0xfffffffffffffull) | (b >> 52 ? 0x10000000000000ull : 0);
+  // x = m 2^(biased exponent - 1075)
+  const int sh = biased_exponent(b) - 1022 - top_exponent(mx) + BITS - 47;   // at most BITS - 47
+  unsigned long long vh = 0, vl = 0;
+  if (mx < 0x7ff0000000000000ull) {
+    if (sh >= 0) {
+      vl = (m << sh) & low;
+      vh = m >> (42 - sh);
+    } else if (sh > -55) {
+      const unsigned long long v = (m + (1ull << (-sh - 1))) >> -sh;
+      vl = v & low;
+      vh = v >> 42;
+    }
   }
+  const bool neg = __double_as_longlong(x) < 0;
+  hi = neg ? -(long long)vh : (long long)vh;
+  lo = neg ? -(long long)vl : (long long)vl;
 }
 
-// digit panels of eight consecutive K entries of one row: dst + i * stride, 16 bytes per digit
+// lowest balanced base-2^DB digit of q, taken off
+template <int DB>
+__device__ __forceinline__ int pop_digit(long long& q) {
+  constexpr long long half = 1ll << (DB - 1), mask = (1ll << DB) - 1;
+  const long long d = ((q + half) & mask) - half;
+  q = (q - d) >> DB;
+  return (int)d;
+}
+
+// digit panels of eight consecutive K entries of one row: dst + i * stride, 16 bytes per digit; lowest
+// digit first, six from the low words, the rest from the high ones
 __device__ __forceinline__ void store_digits(const double (&v)[8], unsigned long long mx, __nv_bfloat16* dst,
                                              int stride) {
-  float s[8][ND];
+  static_assert(ND == 12, "two words of six digits");
+  long long hi[8], q[8];
 #pragma unroll
-  for (int q = 0; q < 8; ++q) digits<7>(v[q], mx, s[q]);
+  for (int k = 0; k < 8; ++k) fixed_point<7 * (ND - 1)>(v[k], mx, hi[k], q[k]);
 #pragma unroll
-  for (int i = 0; i < ND; ++i) {
+  for (int i = ND - 1; i >= 0; --i) {
     uint32_t w[4];
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const __nv_bfloat162 p = __floats2bfloat162_rn(s[2 * q][i], s[2 * q + 1][i]);
-      w[q] = *reinterpret_cast<const uint32_t*>(&p);
+    for (int k = 0; k < 4; ++k) {
+      float f[2];
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        long long& x = q[2 * k + u];
+        if (i == 5) x += hi[2 * k + u];   // what is left of the low word is its carry
+        f[u] = (float)(i ? pop_digit<7>(x) : (int)x);
+      }
+      const __nv_bfloat162 p = __floats2bfloat162_rn(f[0], f[1]);
+      w[k] = *reinterpret_cast<const uint32_t*>(&p);
     }
     *reinterpret_cast<uint4*>(dst + (size_t)i * stride) = make_uint4(w[0], w[1], w[2], w[3]);
   }
@@ -212,7 +247,7 @@ __global__ void __launch_bounds__(256)
   store_digits(v, mx[(size_t)tile * NC + c], dst, NC * TK);
 }
 
-// integer sums of four digit accumulators (exact in FP32, up to 2^24), combined: below 2^50
+// integer sums of four digit accumulators (exact in FP32 up to 2^24), combined: below 2^50
 template <int DB>
 __device__ __forceinline__ double combine4(uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
   const long long v = ((long long)__float2int_rn(__uint_as_float(a)) << (3 * DB)) +
@@ -356,8 +391,9 @@ __global__ void __launch_bounds__(128, 2)
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
         const double hi = combine4<7>(r[0][q], r[1][q], r[2][q], r[3][q]);
-        const double lo = combine4<7>(r[4][q], r[5][q], r[6][q], r[7][q]);
-        part[(c + q) * PART_LD + tid] = fma(lo, 0x1p-49, hi * 0x1p-21);
+        const double mid = combine4<7>(r[4][q], r[5][q], r[6][q], r[7][q]);
+        const double lo = combine4<7>(r[8][q], r[9][q], r[10][q], r[11][q]);
+        part[(c + q) * PART_LD + tid] = fma(hi, 0x1p-21, fma(mid, 0x1p-49, lo * 0x1p-77));
       }
     }
   }
@@ -428,7 +464,7 @@ void product(lat_ctx* h, const OzShape& sh, int mt0, int kp0, const DBuf<__nv_bf
   LAT_LAUNCH(h, k_oz_pack<<<dim3(tiles, div_up(npan * (TK / 8), 16)), 256, 0, h->stream>>>(
                     sh, h->n_cells, kp0, npan, X, rdofs + r_base, ts, tc, h->seg_ptr.p, h->perm.p, h->oz_max.p,
                     h->oz_X.p));
-  const int S = div_up(npan, MAX_PANELS);
+  const int S = std::min(MAX_SPLIT, (int)div_up(npan, EXACT_PANELS));
   const size_t shm = (size_t)STAGES * STAGE_BYTES;
   LAT_CUDA(cudaFuncSetAttribute(k_oz_mm, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm));
   cudaLaunchConfig_t cfg{};
@@ -454,12 +490,13 @@ void product(lat_ctx* h, const OzShape& sh, int mt0, int kp0, const DBuf<__nv_bf
 
 }  // namespace
 
-// Whether the FP64 mode's segmented products run on digits: blocks large enough that streaming 16
+// Whether the FP64 mode's segmented products run on digits: blocks large enough that streaming 24
 // bytes per entry and the launches that split the cell vectors cost less than the FP64 pipe does
-// (36 cells of the strut cell's
-// dual block 50 us against 406, 512 cells of the whole block 0.40 ms against 6.0; the ring cells' dual
-// block is 56 columns, under 10 us either way), no more columns than the largest cluster sums exactly, and digits
-// within 24 GB and a quarter of the free memory.
+// (36 cells of the strut cell's dual block 67 us against 406, 512 cells of the whole block 0.62 ms
+// against 6.0; the ring cells' dual block is 56 columns, under 10 us either way), no more columns than
+// the largest cluster sums exactly in the accumulators 0 .. 7 (in the others beyond 2688 columns a sum
+// of like digits may round, at 2^-68 of row maximum x vector maximum), and digits within 24 GB and a
+// quarter of the free memory.
 bool oz_wanted(const lat_ctx* h) {
   if (h->prec != LAT_FP64 || (int64_t)h->n_keys * 8 > h->n_cells) return false;
   const OzShape g = g_shape(h), s = s_shape(h);
@@ -502,13 +539,15 @@ void run_sdd_oz(lat_ctx* h, const double* X, double* Y) {
 // products and the splitting of C, Pi and R.  Three 2616 matrices: 9 ms against 53 ms.
 namespace {
 
+constexpr int SD = 8;                      // digits, base 256
 constexpr int SW = kSweepPanel;
 constexpr int SP = SW / TK;                // K panels
 constexpr int SN = 32;                     // columns of a product's tile
-constexpr int SB_ELEMS = ND * SN * TK;     // 8 KiB
-constexpr int SSTAGE_BYTES = 2 * (A_ELEMS + SB_ELEMS);
+constexpr int SA_ELEMS = SD * A_SLICE;     // 32 KiB
+constexpr int SB_ELEMS = SD * SN * TK;     // 8 KiB
+constexpr int SSTAGE_BYTES = 2 * (SA_ELEMS + SB_ELEMS);
 constexpr int SSTAGES = 2;                 // 80 KiB, two CTAs per SM
-constexpr int SCOLS = ND * SN;             // 256 tensor-memory columns
+constexpr int SCOLS = SD * SN;             // 256 tensor-memory columns
 
 // digits of one row of a panel (128 values in shared memory, zero beyond the panel's width) by one
 // warp: lane l takes the columns 4l .. 4l + 3; the row's largest magnitude goes to *mx.  base: the
@@ -525,13 +564,19 @@ __device__ __forceinline__ void row_digits(const double* v, int lane, __nv_bfloa
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
   if (lane == 0) *mx = m;
-  float s[4][ND];
+  float s[4][SD];
 #pragma unroll
-  for (int q = 0; q < 4; ++q) digits<8>(x[q], m, s[q]);
+  for (int q = 0; q < 4; ++q) {
+    long long hi, lo;
+    fixed_point<8 * (SD - 1)>(x[q], m, hi, lo);
+    lo += hi * (1ll << 42);
+#pragma unroll
+    for (int i = SD - 1; i >= 0; --i) s[q][i] = (float)(i ? pop_digit<8>(lo) : (int)lo);
+  }
   const int k = 4 * lane;
   __nv_bfloat16* d = base + (size_t)(k / TK) * pstride + core_off(0, k % TK);
 #pragma unroll
-  for (int i = 0; i < ND; ++i) {
+  for (int i = 0; i < SD; ++i) {
     const __nv_bfloat162 a = __floats2bfloat162_rn(s[0][i], s[1][i]), b = __floats2bfloat162_rn(s[2][i], s[3][i]);
     *reinterpret_cast<uint2*>(d + (size_t)i * dstride) =
         make_uint2(*reinterpret_cast<const uint32_t*>(&a), *reinterpret_cast<const uint32_t*>(&b));
@@ -558,8 +603,8 @@ __global__ void __launch_bounds__(256)
   for (int r = warp; r < 32; r += 8) {
     const int row = i0 + r;   // rows up to the padded tile's end have zero digits
     if (row >= MT * TM) continue;
-    __nv_bfloat16* base = Cd + ((size_t)b * MT + row / TM) * SP * A_ELEMS + core_off(row % TM, 0);
-    row_digits(S[r], lane, base, A_ELEMS, A_SLICE, cmax + (size_t)b * MT * TM + row);
+    __nv_bfloat16* base = Cd + ((size_t)b * MT + row / TM) * SP * SA_ELEMS + core_off(row % TM, 0);
+    row_digits(S[r], lane, base, SA_ELEMS, A_SLICE, cmax + (size_t)b * MT * TM + row);
   }
 }
 
@@ -635,8 +680,8 @@ __global__ void __launch_bounds__(128, 2)
       }
       const uint32_t bar = smem_u32(&full[st]), dst = s0 + (uint32_t)(st * SSTAGE_BYTES);
       expect_tx(bar, (uint32_t)SSTAGE_BYTES);
-      bulk_copy(dst, Cd + (((size_t)b * MT + mt) * SP + p) * A_ELEMS, 2 * A_ELEMS, bar);
-      bulk_copy(dst + 2 * A_ELEMS, Bd + (((size_t)b * NT + nt) * SP + p) * SB_ELEMS, 2 * SB_ELEMS, bar);
+      bulk_copy(dst, Cd + (((size_t)b * MT + mt) * SP + p) * SA_ELEMS, 2 * SA_ELEMS, bar);
+      bulk_copy(dst + 2 * SA_ELEMS, Bd + (((size_t)b * NT + nt) * SP + p) * SB_ELEMS, 2 * SB_ELEMS, bar);
       ++n;
     }
     if (!ok) fail = 1;
@@ -650,10 +695,10 @@ __global__ void __launch_bounds__(128, 2)
         break;
       }
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      const uint32_t sa = s0 + (uint32_t)(st * SSTAGE_BYTES), sb = sa + 2 * A_ELEMS;
+      const uint32_t sa = s0 + (uint32_t)(st * SSTAGE_BYTES), sb = sa + 2 * SA_ELEMS;
 #pragma unroll
-      for (int i = 0; i < ND; ++i) {
-        const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)((ND - i) * SN >> 3) << 17) |
+      for (int i = 0; i < SD; ++i) {
+        const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)((SD - i) * SN >> 3) << 17) |
                                ((uint32_t)(TM >> 4) << 24);
         const uint32_t acc = (p > 0 || i > 0) ? 1u : 0u;
         asm volatile(
@@ -692,9 +737,9 @@ __global__ void __launch_bounds__(128, 2)
     const bool ip = gi >= k0 && gi < k0 + kw;
 #pragma unroll 1
     for (int c = 0; c < SN; c += 4) {
-      uint32_t r[ND][4];
+      uint32_t r[SD][4];
 #pragma unroll
-      for (int g = 0; g < ND; ++g) tmem_ld4(base + (uint32_t)(g * SN + c), r[g]);
+      for (int g = 0; g < SD; ++g) tmem_ld4(base + (uint32_t)(g * SN + c), r[g]);
       asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
@@ -726,7 +771,7 @@ __global__ void __launch_bounds__(128, 2)
 
 // matrices of one size whose panels' workspace (run_sweep_panel) stays within 2 GB
 int sweep_panel_batch(int n) {
-  const double per = 2.0 * div_up(n, TM) * SP * A_ELEMS + 2.0 * (div_up(n, SN) + SW / SN) * SP * SB_ELEMS +
+  const double per = 2.0 * div_up(n, TM) * SP * SA_ELEMS + 2.0 * (div_up(n, SN) + SW / SN) * SP * SB_ELEMS +
                      8.0 * n * SW + 8.0 * SW * SW;
   return std::max(1, (int)(2e9 / per));
 }
@@ -734,7 +779,7 @@ int sweep_panel_batch(int n) {
 // one panel [k0, k0 + kw) of the sweep of `batch` n x n matrices (lower triangles)
 void run_sweep_panel(lat_ctx* h, double* A, int n, int batch, int64_t bs, int k0, int kw, int neg_bit) {
   const int MT = div_up(n, TM), NT = div_up(n, SN), PT = SW / SN;
-  h->sp_C.ensure((size_t)batch * MT * SP * A_ELEMS);
+  h->sp_C.ensure((size_t)batch * MT * SP * SA_ELEMS);
   h->sp_B.ensure((size_t)batch * (NT + PT) * SP * SB_ELEMS);
   h->sp_max.ensure((size_t)batch * (MT * TM + (NT + PT) * SN));
   h->sp_P.ensure((size_t)batch * SW * SW);
