@@ -54,6 +54,7 @@ constexpr int TMEM_COLS = 256;            // ND * NC = 192, allocated in powers 
 constexpr int EXACT_PANELS = 336 / TK;    // panels one CTA sums exactly in every accumulator
 constexpr int MAX_PANELS = 512 / TK;      // and in the accumulators 0 .. 7
 constexpr int MAX_SPLIT = 8;              // portable cluster size
+constexpr double kOzBytes = 24e9;         // most digits kept, a twelfth of the device's memory
 constexpr int PART_LD = TM + 1;
 constexpr uint32_t LBO = 128, SBO = (TK / 8) * 128;
 static_assert((size_t)NC * PART_LD * sizeof(double) <= (size_t)STAGES * STAGE_BYTES, "the tile reuses the stages");
@@ -495,18 +496,15 @@ void product(lat_ctx* h, const OzShape& sh, int mt0, int kp0, const DBuf<__nv_bf
 // (36 cells of the strut cell's dual block 67 us against 406, 512 cells of the whole block 0.62 ms
 // against 6.0; the ring cells' dual block is 56 columns, under 10 us either way), no more columns than
 // the largest cluster sums exactly in the accumulators 0 .. 7 (in the others beyond 2688 columns a sum
-// of like digits may round, at 2^-68 of row maximum x vector maximum), and digits within 24 GB and a
-// quarter of the free memory.
+// of like digits may round, at 2^-68 of row maximum x vector maximum), and at most kOzBytes of
+// digits (95 keys of the strut cell).  Sizes alone decide, never the memory that happens to be free: the
+// same call gives the same bits beside any other allocation.
 bool oz_wanted(const lat_ctx* h) {
   if (h->prec != LAT_FP64 || (int64_t)h->n_keys * 8 > h->n_cells) return false;
   const OzShape g = g_shape(h), s = s_shape(h);
   if (h->n_R - h->n_I < 512 || g.KP > MAX_SPLIT * MAX_PANELS) return false;
   const double nG = (double)h->n_keys * A_ELEMS * g.MT * g.KP, nS = (double)h->n_keys * A_ELEMS * s.MT * s.KP;
-  if (2 * (nG + nS) > 24e9) return false;
-  if ((double)h->oz_G.n >= nG && (double)h->oz_S.n >= nS) return true;
-  // room for them beside what the Krylov solves will still allocate
-  size_t free_b = 0, total_b = 0;
-  return cudaMemGetInfo(&free_b, &total_b) == cudaSuccess && 2 * (nG + nS) <= 0.25 * (double)free_b;
+  return 2 * (nG + nS) <= kOzBytes;
 }
 
 // digits of the augmented local matrices and of the dual Schur complements (after the inversions)

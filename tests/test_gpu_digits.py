@@ -29,16 +29,17 @@ def L():
     return lattice
 
 
-def _layer(L, nx, prec=0):
+def _prepare(lat, force_all=False):
+    u = lat.lattice_predictor(0.0)
+    lat.select_principal_cells(u, 1e-3, 1, force_all=force_all)
+    lat.lattice_prepare_solver(u, lat.lattice_default_opts(precond_tangent=0, max_enrich=0))
+
+
+def _layer(L, nx):
     lat_geo = latgen.tile(*CELL, (nx, nx, 1))
     case = latgen.LoadCase(name="digits", lattice=lat_geo, mu=1.0, lam=4.0,
                            mu_scale=latgen.mu_scale(lat_geo.n_cells, None), total_strain=0.01, n_steps=1, eps=1e-3)
-    lat = L.Lattice.from_case(case, prec)
-    u = lat.lattice_predictor(0.0)
-    lat.select_principal_cells(u, 1e-3, 1)
-    lat.lattice_prepare_solver(u, lat.lattice_default_opts(precond_tangent=0, max_enrich=0))
-    assert lat.sizes.n_primal == 0
-    return lat
+    return L.Lattice.from_case(case)
 
 
 def _local(lat, X):
@@ -53,7 +54,10 @@ def _local(lat, X):
 def block(L):
     """(the layer on digits, the layer on the FP64 pipe, remaining free local DOFs, G on them)"""
     pipe, oz = _layer(L, 2), _layer(L, 4)
-    oz.lattice_set_timing(1)
+    for lat in (pipe, oz):
+        _prepare(lat)
+        assert lat.sizes.n_primal == 0
+        lat.lattice_set_timing(1)
     X_ref = CELL[0]
     on_face = (np.abs(X_ref[:, 2]) < 1e-12) | (np.abs(X_ref[:, 2] - 1) < 1e-12)   # clamped, corners among them
     dofs = np.flatnonzero(~np.repeat(on_face, 3))
@@ -171,3 +175,31 @@ def test_block_preconditioner_with_unequal_cells(L, dims):
         assert counts == ([1, 5, 1, 6] if prec == 0 else [0, 0, 0, 0])
         lat.close()
     assert np.linalg.norm(outs[1] - outs[0]) < 1e-3 * np.linalg.norm(outs[0])
+
+
+def test_results_do_not_depend_on_free_memory(L):
+    """The form of the products is a matter of sizes: with most of the device's memory taken by someone
+    else the same call gives the same bits."""
+    def run():
+        lat_geo = latgen.tile(*CELL, (2, 2, 6))
+        case = latgen.LoadCase(name="digits", lattice=lat_geo, mu=1.0, lam=4.0,
+                               mu_scale=latgen.mu_scale(lat_geo.n_cells, 3), total_strain=0.001, n_steps=1, eps=1e-3)
+        lat = L.Lattice.from_case(case)
+        u = lat.lattice_predictor(case.top_displacement(1))
+        lat.select_principal_cells(u, 1e-9, 1)
+        lat.lattice_prepare_solver(u, lat.lattice_default_opts(max_enrich=0))
+        v = lat.feti_from_global(torch.tensor(np.random.default_rng(8).uniform(-1, 1, lat.sizes.n_dof), device="cuda"))
+        out = lat.feti_apply(1, v)
+        lat.close()
+        return out
+
+    ref = run()
+    torch.cuda.empty_cache()
+    left = 1700 * 2 ** 20
+    held = torch.empty(torch.cuda.mem_get_info()[0] - left, dtype=torch.uint8, device="cuda")
+    try:
+        got = run()
+    finally:
+        del held
+        torch.cuda.empty_cache()
+    assert torch.equal(got, ref)
