@@ -1517,6 +1517,8 @@ void run_prepare_solver(lat_ctx* h, const lat_newton_opts* o, const double* u_gl
     h->tile_seg_oz.upload(tseg_oz, h->stream);
     h->tile_c0_oz.upload(tc0_oz, h->stream);
     h->oz_tiles = (int)tseg_oz.size();
+  } else {
+    for (auto* b : {&h->oz_G, &h->oz_S, &h->oz_X}) b->release();   // of an earlier selection
   }
   // dense local blocks
   const int64_t gstride = (int64_t)(nR + nP) * nR;   // augmented [G; Phi^T] per key

@@ -203,3 +203,22 @@ def test_results_do_not_depend_on_free_memory(L):
         del held
         torch.cuda.empty_cache()
     assert torch.equal(got, ref)
+
+
+def test_digits_are_given_back(L):
+    """A selection with too many keys for digits holds no digits of the one before (250 MB for one key,
+    167 with eight digits): as much memory as without that selection, up to small tables."""
+    def held(selections):
+        torch.cuda.synchronize()
+        free = torch.cuda.mem_get_info()[0]
+        lat = _layer(L, 4)
+        for force_all in selections:
+            _prepare(lat, force_all)
+            lat.feti_apply(1, lat.krylov_vector())
+        used = free - torch.cuda.mem_get_info()[0]
+        lat.close()
+        return used
+
+    torch.cuda.empty_cache()
+    held([True])                                  # module load and torch's own first allocations
+    assert held([False, True]) - held([True]) < 100e6
