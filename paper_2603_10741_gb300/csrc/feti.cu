@@ -554,22 +554,12 @@ __global__ void k_densify(int n_keys, const int* __restrict__ key_list, int n_cl
 constexpr int GJB = 32;
 constexpr int kSwRows = 16;   // rows of R per CTA
 
-// 1 / x from the hardware's approximation (about 20 bits) and one cubically convergent correction
-// r (1 + e + e^2), e = 1 - x r: three dependent FP64 operations; the division outside its range
-__device__ __forceinline__ double pivot_rcp(double x) {
-  if (!(fabs(x) > 1e-290 && fabs(x) < 1e290)) return x != 0.0 ? 1.0 / x : 0.0;
-  double r;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
-  const double e = fma(-x, r, 1.0);
-  return fma(r, fma(e, e, e), r);
-}
-
 // Sweeps of the symmetric kw x kw pivot block M in shared memory by 1 x 1 pivots (256 threads), M
 // <- -M^{-1}.  A chain of kw dependent steps, and a dependent FP64 operation takes about 100 clocks:
 // warp 0 runs the chain alone (it keeps the diagonal, so the next reciprocal is formed while the
 // other warps apply the step), the 528 entries of the triangle stay in the others' registers, and
 // a step's column and products go through shared memory.  30 us for 32 columns when every step
-// waited for the division and the division for the step, 24 us now (cold caches).
+// waited for the division and the division for the step, 25 us now (cold caches).
 __device__ void sweep_pivot(int kw, double (&M)[GJB][GJB + 1], double (&col)[2][GJB], double (&rp)[GJB],
                             int* __restrict__ flag, int neg_bit) {
   const int t = threadIdx.x, n_e = kw * (kw + 1) / 2;
@@ -599,7 +589,7 @@ __device__ void sweep_pivot(int kw, double (&M)[GJB][GJB + 1], double (&col)[2][
     diag = t < kw ? M[t][t] : 0.0;
     const double piv = __shfl_sync(0xffffffffu, diag, 0);
     check(piv);
-    d = pivot_rcp(piv);
+    d = piv != 0.0 ? 1.0 / piv : 0.0;
   }
   for (int p = 0; p < kw; ++p) {
     const double (&c)[GJB] = col[p & 1];
@@ -616,7 +606,7 @@ __device__ void sweep_pivot(int kw, double (&M)[GJB][GJB + 1], double (&col)[2][
       const double piv = __shfl_sync(0xffffffffu, diag, min(p + 1, 31));
       if (p + 1 < kw) {
         check(piv);
-        d = pivot_rcp(piv);
+        d = piv != 0.0 ? 1.0 / piv : 0.0;
       }
     } else {
 #pragma unroll
