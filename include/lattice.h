@@ -348,8 +348,8 @@ lat_status feti_from_global(lat_handle h, const double* u_glob, double* v);
  * "phi_schur", "coarse_blocked", "coarse_dense", "coarse_gemv", "coarse_solve", "krylov_orth").  enable = 1
  * times every named kernel; the interface PCG iteration then runs launch by launch instead of
  * as a CUDA-graph replay, so that every launch is timed.  enable = 2 times only the tangent
- * action kernels ("apply_*") and keeps the graph replays.  lattice_set_timing clears the
- * records; lattice_kernel_time returns the summed duration (host ms) and the launch count of
+ * action kernels ("apply_*") and keeps the graph replays unless they hold one (the lumped interface
+ * preconditioner's action).  lattice_set_timing clears the records; lattice_kernel_time returns the summed duration (host ms) and the launch count of
  * one name since then. */
 lat_status lattice_set_timing(lat_handle h, int32_t enable);
 lat_status lattice_kernel_time(lat_handle h, const char* name, double* total_ms, int32_t* launches);

@@ -1918,7 +1918,7 @@ void run_block_precond(lat_ctx* h, const double* v, double* w, int pcg_iters, do
     // PCG until the preconditioned residual r^T M r has dropped by pcg_rtol^2 (0: never), at most
     // pcg_iters iterations, or until breakdown.  An iteration updates the search direction first (p =
     // z + beta p; p = z on the first pass, from p = 0 and beta = 0), so that every one is the same
-    // sequence of launches.  Outside the kernel-timing mode it is the body of a graph's while node,
+    // sequence of launches.  Unless its kernels are timed it is the body of a graph's while node,
     // captured once per preconditioner setup: the loop runs on the device, and the host, which used
     // to read the residual after every iteration (about 15 us of an iteration of 60 to 300), waits
     // once per solve.  The two dot products share the jump kernels' pass and their last block leaves
@@ -1956,7 +1956,9 @@ void run_block_precond(lat_ctx* h, const double* v, double* w, int pcg_iters, do
       }
       LAT_CHECK_LAUNCH();
     };
-    bool graph = (!h->timing || h->timing_apply_only) && h->graphs_ok;
+    // the loop's launches have no events of their own; with the lumped preconditioner every iteration
+    // holds an action, which timing_apply_only is there to time
+    bool graph = (!h->timing || (h->timing_apply_only && h->iface == 0)) && h->graphs_ok;
     if (graph && !h->pcg_exec) graph = capture_pcg_loop(h, body);
     auto* hs = reinterpret_cast<PcgScalars*>(h->h_pinned + 8);
     auto read = [&] {
