@@ -265,7 +265,7 @@ struct KernelTimer {
     return e;
   }
   KernelTimer(lat_ctx* h_, const char* n) : h(h_), name(n) {
-    if (!h->timing) return;
+    if (!h || !h->timing) return;
     if (h->timing_apply_only && std::strncmp(n, "apply_", 6) != 0) return;
     a = take(h);
     b = take(h);

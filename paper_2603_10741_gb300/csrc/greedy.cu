@@ -204,16 +204,19 @@ __global__ void __launch_bounds__(kColThreads)
 // Algorithm 1 on the workspaces given: the launches of one chunk of iterations [it0, it1).  The
 // selection of iteration it runs at the end of the pass before (init for it = 0), so the update of
 // the last iteration a chunk can reach also decides the end.
-void launch_greedy(cudaStream_t st, int n_sm, int it0, int it1, int64_t n_rows, int n_cols, double* delta, double* Z,
-                   double* part, double* beta, const SelectArgs& base) {
+// h: the handle whose kernel timing and launch count take the launches, or null.
+void launch_greedy(lat_ctx* h, cudaStream_t st, int n_sm, int it0, int it1, int64_t n_rows, int n_cols, double* delta,
+                   double* Z, double* part, double* beta, const SelectArgs& base) {
   const int zgrid = std::min(div_up(n_rows, 256), 4 * n_sm);
   for (int it = it0; it < it1; ++it) {
     k_g_norm<<<kNormBlocks, 256, 0, st>>>(n_rows, delta, base.state, part);
     k_g_zeta<<<zgrid, 256, 0, st>>>(it, n_rows, delta, base.state, part, Z);
     SelectArgs A = base;
     A.it = it + 1;
+    KernelTimer kt(h, "greedy_update");
     k_g_update<<<n_cols, kColThreads, 0, st>>>(it, n_rows, delta, Z, beta, A);
   }
+  if (h) h->n_launch += 3 * (it1 - it0);
 }
 
 // alpha^s from R alpha^s = ||t^s|| beta^s, R_ir = ||t^{s_r}|| beta_i^{s_r} (i <= r): the
@@ -273,11 +276,8 @@ void run_greedy(lat_ctx* h, const double* T, int64_t n_rows, int n_cols, double 
   const int chunk = 8;
   for (int it0 = 0; it0 < limit; it0 += chunk) {
     const int it1 = std::min(it0 + chunk, limit);
-    {
-      KernelTimer kt(h, "greedy_update");
-      launch_greedy(h->stream, h->n_sm, it0, it1, n_rows, n_cols, h->g_delta.p, h->g_Z.p, h->g_part.p, h->g_beta.p, base);
-      h->n_launch += 3 * (it1 - it0);
-    }
+    launch_greedy(h, h->stream, h->n_sm, it0, it1, n_rows, n_cols, h->g_delta.p, h->g_Z.p, h->g_part.p, h->g_beta.p,
+                  base);
     LAT_CHECK_LAUNCH();
     LAT_CUDA(cudaMemcpyAsync(hp, h->g_state.p, 2 * sizeof(int), cudaMemcpyDeviceToHost, h->stream));
     LAT_CUDA(cudaStreamSynchronize(h->stream));
@@ -500,7 +500,7 @@ extern "C" lat_status greedy_select_static(const double* T, int64_t n_rows, int3
   int hstate[2] = {0, 0};
   const int chunk = 8;
   for (int it0 = 0; it0 < limit; it0 += chunk) {
-    launch_greedy(st, n_sm, it0, std::min(it0 + chunk, limit), n_rows, n_cols, W.delta, W.Z, W.part, W.beta, base);
+    launch_greedy(nullptr, st, n_sm, it0, std::min(it0 + chunk, limit), n_rows, n_cols, W.delta, W.Z, W.part, W.beta, base);
     if (cudaGetLastError() != cudaSuccess) return LAT_ECUDA;
     if (cudaMemcpyAsync(hstate, W.state, 2 * sizeof(int), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
         cudaStreamSynchronize(st) != cudaSuccess)

@@ -16,6 +16,17 @@ def L():
     return lattice
 
 
+def test_greedy_update_counts_updates(L):
+    """One record per projection of the columns: five principals, five updates."""
+    T = torch.tensor(np.random.default_rng(3).normal(size=(40, 257)), device="cuda")
+    lat = L.Lattice.from_case(latgen.make_case("ring2"))
+    lat.lattice_set_timing(1)
+    out = lat.greedy_select(T, 1e-12, 5)
+    assert out["S"].numel() == 5
+    assert lat.lattice_kernel_time("greedy_update")[1] == 5
+    lat.close()
+
+
 @pytest.mark.parametrize("prec,name", [(0, "apply_reduced"), (1, "apply_reduced_fp32")])
 def test_action_timing_covers_the_lumped_interface_loop(L, prec, name):
     """enable = 2 times every launch of the action: with the lumped interface preconditioner each
