@@ -790,17 +790,27 @@ void run_sweep_panel(lat_ctx* h, double* A, int n, int batch, int64_t bs, int k0
   const size_t shm = (size_t)SSTAGES * SSTAGE_BYTES;
   LAT_CUDA(cudaFuncSetAttribute(k_sp_mm<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm));
   LAT_CUDA(cudaFuncSetAttribute(k_sp_mm<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm));
-  LAT_LAUNCH(h, k_sp_panel<<<dim3(MT * TM / 32, batch), 256, 0, h->stream>>>(n, bs, k0, kw, MT, A, h->sp_C.p, cmax,
-                                                                            h->sp_P.p));
+  {
+    KernelTimer kt(h, "gj_pivot");
+    LAT_LAUNCH(h, k_sp_panel<<<dim3(MT * TM / 32, batch), 256, 0, h->stream>>>(n, bs, k0, kw, MT, A, h->sp_C.p, cmax,
+                                                                              h->sp_P.p));
+  }
   sweep_small(h, h->sp_P.p, kw, batch, (int64_t)SW * SW, neg_bit);
-  LAT_LAUNCH(h, k_sp_rows<<<dim3(SW / 8, batch), 256, 0, h->stream>>>(kw, kw, (int64_t)SW * SW, kw, PT, h->sp_P.p, Pd,
-                                                                      pmax));
-  LAT_LAUNCH(h, k_sp_mm<false><<<dim3(MT * PT, batch), 128, shm, h->stream>>>(n, bs, k0, kw, MT, PT, h->sp_C.p, cmax, Pd,
-                                                                              pmax, h->sp_P.p, h->sp_R.p, A, h->flag.p,
-                                                                              h->wait_polls));
-  LAT_LAUNCH(h, k_sp_rows<<<dim3(NT * SN / 8, batch), 256, 0, h->stream>>>(n, SW, (int64_t)n * SW, kw, NT, h->sp_R.p, Rd,
-                                                                          rmax));
-  LAT_LAUNCH(h, k_sp_mm<true><<<dim3(2 * MT * (MT + 1), batch), 128, shm, h->stream>>>(
-                    n, bs, k0, kw, MT, NT, h->sp_C.p, cmax, Rd, rmax, h->sp_P.p, h->sp_R.p, A, h->flag.p, h->wait_polls));
+  {
+    KernelTimer kt(h, "gj_pivot");
+    LAT_LAUNCH(h, k_sp_rows<<<dim3(SW / 8, batch), 256, 0, h->stream>>>(kw, kw, (int64_t)SW * SW, kw, PT, h->sp_P.p, Pd,
+                                                                        pmax));
+    LAT_LAUNCH(h, k_sp_mm<false><<<dim3(MT * PT, batch), 128, shm, h->stream>>>(
+                      n, bs, k0, kw, MT, PT, h->sp_C.p, cmax, Pd, pmax, h->sp_P.p, h->sp_R.p, A, h->flag.p,
+                      h->wait_polls));
+    LAT_LAUNCH(h, k_sp_rows<<<dim3(NT * SN / 8, batch), 256, 0, h->stream>>>(n, SW, (int64_t)n * SW, kw, NT, h->sp_R.p,
+                                                                            Rd, rmax));
+  }
+  {
+    KernelTimer kt(h, "gj_update");
+    LAT_LAUNCH(h, k_sp_mm<true><<<dim3(2 * MT * (MT + 1), batch), 128, shm, h->stream>>>(
+                      n, bs, k0, kw, MT, NT, h->sp_C.p, cmax, Rd, rmax, h->sp_P.p, h->sp_R.p, A, h->flag.p,
+                      h->wait_polls));
+  }
   LAT_CHECK_LAUNCH();
 }

@@ -27,6 +27,23 @@ def test_greedy_update_counts_updates(L):
     lat.close()
 
 
+def test_trailing_updates_of_large_inversions_are_timed(L):
+    """One cell of 1005 remaining DOFs, 375 of them interior, every corner fixed (no coarse matrix): 3 +
+    5 panels of 128 columns, each with its trailing update and the four of its pivot block."""
+    Xr, E = latgen.solid_cell(6, 3)
+    lat_geo = latgen.tile(Xr, E, (1, 1, 1))
+    case = latgen.LoadCase(name="timing", lattice=lat_geo, mu=1.0, lam=4.0, mu_scale=latgen.mu_scale(1, None),
+                           total_strain=0.01, n_steps=1, eps=1e-3)
+    lat = L.Lattice.from_case(case)
+    u = lat.lattice_predictor(case.top_displacement(1))
+    lat.select_principal_cells(u, 0.0, 1, force_all=True)
+    lat.lattice_set_timing(1)
+    lat.lattice_prepare_solver(u, lat.lattice_default_opts(max_enrich=0))
+    assert lat.sizes.n_primal == 0 and lat.sizes.n_r_local == 1005
+    assert lat.lattice_kernel_time("gj_update")[1] == 8 * 5
+    lat.close()
+
+
 @pytest.mark.parametrize("prec,name", [(0, "apply_reduced"), (1, "apply_reduced_fp32")])
 def test_action_timing_covers_the_lumped_interface_loop(L, prec, name):
     """enable = 2 times every launch of the action: with the lumped interface preconditioner each
