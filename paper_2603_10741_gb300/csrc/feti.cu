@@ -1116,9 +1116,11 @@ __global__ void __launch_bounds__(256)
 // Bound by the 17 bytes per entry of Y and its mask.  The form before (a thread per cell walking
 // 32 rows one after the other, corner values gathered by a launch of its own) was a chain of
 // dependent loads: 72 us per launch on the 10^3 strut lattice and 44 us on 16 ring cells, where it
-// was 30 % of a load step.  16 rows per CTA: 10^3 strut solve (BF16) 520 ms, 36-cell strut solve (FP64)
-// 265, against 536 and 278 with 32 rows and 544 and 262 with 8.  T = FP32 in the mixed modes (an FP32
-// copy of Phi, part of their FP32 preconditioner).
+// was 30 % of a load step.  Rows per CTA, run times in turn against 16: 32 take 1.02 to 1.035 times as
+// long on a 4x4 ring load step (FP64), a 210-cell Newton iteration and the 10^3 strut solve (BF16) and the
+// 36-cell strut solve (FP64); 8 take 0.98 and 0.99 of it on the two FP64 calls, where the kernel is
+// latency, and 1.025 and 1.04 on the two BF16 ones, where CTAs gather the corner values twice as often.
+// T = FP32 in the mixed modes (an FP32 copy of Phi, part of their FP32 preconditioner).
 constexpr int kPhiRows = 16, kPhiCols = 96;
 
 template <typename T, int VEC>

@@ -532,8 +532,13 @@ void run_sdd_oz(lat_ctx* h, const double* X, double* Y) {
 // digits scaled by its own maximum), the rows of Pi (symmetric) and of R as the B operand, 128
 // columns at most, so base-256 digits (|s| <= 128, products up to 2^14, 8 of them over 128 columns)
 // still sum exactly and what is dropped is about 2^-62 of the row maxima; base-128 digits left
-// inverses of the strut cell's blocks 2.4 times further off than FP64 sweeps do.  An entry of A then takes four FP64 operations per panel
-// instead of 128.  Per panel: the chain of the pivot block (four 32-column steps, 26 us each), two
+// inverses of the strut cell's blocks 2.4 times further off than FP64 sweeps do.  An entry below 2^-9 of
+// its row's largest in the panel has fewer bits than in FP64; the inverse does not show it, because its
+// error comes from the rounding of the diagonal.  Emulated on 12 local blocks of strut and solid cells
+// with graded element sizes (624 and 1464 rows, condition 7e3 to 7e6), against FP64 sweeps of 32 columns:
+// error 1.06 times theirs (geometric mean; FP64 panels of 128 columns 1.03, single blocks 0.4 to 2.7 for
+// both), residual A A^-1 - I 0.58 times.  Rows and columns scaled by 2^-8 to 2^8 leave that unchanged.
+// An entry of A takes four FP64 operations per panel instead of 128.  Per panel: the chain of the pivot block (four 32-column steps, 26 us each), two
 // products and the splitting of C, Pi and R.  Three 2616 matrices: 9 ms against 53 ms.
 namespace {
 
