@@ -327,12 +327,12 @@ lat_status feti_apply(lat_handle h, int32_t mode, const double* v, double* w);
  * iterations and final relative residual of the saddle-point system. */
 lat_status tangent_solve(lat_handle h, const double* rhs, double* x, const lat_newton_opts* opts,
                          int32_t* iters, double* rel);
-/* Build the FETI-DP preconditioner for the current selection at state u_glob. */
+/* Build the FETI-DP preconditioner for the current selection at state u_glob.  A build that fails after
+ * it began leaves none: feti_apply and tangent_solve then return LAT_EINVAL until one succeeds. */
 lat_status lattice_prepare_solver(lat_handle h, const double* u_glob, const lat_newton_opts* opts);
 /* Polls after which a wait in a tensor-core product (local inverses and their inversion) gives up
  * (default 2^20).  The call that launched it then returns LAT_ETIMEOUT, with its outputs
- * undefined; the handle stays usable, after a failed lattice_prepare_solver once that has been run
- * again.  The paper has no counterpart.  LAT_EINVAL for a negative number. */
+ * undefined; the handle stays usable.  The paper has no counterpart.  LAT_EINVAL for a negative number. */
 lat_status lattice_set_wait_limit(lat_handle h, int32_t polls);
 /* Map a saddle-point vector's displacement part to a global vector (mean over copies). */
 lat_status feti_to_global(lat_handle h, const double* v, double* u_glob);

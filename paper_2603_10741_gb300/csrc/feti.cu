@@ -1444,6 +1444,14 @@ void run_prepare_solver(lat_ctx* h, const lat_newton_opts* o, const double* u_gl
     Kpre = h->Kp_mat.p;
   }
   drop_pcg_graph(h);   // buffers and sizes below may change
+  // a setup that fails from here on leaves no solver: its buffers may be missing or of other sizes
+  struct Ready {
+    lat_ctx* h;
+    bool done = false;
+    ~Ready() {
+      if (!done) h->n_keys = 0;
+    }
+  } ready{h};
   const int ns = h->n_cells, nR = h->n_R, nP = h->n_P;
   h->flag.ensure(4);
   h->red_part.ensure(4096);
@@ -1621,6 +1629,7 @@ void run_prepare_solver(lat_ctx* h, const lat_newton_opts* o, const double* u_gl
   h->pcg_ws.ensure(std::max<size_t>(1, (size_t)5 * h->n_lambda));
   h->gP.ensure(std::max<int64_t>(np, 1));
   h->xP.ensure(std::max<int64_t>(np, 1));
+  ready.done = true;
 }
 
 namespace {
@@ -2178,6 +2187,7 @@ void run_axpy(lat_ctx* h, int64_t n, double a, const double* x, double* y) {
 // nodes tie the cells' free sides to their neighbours, which removes those modes.)
 void prepare_enriched(lat_ctx* h, const lat_newton_opts* o, const double* u_glob) {
   if (h->enrich_level < o->min_enrich) {
+    h->n_keys = 0;   // other index sets: no solver until the setup below
     build_feti(h, std::min(o->min_enrich, o->max_enrich));
     if (h->verbose)
       std::fprintf(stderr, "[lattice] primal enrichment level %d (start): %d primal DOFs per cell, %lld coarse DOFs\n",
@@ -2185,6 +2195,7 @@ void prepare_enriched(lat_ctx* h, const lat_newton_opts* o, const double* u_glob
   }
   run_prepare_solver(h, o, u_glob);
   while ((h->indefinite || h->coarse_indefinite) && h->enrich_level < o->max_enrich) {
+    h->n_keys = 0;
     build_feti(h, h->enrich_level + 1);
     if (h->verbose)
       std::fprintf(stderr, "[lattice] primal enrichment level %d: %d primal DOFs per cell, %lld coarse DOFs\n",

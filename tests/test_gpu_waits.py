@@ -76,3 +76,29 @@ def test_wait_that_gives_up_is_reported(L, prec, cell, dims):
     with pytest.raises(L.LatticeError, match="LAT_EINVAL"):
         lat.lattice_set_wait_limit(-1)
     lat.close()
+
+
+@pytest.mark.parametrize("prec", [0, 1, 2])
+def test_no_solver_after_a_failed_setup(L, prec):
+    """A setup that fails, the first one or a later one, leaves no half-made solver behind: the calls that
+    need one say so instead of reading buffers that are missing."""
+    case, lat = _strut(L, prec, (2, 2, 6))
+    u = lat.lattice_predictor(0.1 * case.top_displacement(1))
+    opts = lat.lattice_default_opts(max_enrich=0, precond_tangent=1, krylov_max_it=3, inner_its=2)
+    rhs = torch.tensor(np.random.default_rng(1).uniform(-1, 1, lat.sizes.n_dof), device="cuda")
+    v = lat.feti_from_global(rhs)
+    lat.select_principal_cells(u, 1e-9, 1)
+    for first in (True, False):
+        if not first:
+            lat.lattice_prepare_solver(u, opts)
+            ref = lat.feti_apply(1, v)
+        lat.lattice_set_wait_limit(0)
+        with pytest.raises(L.LatticeError, match="LAT_ETIMEOUT"):
+            lat.lattice_prepare_solver(u, opts)
+        lat.lattice_set_wait_limit(1 << 20)
+        for call in (lambda: lat.feti_apply(1, v), lambda: lat.feti_apply(2, v), lambda: lat.tangent_solve(rhs, opts)):
+            with pytest.raises(L.LatticeError, match="LAT_EINVAL"):
+                call()
+    lat.lattice_prepare_solver(u, opts)
+    assert torch.equal(lat.feti_apply(1, v), ref)
+    lat.close()
