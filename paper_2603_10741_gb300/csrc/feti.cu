@@ -106,7 +106,7 @@ struct ArnoldiArgs {
 };
 
 // the block that ends last adds the partial sums of `cnt` dots into out
-__device__ __forceinline__ bool last_block_sums(const ArnoldiArgs& A, int cnt, double* out, double* red) {
+__device__ __forceinline__ bool last_block_sums(const ArnoldiArgs& A, int cnt, double* out) {
   __shared__ bool last;
   __syncthreads();
   if (threadIdx.x == 0) {
@@ -124,7 +124,6 @@ __device__ __forceinline__ bool last_block_sums(const ArnoldiArgs& A, int cnt, d
     if (lane == 0) out[i] = v;
   }
   if (threadIdx.x == 0) *A.ticket = 0;
-  (void)red;
   return true;
 }
 
@@ -143,7 +142,7 @@ __device__ __forceinline__ void partial_dots(const ArnoldiArgs& A, double* red) 
 __global__ void __launch_bounds__(256) k_arnoldi_dots(ArnoldiArgs A) {
   __shared__ double red[32];
   partial_dots(A, red);
-  last_block_sums(A, A.j + 1, A.h1, red);
+  last_block_sums(A, A.j + 1, A.h1);
 }
 
 // w -= V h1, h2 = V^T w
@@ -156,7 +155,7 @@ __global__ void __launch_bounds__(256) k_arnoldi_pass(ArnoldiArgs A) {
     A.w[k] = v;
   }
   partial_dots(A, red);
-  last_block_sums(A, A.j + 1, A.h2, red);
+  last_block_sums(A, A.j + 1, A.h2);
 }
 
 // w -= V h2, ||w||^2; then H's column h1 + h2, its rotations and the residual estimate
@@ -172,7 +171,7 @@ __global__ void __launch_bounds__(256) k_arnoldi_finish(ArnoldiArgs A) {
   }
   nrm = block_sum(nrm, red);
   if (threadIdx.x == 0) A.part[blockIdx.x] = nrm;
-  if (!last_block_sums(A, 1, A.sc, red)) return;
+  if (!last_block_sums(A, 1, A.sc)) return;
   __syncthreads();
   if (threadIdx.x != 0) return;
   // Givens rotations on one thread (Hessenberg column j, column major)
@@ -196,12 +195,12 @@ __global__ void __launch_bounds__(256) k_arnoldi_finish(ArnoldiArgs A) {
   A.sc[1] = fabs(g[j + 1]);
 }
 
-// w += sgn * sum_i h[i] V_i
+// w += sum_i h[i] V_i
 __global__ void k_multi_axpy(int64_t n, int m, const double* __restrict__ V, const double* __restrict__ hcoef,
-                             double sgn, double* __restrict__ w) {
+                             double* __restrict__ w) {
   for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n; k += (int64_t)gridDim.x * blockDim.x) {
     double v = w[k];
-    for (int i = 0; i < m; ++i) v += sgn * hcoef[i] * V[(size_t)i * n + k];
+    for (int i = 0; i < m; ++i) v += hcoef[i] * V[(size_t)i * n + k];
     w[k] = v;
   }
 }
@@ -2098,7 +2097,7 @@ int fgmres_core(lat_ctx* h, const GmresLevel& L, const double* b, double* x, boo
     }
     // x += Z y
     LAT_LAUNCH(h, k_gmres_solve<<<1, 1, 0, h->stream>>>(j, m, L.H->p, L.small->p, yv));
-    LAT_LAUNCH(h, k_multi_axpy<<<eb, 256, 0, h->stream>>>(n, j, L.Z->p, yv, 1.0, x));
+    LAT_LAUNCH(h, k_multi_axpy<<<eb, 256, 0, h->stream>>>(n, j, L.Z->p, yv, x));
     LAT_CHECK_LAUNCH();
     if (rel <= rtol) break;
   }
