@@ -26,15 +26,17 @@
 //   20 entries over 1e-6           9.8e-16 5.5e-15    5.0e-15 1.0e-10    3.7e-17 1.0e-16
 //   one entry over 1e-8            7.5e-16 5.8e-15    1.3e-14 1.0e-07    6.5e-17 8.0e-16
 //   one entry over 1e-12           4.1e-16 7.4e-15    5.4e-15 3.5e-04    4.3e-17 5.9e-12
-// (G itself is denser: 1.0e-16 in every row of its dual block.)  Only entries whose terms all lie below
-// 2^-26 of row maximum x vector maximum come out less exact than an FP64 sum leaves them.
+// (G itself is denser: 1.0e-16 in every row of its dual block.)  What is left are results far below row
+// maximum x vector maximum, whose terms may lie where the digits end: those below 2^-26 of it are summed
+// again in FP64 from the matrix and vector themselves, by the CTA that holds them (k_oz_mm's last loop;
+// cancellation alone takes few results that far).
 //
 // One tensor-memory tile is 128 rows x (12 accumulators of 16 cells): for digit i of the matrix one
 // MMA multiplies the digits 0 .. 11-i of the 16 cells (N = 16 (12 - i), consecutive rows of the B
 // panel) into the accumulators i .. 11, consecutive columns from 16 i on.  K is split over a cluster
 // of CTAs (336 columns at most each while eight CTAs suffice, which the exactness needs) that add their
 // FP64 tiles through distributed shared memory.  Bound by streaming the digits, 24 bytes per matrix
-// entry: the strut cell's dual block (1716 x 1692) for 3 keys and 36 cells is 227 MB: 67 us with
+// entry: the strut cell's dual block (1716 x 1692) for 3 keys and 36 cells is 227 MB: 68 us with
 // splitting the vectors (54 us with 8 digits) against 406 us on the FP64 pipe (175 us at its full rate).
 #include <algorithm>
 
@@ -57,7 +59,9 @@ constexpr int MAX_SPLIT = 8;              // portable cluster size
 constexpr double kOzBytes = 24e9;         // most digits kept, a twelfth of the device's memory
 constexpr int PART_LD = TM + 1;
 constexpr uint32_t LBO = 128, SBO = (TK / 8) * 128;
-static_assert((size_t)NC * PART_LD * sizeof(double) <= (size_t)STAGES * STAGE_BYTES, "the tile reuses the stages");
+constexpr size_t PART_BYTES = (size_t)NC * PART_LD * sizeof(double);   // the tile, then the list of small entries
+static_assert(PART_BYTES + (size_t)NC * TM * sizeof(int) <= (size_t)STAGES * STAGE_BYTES, "both reuse the stages");
+constexpr double SMALL = 0x1p-14;         // 2^-26 of row maximum x vector maximum, or up to four times that
 
 __device__ __forceinline__ uint64_t desc(uint32_t saddr) {
   return (uint64_t)((saddr >> 4) & 0x3FFFu) | (uint64_t)(LBO >> 4) << 16 | (uint64_t)(SBO >> 4) << 32 | (uint64_t)1 << 46;
@@ -283,13 +287,14 @@ __global__ void __launch_bounds__(128, 2)
             const int* __restrict__ tile_c0, const int* __restrict__ seg_ptr, const int* __restrict__ perm,
             const double* __restrict__ cscale, int n_R, int r_base, const int* __restrict__ rdofs,
             const int* __restrict__ pdofs, double* __restrict__ Y, int* __restrict__ err, int mul_scale,
-            int polls) {
+            int polls, const double* __restrict__ G, int ld, int64_t kstride, const double* __restrict__ X, int lo_c,
+            const uint8_t* __restrict__ fixed, const int2* __restrict__ lk) {
   extern __shared__ __align__(1024) unsigned char smem[];
   __shared__ __align__(8) uint64_t full[STAGES], empty[STAGES], done;
   __shared__ uint32_t tmem_slot;
   __shared__ int fail, issued;   // a wait gave up; panels whose copies were issued
-  __shared__ int cell[NC];
-  __shared__ double cs1[NC], cs2[NC];      // factor of a column's scaled rows, and of its corner rows
+  __shared__ int cell[NC], n_small;
+  __shared__ double cw[NC], cs1[NC], cs2[NC];   // a cell's factor; that times its digits' scale, and the scale
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int rank = blockIdx.x % S, tile = blockIdx.x / S, mt = mt0 + blockIdx.y;
   const int key = tile_seg[tile];
@@ -308,6 +313,7 @@ __global__ void __launch_bounds__(128, 2)
     }
     mbar_init(smem_u32(&done));
     fail = 0;
+    n_small = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -365,7 +371,8 @@ __global__ void __launch_bounds__(128, 2)
     const int s = pos < seg_ptr[key + 1] ? perm[pos] : -1;
     const double w = s >= 0 ? cscale[s] : 1.0, d = digit_scale(cmax[(size_t)tile * NC + c]);
     cell[c] = s;
-    cs1[c] = d * (mul_scale ? w : 1.0 / w);   // c_s (S_DD rows) or 1 / c_s (G rows)
+    cw[c] = mul_scale ? w : 1.0 / w;          // c_s (S_DD rows) or 1 / c_s (G rows)
+    cs1[c] = d * cw[c];
     cs2[c] = d;
   }
   __syncwarp();
@@ -381,6 +388,7 @@ __global__ void __launch_bounds__(128, 2)
   __syncwarp();
   // digit sums of the tile's row (this thread's) and each cell to one FP64 value, in shared memory
   double* part = reinterpret_cast<double*>(smem);   // [cell][129]
+  int* small = reinterpret_cast<int*>(smem + PART_BYTES);
   if (good) {
     const uint32_t base = tmem + ((uint32_t)(warp * 32) << 16);
 #pragma unroll 1
@@ -411,11 +419,34 @@ __global__ void __launch_bounds__(128, 2)
     if (S == 1) v = part[c * PART_LD + tid];
     else
       for (int q = 0; q < S; ++q) v += ld_cluster(a, (uint32_t)q);
-    if (cell[c] >= 0 && o >= 0 && good)
-      Y[(size_t)o * n_cells + cell[c]] = v * rs * (r_base + gi < n_R ? cs1[c] : cs2[c]);
+    if (cell[c] >= 0 && o >= 0 && good) {
+      const bool scaled = r_base + gi < n_R;
+      Y[(size_t)o * n_cells + cell[c]] = v * rs * (scaled ? cs1[c] : cs2[c]);
+      // an entry far below row maximum x vector maximum (v counts 2^-12 of their powers of two), unless it
+      // is not read (Dirichlet rows; of S_DD those without a multiplier) or the vector has the smallest
+      // exponent (its digits hold it whole; zero vectors alike)
+      if (fabs(v) < SMALL && rs != 0.0 && !(cs2[c] <= 0x1p-1027) &&
+          !(scaled && fixed[(size_t)o * n_cells + cell[c]])) {
+        const int2 m = lk ? lk[(size_t)gi * n_cells + cell[c]] : make_int2(1, 0);
+        if (m.x || m.y) small[atomicAdd(&n_small, 1)] = c * TM + tid;
+      }
+    }
   }
   if (S > 1) cluster_sync();   // peers have read this CTA's tile
   else __syncthreads();
+  // those entries in FP64, a warp each: their terms may lie where the digits end
+  for (int q = warp; q < n_small; q += 4) {
+    const int c = small[q] / TM, gr = sh.row(mt * TM + small[q] % TM), s = cell[c];
+    const double* g = G + key * kstride + (int64_t)gr * ld;
+    double a = 0.0;
+#pragma unroll 4
+    for (int k = lo_c + lane; k < sh.cols; k += 32) a = fma(g[k], X[(size_t)rdofs[r_base + k] * n_cells + s], a);
+    a = warp_sum(a);
+    if (lane == 0) {
+      const bool scaled = r_base + gr < n_R;
+      Y[(size_t)(scaled ? rdofs[r_base + gr] : pdofs[r_base + gr - n_R]) * n_cells + s] = scaled ? a * cw[c] : a;
+    }
+  }
   if (warp == 0) {
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TMEM_COLS) : "memory");
@@ -452,7 +483,8 @@ void split_matrix(lat_ctx* h, const OzShape& sh, int ld, int64_t kstride, const 
 }
 
 void product(lat_ctx* h, const OzShape& sh, int mt0, int kp0, const DBuf<__nv_bfloat16>& T, const DBuf<double>& scale,
-             const int* rdofs, int r_base, const double* X, double* Y, int n_R, int mul_scale) {
+             const double* G, int ld, int64_t kstride, const int* rdofs, int r_base, const double* X, double* Y, int n_R,
+             int mul_scale, const int2* lk) {
   const int npan = sh.KP - kp0, tiles = h->oz_tiles;
   const int lo_c = kp0 ? sh.nI : 0, n_K = sh.cols - lo_c;
   h->oz_X.ensure((size_t)tiles * npan * B_ELEMS);
@@ -485,7 +517,8 @@ void product(lat_ctx* h, const OzShape& sh, int mt0, int kp0, const DBuf<__nv_bf
                                             (const __nv_bfloat16*)h->oz_X.p, (const unsigned long long*)h->oz_max.p, ts,
                                             tc, (const int*)h->seg_ptr.p, (const int*)h->perm.p,
                                             (const double*)h->c_cell.p, n_R, r_base, rdofs, (const int*)h->pdofs.p, Y,
-                                            h->flag.p, mul_scale, h->wait_polls)));
+                                            h->flag.p, mul_scale, h->wait_polls, G, ld, kstride, X, lo_c,
+                                            (const uint8_t*)h->loc_fixed.p, lk)));
   LAT_CHECK_LAUNCH();
 }
 
@@ -493,7 +526,7 @@ void product(lat_ctx* h, const OzShape& sh, int mt0, int kp0, const DBuf<__nv_bf
 
 // Whether the FP64 mode's segmented products run on digits: blocks large enough that streaming 24
 // bytes per entry and the launches that split the cell vectors cost less than the FP64 pipe does
-// (36 cells of the strut cell's dual block 67 us against 406, 512 cells of the whole block 0.62 ms
+// (36 cells of the strut cell's dual block 68 us against 406, 512 cells of the whole block 0.62 ms
 // against 6.0; the ring cells' dual block is 56 columns, under 10 us either way), no more columns than
 // the largest cluster sums exactly in the accumulators 0 .. 7 (in the others beyond 2688 columns a sum
 // of like digits may round, at 2^-68 of row maximum x vector maximum), and at most kOzBytes of
@@ -516,12 +549,14 @@ void run_oz_split(lat_ctx* h) {
 
 void run_local_oz(lat_ctx* h, const double* X, double* Y, KinvMode mode) {
   const OzShape g = g_shape(h);
-  product(h, g, mode == KINV_DUAL ? g.MTI : 0, mode == KINV_FULL ? 0 : g.KI, h->oz_G, h->oz_Gs, h->rdofs.p, 0, X, Y,
-          h->n_R, 0);
+  product(h, g, mode == KINV_DUAL ? g.MTI : 0, mode == KINV_FULL ? 0 : g.KI, h->oz_G, h->oz_Gs, h->G.p, h->n_R,
+          (int64_t)(h->n_R + h->n_P) * h->n_R, h->rdofs.p, 0, X, Y, h->n_R, 0, nullptr);
 }
 
 void run_sdd_oz(lat_ctx* h, const double* X, double* Y) {
-  product(h, s_shape(h), 0, 0, h->oz_S, h->oz_Ss, h->rdofs.p, h->n_I, X, Y, h->n_R, 1);
+  const int nD = h->n_R - h->n_I;
+  product(h, s_shape(h), 0, 0, h->oz_S, h->oz_Ss, h->SDD.p, nD, (int64_t)nD * nD, h->rdofs.p, h->n_I, X, Y, h->n_R, 1,
+          h->dual_lk.p);
 }
 
 // ------------------------------------------------------------------------------------------------
